@@ -69,7 +69,7 @@ __device__ __forceinline__ void theta_terms(const MechView& M, const double* hRT
                                             double* GA, double* GE, const Grp1& g) {
   const double c1 = (w[0] * kRu) * T / (rho * cp);
   for (int k = g.lane; k < M.n; k += g.size)
-    a[k] = fma(__ldg(M.sp + (size_t)k * SP_STRIDE + 1) * w[1 + k], irho, -(c1 * hRT[k]));
+    a[k] = fma(__ldg(M.sp + M.n + k) * w[1 + k], irho, -(c1 * hRT[k]));
   g.sync();
   const double iRT = 1.0 / (kRu * T);
   for (int r = g.lane; r < M.R; r += g.size) {
@@ -175,7 +175,7 @@ __device__ __forceinline__ void theta_tangents(const MechView& M, const DualN<NT
     const Dual irho = tangent_of(sc.irho, st);
     const Dual c1 = (w[0] * kRu) * T / (rho * cp);
     for (int k = g.lane; k < M.n; k += g.size)
-      a[k] = sfma(Dual(__ldg(M.sp + (size_t)k * SP_STRIDE + 1) * w[1 + k]), irho, -(c1 * tangent_of(s[L.hRT + k], st)));
+      a[k] = sfma(Dual(__ldg(M.sp + M.n + k) * w[1 + k]), irho, -(c1 * tangent_of(s[L.hRT + k], st)));
     g.sync();
     const Dual iRT = 1.0 / (kRu * T);
     for (int r = g.lane; r < M.R; r += g.size) {

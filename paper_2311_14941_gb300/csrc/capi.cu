@@ -571,7 +571,8 @@ chem_status chem_create(const chem_mech_desc* desc, int device, chem_handle* out
          o_eam = put(buf, hm.eff_am1), o_dsp = put(buf, hm.dslot_sp), o_dmask = put(buf, hm.dslot_mask),
          o_dam = put(buf, hm.dslot_am1), o_er = put(buf, hm.entry_row), o_ec = put(buf, hm.entry_col),
          o_ew = put(buf, hm.entry_wratio), o_lsrc = put(buf, hm.lu_src), o_ldiag = put(buf, hm.lu_diag),
-         o_sout = put(buf, hm.s_out), o_rxo = put(buf, hm.rx_order), o_rxd0 = put(buf, hm.rxd);
+         o_sout = put(buf, hm.s_out), o_rxo = put(buf, hm.rx_order), o_rxd0 = put(buf, hm.rxd),
+         o_rxr = put(buf, hm.rxr);
   const int n_jp = (int)hm.jpass.size() / 4;
   if (n_jp > kMaxJPass) { delete h; return fail(CHEM_EUNSUPPORTED, "too many Jacobian passes"); }
   constexpr int kMaxG = 3 + kMaxJPass;
@@ -599,6 +600,7 @@ chem_status chem_create(const chem_mech_desc* desc, int device, chem_handle* out
     V.n = hm.n; V.R = hm.R; V.m = hm.m; V.n_troe = hm.n_troe; V.n_tb = hm.n_tb; V.nY = hm.nY; V.nnz_S = hm.nnz_S;
     V.nnz_LU = hm.nnz_LU; V.n_dslot = hm.n_dslot;
     V.sp = (const double*)(b + o_sp); V.rxd = (const double*)(b + o_rxd); V.rxi = (const int*)(b + o_rxi);
+    V.rxr = (const RxRec*)(b + o_rxr);
     V.eff_sp = (const int*)(b + o_esp); V.eff_am1 = (const double*)(b + o_eam);
     V.dslot_sp = (const int*)(b + o_dsp); V.dslot_mask = (const int*)(b + o_dmask);
     V.dslot_am1 = (const double*)(b + o_dam);

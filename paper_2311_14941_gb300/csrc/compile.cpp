@@ -309,16 +309,14 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
   // ---- species table
   hm.sp.assign((size_t)n * SP_STRIDE, 0.0);
   for (int k = 0; k < n; ++k) {
-    double* s = &hm.sp[(size_t)k * SP_STRIDE];
-    s[0] = 1.0 / d.W[k]; s[1] = d.W[k]; s[2] = d.T_mid[k];
+    auto field = [&](int f) -> double& { return hm.sp[(size_t)f * n + k]; };
+    field(0) = 1.0 / d.W[k]; field(1) = d.W[k]; field(2) = d.T_mid[k];
     for (int rg = 0; rg < 2; ++rg) {
       const double* a = rg ? &d.nasa_hi[7 * k] : &d.nasa_lo[7 * k];
-      double* c = s + 4 + rg * SP_RANGE;
-      for (int i = 0; i < 5; ++i) c[i] = a[i];
-      c[5] = a[1] / 2.0; c[6] = a[2] / 3.0; c[7] = a[3] / 4.0; c[8] = a[4] / 5.0;
-      c[9] = -a[1] / 2.0; c[10] = -a[2] / 6.0; c[11] = -a[3] / 12.0; c[12] = -a[4] / 20.0;
-      c[13] = a[5]; c[14] = a[6];
-      c[15] = 2.0 * a[2]; c[16] = 3.0 * a[3]; c[17] = 4.0 * a[4];
+      const double c[SP_RANGE] = {a[0], a[1], a[2], a[3], a[4], a[1] / 2.0, a[2] / 3.0, a[3] / 4.0, a[4] / 5.0,
+                                  -a[1] / 2.0, -a[2] / 6.0, -a[3] / 12.0, -a[4] / 20.0, a[5], a[6], 2.0 * a[2],
+                                  3.0 * a[3], 4.0 * a[4]};
+      for (int i = 0; i < SP_RANGE; ++i) field(4 + rg * SP_RANGE + i) = c[i];
     }
   }
   // ---- reaction tables, derivative slots
@@ -329,11 +327,11 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
   std::vector<std::vector<int>> slots_sp(R);
   for (int r = 0; r < R; ++r) {
     const Rx& x = rx[hm.rx_order[r]];
-    double* D = &hm.rxd[(size_t)r * RX_D];
-    D[0] = std::log(x.A); D[1] = x.b; D[2] = x.Ea / kRu;
+    auto D = [&](int f) -> double& { return hm.rxd[(size_t)f * R + r]; };
+    D(0) = std::log(x.A); D(1) = x.b; D(2) = x.Ea / kRu;
     if (x.type == 2) {
-      D[3] = std::log(x.A0); D[4] = x.b0; D[5] = x.Ea0 / kRu;
-      D[6] = 1.0 - x.alpha; D[7] = x.alpha; D[8] = 1.0 / x.T3; D[9] = 1.0 / x.T1; D[10] = x.T2 > 0.0 ? x.T2 : 0.0;
+      D(3) = std::log(x.A0); D(4) = x.b0; D(5) = x.Ea0 / kRu;
+      D(6) = 1.0 - x.alpha; D(7) = x.alpha; D(8) = 1.0 / x.T3; D(9) = 1.0 / x.T1; D(10) = x.T2 > 0.0 ? x.T2 : 0.0;
     }
     int* I = &hm.rxi[(size_t)r * RX_I];
     I[0] = x.type; I[1] = x.rev; I[2] = (int)x.ro.size(); I[3] = (int)x.po.size();
@@ -413,17 +411,13 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
 
   // ---- gather programs
   {
-    std::vector<std::vector<std::pair<int, int>>> gw(n), gr(n), gc(n);
-    for (int r = 0; r < R; ++r)
-      for (auto& kv : netmap[r])
-        if (kv.second != 0) gw[kv.first].push_back({r, enc_nu(kv.second)});
+    std::vector<std::vector<std::pair<int, int>>> gr(n), gc(n);
     for (int e = 0; e < hm.nY; ++e) {
       gr[hm.entry_row[e]].push_back({e, hm.entry_col[e]});
       gc[hm.entry_col[e]].push_back({e, hm.entry_row[e]});
     }
     for (HostProg& P : hm.prog)
-      if (!build_gather(gw, P.g_omega, err, P.width) || !build_gather(gr, P.g_row, err, P.width) ||
-          !build_gather(gc, P.g_col, err, P.width))
+      if (!build_gather(gr, P.g_row, err, P.width) || !build_gather(gc, P.g_col, err, P.width))
         return CHEM_EUNSUPPORTED;
   }
 
@@ -624,20 +618,67 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
       if (biggest <= cap || P >= kMaxJPass || P >= R) break;
     }
     const int P = (int)cut.size() - 1;
+    // Place the reactions: within every class of every pass the simple ones together (after the others in the
+    // first pass, before them in later ones), so that nearly every round of lanes is simple throughout.  Only
+    // the position of a reaction changes: the terms of every sum below keep the description's order.
+    std::vector<RxRec> rec(R);
+    for (int r = 0; r < R; ++r) {
+      const Rx& x = rx[hm.rx_order[r]];
+      auto sp_of = [&](const std::vector<int>& o, size_t i) { return (uint32_t)(i < o.size() ? o[i] : 0); };
+      auto rep = [](const std::vector<int>& o) { return std::set<int>(o.begin(), o.end()).size() < o.size(); };
+      std::set<int> all(x.ro.begin(), x.ro.end());
+      all.insert(x.po.begin(), x.po.end());
+      const bool simple = x.type == 0 && x.rev && x.ro.size() == 2 && x.po.size() == 2 && all.size() == 4;
+      rec[r] = RxRec{sp_of(x.ro, 0) | sp_of(x.ro, 1) << 16, sp_of(x.ro, 2) | sp_of(x.po, 0) << 16,
+                     sp_of(x.po, 1) | sp_of(x.po, 2) << 16,
+                     (uint32_t)((x.rev ? RXF_REV : 0) | x.ro.size() << 1 | x.po.size() << 3 | (simple ? RXF_SIMPLE : 0) |
+                                (rep(x.ro) || rep(x.po) ? RXF_REP : 0))};
+    }
+    std::vector<int> at(R), pos(R);   // at[i]: reaction placed at i; pos: its inverse
+    std::iota(at.begin(), at.end(), 0);
+    for (int p = 0; p < P; ++p) {
+      const int cls[4] = {0, hm.n_troe, hm.n_troe + hm.n_tb, R};
+      for (int c = 0; c < 3; ++c) {
+        const int lo = std::max(cut[p], cls[c]), hi = std::min(cut[p + 1], cls[c + 1]);
+        if (lo >= hi) continue;
+        std::stable_partition(at.begin() + lo, at.begin() + hi,
+                              [&](int r) { return ((rec[r].flags & RXF_SIMPLE) != 0) == (p > 0); });
+      }
+    }
+    for (int i = 0; i < R; ++i) pos[at[i]] = i;
+    {
+      const std::vector<int> order = hm.rx_order, rxi = hm.rxi;
+      const std::vector<double> rxd = hm.rxd;
+      hm.rxr.resize(R);
+      for (int i = 0; i < R; ++i) {
+        const int r = at[i];
+        hm.rx_order[i] = order[r];
+        hm.rxr[i] = rec[r];
+        std::copy(&rxi[(size_t)r * RX_I], &rxi[(size_t)r * RX_I] + RX_I, &hm.rxi[(size_t)i * RX_I]);
+        for (int f = 0; f < RX_D; ++f) hm.rxd[(size_t)f * R + i] = rxd[(size_t)f * R + r];
+      }
+    }
+    std::vector<std::vector<std::pair<int, int>>> gw(n);
+    for (int r = 0; r < R; ++r)
+      for (auto& kv : netmap[r])
+        if (kv.second != 0) gw[kv.first].push_back({pos[r], enc_nu(kv.second)});
+    for (HostProg& Pg : hm.prog)
+      if (!build_gather(gw, Pg.g_omega, err, Pg.width)) return CHEM_EUNSUPPORTED;
     hm.jpass.clear();
     for (HostProg& Pg : hm.prog) Pg.g_jac.assign(P, HostGather());
     for (int p = 0; p < P; ++p) {
       const int rb = cut[p], re = cut[p + 1];
-      const int sb = R > 0 && rb < R ? hm.rxi[(size_t)rb * RX_I + 13] : hm.n_dslot;
+      int sb = hm.n_dslot;   // a pass's derivative slots are consecutive (its reactions only trade places)
+      for (int i = rb; i < re; ++i) sb = std::min(sb, hm.rxi[(size_t)i * RX_I + 13]);
       const int cnt = re - rb;
       hm.jpass.insert(hm.jpass.end(), {rb, re, sb, cnt});
       std::vector<std::vector<std::pair<int, int>>> gj(hm.nY + n);
       for (int r = rb; r < re; ++r) {
-        const int base = hm.rxi[(size_t)r * RX_I + 13];
+        const int base = hm.rxi[(size_t)pos[r] * RX_I + 13];
         for (auto& kv : netmap[r]) {
           if (kv.second == 0) continue;
           const int nu = enc_nu(kv.second);
-          gj[hm.nY + kv.first].push_back({r - rb, nu});
+          gj[hm.nY + kv.first].push_back({pos[r] - rb, nu});
           for (size_t c = 0; c < slots_sp[r].size(); ++c)
             gj[eidx[kv.first][slots_sp[r][c]]].push_back({cnt + base + (int)c - sb, nu});
         }
@@ -667,14 +708,14 @@ constexpr int kTabMaxDeg = 8;
 double tab_function(const HostMech& hm, int cls, int f, double T) {
   const double lnT = std::log(T), invT = 1.0 / T;
   if (cls == TC_E || cls == TC_IE) {
-    const double* s = &hm.sp[(size_t)f * SP_STRIDE];
-    const double* c = s + 4 + (T < s[2] ? 0 : SP_RANGE);
-    const double g = c[0] * (1.0 - lnT) + T * (c[9] + T * (c[10] + T * (c[11] + T * c[12]))) + c[13] * invT - c[14];
+    const int base = 4 + (T < hm.sp[(size_t)2 * hm.n + f] ? 0 : SP_RANGE);
+    auto c = [&](int i) { return hm.sp[(size_t)(base + i) * hm.n + f]; };
+    const double g = c(0) * (1.0 - lnT) + T * (c(9) + T * (c(10) + T * (c(11) + T * c(12)))) + c(13) * invT - c(14);
     return std::exp(cls == TC_E ? g : -g);
   }
-  const double* D = &hm.rxd[(size_t)f * RX_D];
-  if (cls == TC_KF) return std::exp(D[0] + D[1] * lnT - D[2] * invT);
-  return D[6] * std::exp(-T * D[8]) + D[7] * std::exp(-T * D[9]) + (D[10] > 0.0 ? std::exp(-D[10] * invT) : 0.0);
+  auto D = [&](int i) { return hm.rxd[(size_t)i * hm.R + f]; };
+  if (cls == TC_KF) return std::exp(D(0) + D(1) * lnT - D(2) * invT);
+  return D(6) * std::exp(-T * D(8)) + D(7) * std::exp(-T * D(9)) + (D(10) > 0.0 ? std::exp(-D(10) * invT) : 0.0);
 }
 
 // mono[d][k][i]: coefficient of tau^i in the Chebyshev polynomial T_k, for every degree bound d <= 8.

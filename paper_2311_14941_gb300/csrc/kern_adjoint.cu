@@ -77,13 +77,13 @@ __global__ void k_set_params(MechView M, const double* __restrict__ rxd0, double
   if (r >= M.R) return;
   const int d = __ldg(M.rx_order + r);
   const double a = dlnA ? dlnA[d] : 0.0, e = dEa ? dEa[d] / kRu : 0.0;
-  const double* src = rxd0 + (size_t)r * RX_D;
-  double* dst = rxd + (size_t)r * RX_D;
+  const double* src = rxd0 + r;
+  double* dst = rxd + r;
   dst[0] = src[0] + a;
-  dst[2] = src[2] + e;
+  dst[2 * (size_t)M.R] = src[2 * (size_t)M.R] + e;
   if (__ldg((const int*)(M.rxi + (size_t)r * RX_I)) == 2) {
-    dst[3] = src[3] + a;
-    dst[5] = src[5] + e;
+    dst[3 * (size_t)M.R] = src[3 * (size_t)M.R] + a;
+    dst[5 * (size_t)M.R] = src[5 * (size_t)M.R] + e;
   }
 }
 

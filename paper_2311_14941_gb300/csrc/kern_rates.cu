@@ -21,7 +21,7 @@ __global__ void k_rates(MechView M, CellLayout L, int N, const double* __restric
     else dYdt[(size_t)(i - 1) * N + c] = f[i];
   }
   if (wdot) {
-    for (int k = lane; k < M.n; k += kWarp) wdot[(size_t)k * N + c] = f[1 + k] * sc.rho * __ldg(M.sp + (size_t)k * SP_STRIDE);
+    for (int k = lane; k < M.n; k += kWarp) wdot[(size_t)k * N + c] = f[1 + k] * sc.rho * __ldg(M.sp + k);
   }
 }
 

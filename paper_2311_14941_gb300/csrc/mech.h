@@ -30,7 +30,8 @@ constexpr int kMaxWarpsPerCell = 2;   // a cell is integrated by one warp or by 
 constexpr int kNumGroups = 3;
 constexpr int kGroupWidth[kNumGroups] = {32, 64, 16};
 
-// ---- species table: SP_STRIDE doubles per species
+// ---- species table, structure of arrays: field f of species k at sp[f * n + k], SP_STRIDE fields (lanes hold
+// consecutive species, so a warp's read of one field is one or two cache lines instead of 32)
 //   [0] 1/W  [1] W  [2] T_mid  [3] unused
 //   [4 .. 4+RANGE)   low range, [4+RANGE .. 4+2 RANGE) high range, each:
 //   a0 a1 a2 a3 a4 | h1..h4 = a1/2 a2/3 a3/4 a4/5 | g1..g4 = -a1/2 -a2/6 -a3/12 -a4/20 | a5 a6 |
@@ -41,8 +42,9 @@ constexpr int kGroupWidth[kNumGroups] = {32, 64, 16};
 constexpr int SP_RANGE = 18;
 constexpr int SP_STRIDE = 4 + 2 * SP_RANGE;
 
-// ---- reaction tables (reactions ordered: Troe, then third-body, then elementary)
-// doubles, RX_D per reaction:
+// ---- reaction tables.  Reactions are ordered Troe, third-body, elementary; within a class and a Jacobian
+// pass the simple ones (see RXF_SIMPLE) stand together, so that whole rounds of lanes are simple.
+// doubles, structure of arrays (field f of reaction r at rxd[f * R + r]), RX_D fields:
 //   [0] ln A  [1] b  [2] Ea/Ru  [3] ln A0  [4] b0  [5] Ea0/Ru  [6] 1-alpha  [7] alpha  [8] 1/T3  [9] 1/T1
 //   [10] T2 (0: absent)  [11] unused
 constexpr int RX_D = 12;
@@ -52,6 +54,15 @@ constexpr int RX_D = 12;
 //   nu occurrences)  [7..9] product occurrences  [10] sum of net coefficients  [11] efficiency offset
 //   [12] efficiency count  [13] derivative-slot offset  [14] derivative-slot count  [15] unused
 constexpr int RX_I = 16;
+// one 16-byte record per reaction with what the rate of progress needs: six 16-bit species indices (reactant,
+// then product occurrences; absent ones are 0) and the flags below
+struct alignas(16) RxRec {
+  uint32_t r01, r2p0, p12, flags;   // r0 | r1 << 16, r2 | p0 << 16, p1 | p2 << 16
+};
+// flags: bit 0 reversible, bits 1-2 reactant occurrences, bits 3-4 product occurrences, bit 5 simple
+// (elementary, reversible, two reactants and two products, all four different species), bit 6: a species
+// occurs more than once on one side
+enum : int { RXF_REV = 1, RXF_SIMPLE = 32, RXF_REP = 64 };
 
 // ---- warp programs, compiled for a group of `width` lanes (one warp per cell: 32, two: 64, half: 16)
 // Gather ("flattened segmented reduction"): step s, lane l executes op[s*width + l]:
@@ -94,9 +105,10 @@ struct MechView {
   int nnz_S;                 // nY + n (T column) + m (T row)
   int nnz_LU;
   int n_dslot;
-  const double* sp;          // [n * SP_STRIDE]
-  const double* rxd;         // [R * RX_D]
+  const double* sp;          // [SP_STRIDE * n]
+  const double* rxd;         // [RX_D * R]
   const int* rxi;            // [R * RX_I]
+  const RxRec* rxr;          // [R]
   const int* eff_sp;         // listed efficiencies
   const double* eff_am1;     // alpha - 1
   const int* dslot_sp;       // [n_dslot] column species of each derivative slot

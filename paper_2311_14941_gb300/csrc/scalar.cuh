@@ -160,6 +160,18 @@ __device__ __forceinline__ double sfma(double a, double b, double c) { return fm
 __device__ __forceinline__ Dual sfma(Dual a, Dual b, Dual c) {
   return Dual(fma(a.v, b.v, c.v), fma(a.v, b.d, fma(a.d, b.v, c.d)));
 }
+// a product that is rounded by itself: the compiler may not fuse it with an addition that follows
+__device__ __forceinline__ double smul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ Dual smul(Dual a, Dual b) {
+  return Dual(__dmul_rn(a.v, b.v), fma(a.v, b.d, a.d * b.v));
+}
+template <int K>
+__device__ __forceinline__ DualN<K> smul(const DualN<K>& a, const DualN<K>& b) {
+  DualN<K> r; r.v = __dmul_rn(a.v, b.v);
+#pragma unroll
+  for (int i = 0; i < K; ++i) r.d[i] = fma(a.v, b.d[i], a.d[i] * b.v);
+  return r;
+}
 // ln x by table-driven reduction (Tang, ACM TOMS 16(4), 1990), in a variant with 256 table entries:
 //   x = 2^k y, y in [1, 2); j = top 8 bits of y's fraction; u = y c_j - 1 with c_j the rounded reciprocal
 //   of the centre of y's interval (1 and 2 for the first and last intervals), |u| <= 2^-8;
