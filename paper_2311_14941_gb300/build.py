@@ -27,7 +27,7 @@ CUDA_UNITS = ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd
               "kern_adjoint")
 HOST_UNITS = ("compile", "balance", "specialize")
 # device headers the run-time compiler sees, under the names integrate.cuh includes them by
-RTC_HEADERS = ("mech.h", "elementary_tables.h", "scalar.cuh", "device.cuh", "integrate.cuh")
+RTC_HEADERS = ("mech.h", "elementary_tables.h", "intdiv.cuh", "scalar.cuh", "device.cuh", "integrate.cuh")
 RTC_INC = os.path.join(OUT, "rtc_headers.inc")
 
 

@@ -67,11 +67,11 @@ __device__ __forceinline__ void vjp(const MechView& M, const Sc* S, const Sc* u,
 __device__ __forceinline__ void theta_terms(const MechView& M, const double* hRT, const double* q, double T,
                                             double rho, double cp, double irho, const double* w, double* a,
                                             double* GA, double* GE, const Grp1& g) {
-  const double c1 = (w[0] * kRu) * T / (rho * cp);
+  const double c1 = div_rn((w[0] * kRu) * T, rho * cp);
   for (int k = g.lane; k < M.n; k += g.size)
     a[k] = fma(__ldg(M.sp + M.n + k) * w[1 + k], irho, -(c1 * hRT[k]));
   g.sync();
-  const double iRT = 1.0 / (kRu * T);
+  const double iRT = rcp_rn(kRu * T);
   for (int r = g.lane; r < M.R; r += g.size) {
     const int* I = M.rxi + (size_t)r * RX_I;
     const int nro = __ldg(I + 2), npo = __ldg(I + 3);
@@ -226,7 +226,7 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
                                              double* GE, const Grp1& g) {
   const CellLayout& L = A.L;
   const int m = M.m;
-  const double ih = 1.0 / h;
+  const double ih = rcp_rn(h);
   double* W1 = ws + A.W1; double* W2 = ws + A.W2; double* W3 = ws + A.W3; double* W4 = ws + A.W4;
   double* MU1 = ws + A.MU1; double* MU2 = ws + A.MU2; double* MU3 = ws + A.MU3; double* MU4 = ws + A.MU4;
   double* LAM = ws + A.LAM; double* G = ws + A.G; double* Y3 = ws + A.Y3; double* Y4 = ws + A.Y4;
@@ -244,7 +244,7 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
   double uz = 0.0;
   for (int i = g.lane; i < m; i += g.size) uz = fma(UY[i], X[i], uz);
   uz = gsum(g, uz);
-  const double idenT = 1.0 / (1.0 - uz);
+  const double idenT = rcp_rn(1.0 - uz);
   vset(ZT, X, m, g);
   // ---- reverse sweep over the stages, one pass of the loop per stage, so that the kernel holds one copy
   //      of the transposed solve and of the stage Jacobian code (written out, the stages overflowed the

@@ -5,22 +5,32 @@
 #pragma once
 
 #include "elementary_tables.h"
+#include "intdiv.cuh"
 
 namespace chemgb {
+
+// k as a double, from its bits (the conversion instruction takes the FP64 pipe).
+__device__ __forceinline__ double double_of_int(int k) {
+  const unsigned a = (unsigned)(k < 0 ? -k : k);
+  const int z = __clz((int)a);
+  const unsigned f = (a << z) << 1;   // the bits after the leading one
+  const unsigned hi = ((unsigned)k & 0x80000000u) | ((unsigned)(1023 + 31 - z) << 20) | (f >> 12);
+  return __hiloint2double(a ? (int)hi : 0, (int)(f << 20));
+}
 
 // e^x by table-driven reduction (Tang, ACM TOMS 15(2), 1989), in a variant with 256 table entries:
 //   k = nearest integer to 256 x / ln2, read from the low word of x * 256/ln2 + 1.5 * 2^52;
 //   r = x - k ln2/256 in two fused steps (the first is exact because k * kExpCHi is), |r| <= ln2/512;
 //   e^r - 1 = r (1 + r/2 + r^2/6 + r^3/24), truncation below r^5/120 < 4e-17 relative;
 //   e^x = 2^m * T[j] * e^r with k = 256 m + j, the power of two added to the exponent field.
-// Nine FP64 operations; error about one ulp.  |x| >= 704 (results near overflow or in the subnormal
+// Eight FP64 operations; error about one ulp.  |x| >= 704 (results near overflow or in the subnormal
 // range) and NaN take the library exp.
 __device__ __forceinline__ double fast_exp(double x) {
   if ((__double2hiint(x) & 0x7fffffff) >= 0x40860000) return exp(x);
   constexpr double kShift = 0x1.8p52;
   const double t = fma(x, kExpInvC, kShift);
   const int k = __double2loint(t);
-  const double kd = t - kShift;
+  const double kd = double_of_int(k);   // t - kShift, without the FP64 pipe
   double r = fma(kd, -kExpCHi, x);
   r = fma(kd, -kExpCLo, r);
   double q = fma(r, 1.0 / 24.0, 1.0 / 6.0);
@@ -49,13 +59,13 @@ __device__ __forceinline__ Dual operator+(double a, Dual b) { return Dual(a + b.
 __device__ __forceinline__ Dual operator-(Dual a, double b) { return Dual(a.v - b, a.d); }
 __device__ __forceinline__ Dual operator-(double a, Dual b) { return Dual(a - b.v, -b.d); }
 __device__ __forceinline__ Dual operator/(Dual a, Dual b) {
-  const double q = a.v / b.v;
-  return Dual(q, (a.d - q * b.d) / b.v);
+  const double q = div_rn(a.v, b.v);
+  return Dual(q, div_rn(a.d - q * b.d, b.v));
 }
-__device__ __forceinline__ Dual operator/(Dual a, double b) { return Dual(a.v / b, a.d / b); }
+__device__ __forceinline__ Dual operator/(Dual a, double b) { return Dual(div_rn(a.v, b), div_rn(a.d, b)); }
 __device__ __forceinline__ Dual operator/(double a, Dual b) {
-  const double q = a / b.v;
-  return Dual(q, -q * b.d / b.v);
+  const double q = div_rn(a, b.v);
+  return Dual(q, div_rn(-q * b.d, b.v));
 }
 __device__ __forceinline__ Dual& operator+=(Dual& a, Dual b) { a = a + b; return a; }
 __device__ __forceinline__ Dual& operator-=(Dual& a, Dual b) { a = a - b; return a; }
@@ -123,7 +133,7 @@ template <int K>
 __device__ __forceinline__ DualN<K> operator-(double a, const DualN<K>& b) { return (-b) + a; }
 template <int K>
 __device__ __forceinline__ DualN<K> operator/(const DualN<K>& a, const DualN<K>& b) {
-  const double ib = 1.0 / b.v;
+  const double ib = rcp_rn(b.v);
   DualN<K> r; r.v = a.v * ib;
 #pragma unroll
   for (int i = 0; i < K; ++i) r.d[i] = (a.d[i] - r.v * b.d[i]) * ib;
@@ -131,7 +141,7 @@ __device__ __forceinline__ DualN<K> operator/(const DualN<K>& a, const DualN<K>&
 }
 template <int K>
 __device__ __forceinline__ DualN<K> operator/(const DualN<K>& a, double b) {
-  const double ib = 1.0 / b;
+  const double ib = rcp_rn(b);
   DualN<K> r; r.v = a.v * ib;
 #pragma unroll
   for (int i = 0; i < K; ++i) r.d[i] = a.d[i] * ib;
@@ -139,7 +149,7 @@ __device__ __forceinline__ DualN<K> operator/(const DualN<K>& a, double b) {
 }
 template <int K>
 __device__ __forceinline__ DualN<K> operator/(double a, const DualN<K>& b) {
-  const double ib = 1.0 / b.v;
+  const double ib = rcp_rn(b.v);
   DualN<K> r; r.v = a * ib;
   const double s = -r.v * ib;
 #pragma unroll
@@ -178,7 +188,7 @@ __device__ __forceinline__ DualN<K> smul(const DualN<K>& a, const DualN<K>& b) {
 //   ln x = (k ln2_lead + lnF_lead_j) + (k ln2_trail + lnF_trail_j + log1p(u)), where lnF_j = -ln c_j
 //   (so the rounding of c_j needs no correction) and the first sum is exact (leads on the grid 2^-43);
 //   log1p(u) = u - u^2 (1/2 - u/3 + u^2/4 - u^3/5 + u^4/6 - u^5/7), truncation below 2^-59 relative.
-// Thirteen FP64 operations; error about one ulp; ln of values near 1 keeps full relative accuracy.
+// Twelve FP64 operations; error about one ulp; ln of values near 1 keeps full relative accuracy.
 // Zero, negative, subnormal, infinite and NaN arguments take the library log.
 __device__ __forceinline__ double fast_log(double x) {
   const int hx = __double2hiint(x);
@@ -195,8 +205,7 @@ __device__ __forceinline__ double fast_log(double x) {
   q = fma(u, q, -1.0 / 3.0);
   q = fma(u, q, 0.5);
   const double p = fma(-(u * u), q, u);
-  // k as a double without a conversion instruction: 2^52 + 2^31 + k from its bits, minus 2^52 + 2^31
-  const double kd = __hiloint2double(0x43300000, k ^ (int)0x80000000) - 0x1.00000800p52;
+  const double kd = double_of_int(k);
   const double t1 = fma(kd, kLn2Lead, lead);
   const double t2 = fma(kd, kLn2Trail, trail) + p;
   return t1 + t2;
@@ -224,13 +233,35 @@ __device__ __forceinline__ DualN<K> sexp(const DualN<K>& a) {
 template <int K>
 __device__ __forceinline__ DualN<K> slog(const DualN<K>& a) {
   DualN<K> r; r.v = fast_log(a.v);
-  const double ia = 1.0 / a.v;
+  const double ia = rcp_rn(a.v);
 #pragma unroll
   for (int i = 0; i < K; ++i) r.d[i] = a.d[i] * ia;
   return r;
 }
 __device__ __forceinline__ double slog(double a) { return fast_log(a); }
-__device__ __forceinline__ Dual slog(Dual a) { return Dual(fast_log(a.v), a.d / a.v); }
+__device__ __forceinline__ Dual slog(Dual a) { return Dual(fast_log(a.v), div_rn(a.d, a.v)); }
+// quotient and reciprocal (integer arithmetic for doubles, see intdiv.cuh; IEEE results)
+__device__ __forceinline__ double sdiv(double a, double b) { return div_rn(a, b); }
+__device__ __forceinline__ double srcp(double a) { return rcp_rn(a); }
+template <class Sc>
+__device__ __forceinline__ Sc sdiv(const Sc& a, const Sc& b) { return a / b; }
+template <class Sc>
+__device__ __forceinline__ Sc srcp(const Sc& a) { return 1.0 / a; }
+
+// Decisions from the bits of doubles (floating-point comparisons, minima and maxima take the FP64 pipe).
+// Finite:
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+// a < b and a <= b where b > 0 and neither is NaN (a may have either sign: negative bits are negative integers):
+__device__ __forceinline__ bool less_pos(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+__device__ __forceinline__ bool leq_pos(double a, double b) { return __double_as_longlong(a) <= __double_as_longlong(b); }
+// the larger magnitude; the smaller and the larger of two numbers >= 0
+__device__ __forceinline__ double max_mag(double a, double b) {
+  const long long x = __double_as_longlong(a) & 0x7fffffffffffffffll, y = __double_as_longlong(b) & 0x7fffffffffffffffll;
+  return __longlong_as_double(x > y ? x : y);
+}
+__device__ __forceinline__ double min_pos(double a, double b) { return less_pos(a, b) ? a : b; }
+__device__ __forceinline__ double max_pos(double a, double b) { return less_pos(a, b) ? b : a; }
+
 __device__ __forceinline__ double val(double a) { return a; }
 __device__ __forceinline__ double val(Dual a) { return a.v; }
 template <int K>
