@@ -45,18 +45,19 @@ struct AdjLayout {
 };
 
 // out = J^T w = S^T w + v (u . w) with S in the internal entry order
-template <class Sc>
-__device__ __forceinline__ void vjp(const MechView& M, const Sc* S, const Sc* u, const Sc* v, const double* w, Sc* out,
-                                    Sc* part, const Grp1& g) {
-  run_gather(M.g_col, out + 1, part, [&](int a, int b) { return S[a] * w[1 + b]; }, g);
+template <class P, class Q>
+__device__ __forceinline__ void vjp(const MechView& M, P S, P u, P v, const double* w, double* out, Q part,
+                                    const Grp1& g) {
+  using Sc = double;
+  gather_xy(M.g_col, out + 1, part, S, w + 1, g);
   Sc t0 = Sc(0.0), uw = Sc(0.0);
-  for (int k = g.lane; k < M.n; k += g.size) t0 = sfma(S[M.nY + k], Sc(w[1 + k]), t0);
-  for (int i = g.lane; i < M.m; i += g.size) uw = sfma(u[i], Sc(w[i]), uw);
+  for (int k = g.lane; k < M.n; k += g.size) t0 = sfma(Sc(S[M.nY + k]), Sc(w[1 + k]), t0);
+  for (int i = g.lane; i < M.m; i += g.size) uw = sfma(Sc(u[i]), Sc(w[i]), uw);
   t0 = gsum(g, t0);
   uw = gsum(g, uw);
   for (int c = g.lane; c < M.m; c += g.size) {
     const Sc base = (c == 0) ? t0 : out[c];
-    out[c] = sfma(v[c], uw, sfma(S[M.nY + M.n + c], Sc(w[0]), base));
+    out[c] = sfma(Sc(v[c]), uw, sfma(Sc(S[M.nY + M.n + c]), Sc(w[0]), base));
   }
   g.sync();
 }
@@ -64,12 +65,13 @@ __device__ __forceinline__ void vjp(const MechView& M, const Sc* S, const Sc* u,
 // dL/dtheta += w^T f_theta at an evaluated state: for reaction r, q_r * E_r with E_r = sum_products a_k -
 // sum_reactants a_k, a_k = W_k w_k / rho - w_T H_k / (rho c_p).  hRT, q: the evaluation's h/RT and rates
 // of progress; a: n doubles of scratch (shared memory, read by index).
-__device__ __forceinline__ void theta_terms(const MechView& M, const double* hRT, const double* q, double T,
-                                            double rho, double cp, double irho, const double* w, double* a,
+template <class P>
+__device__ __forceinline__ void theta_terms(const MechView& M, P hRT, P q, double T,
+                                            double rho, double cp, double irho, const double* w, SPtr a,
                                             double* GA, double* GE, const Grp1& g) {
   const double c1 = div_rn((w[0] * kRu) * T, rho * cp);
   for (int k = g.lane; k < M.n; k += g.size)
-    a[k] = fma(__ldg(M.sp + M.n + k) * w[1 + k], irho, -(c1 * hRT[k]));
+    a[k] = fma(__ldg(M.sp + M.n + k) * w[1 + k], irho, -(c1 * (double)hRT[k]));
   g.sync();
   const double iRT = rcp_rn(kRu * T);
   for (int r = g.lane; r < M.R; r += g.size) {
@@ -85,24 +87,15 @@ __device__ __forceinline__ void theta_terms(const MechView& M, const double* hRT
   g.sync();
 }
 
-// x <- A^-T x (transposed substitution with the factor LU, dinv; x in shared memory)
-__device__ __forceinline__ void lu_solveT(const MechView& M, const double* LU, const double* dinv, double* x,
-                                          const Grp1& g) {
-  const ElimOp* op = M.svT_ops + g.lane;
-  for (int st = 0; st < M.svT_steps; ++st, op += g.size) {
-    const ElimOp o = ld_eop(op);
-    if (o.t != OP_IDLE) {
-      if (o.kind == K_UPDATE) x[o.t] = fma(-LU[o.a], x[o.b], x[o.t]);
-      else x[o.t] *= dinv[o.a];
-    }
-    g.sync();
-  }
+// x <- A^-T x (transposed substitution with the factor LU and the reciprocal pivots behind it; x in shared memory)
+__device__ __forceinline__ void lu_solveT(const MechView& M, SPtr LU, SPtr x, const Grp1& g) {
+  run_fma<false>(M.svT, LU, x, g.lane, g.size, g);
 }
 
 // x <- M^-T x with M^T = A^T - v u^T:  x = A^-T x + zt (u . A^-T x) / (1 - u . zt),  zt = A^-T v
-__device__ __forceinline__ void smT_solve(const MechView& M, const double* LU, const double* dinv, const double* u,
-                                          const double* zt, double* x, double idenT, const Grp1& g) {
-  lu_solveT(M, LU, dinv, x, g);
+__device__ __forceinline__ void smT_solve(const MechView& M, SPtr LU, const double* u, const double* zt, SPtr x,
+                                          double idenT, const Grp1& g) {
+  lu_solveT(M, LU, x, g);
   double d = 0.0;
   for (int i = g.lane; i < M.m; i += g.size) d = fma(u[i], x[i], d);
   d = gsum(g, d) * idenT;
@@ -110,7 +103,8 @@ __device__ __forceinline__ void smT_solve(const MechView& M, const double* LU, c
   g.sync();
 }
 
-__device__ __forceinline__ void vset(double* dst, const double* src, int m, const Grp1& g) {
+template <class P, class Q>
+__device__ __forceinline__ void vset(P dst, Q src, int m, const Grp1& g) {
   for (int i = g.lane; i < m; i += g.size) dst[i] = src[i];
   g.sync();
 }
@@ -131,7 +125,7 @@ __device__ __forceinline__ void vjp_tangents(const MechView& M, const DualN<NT>*
 #pragma unroll
     for (int st = 0; st < NT; ++st) acc = fma(S[a].d[st], Ws[st][1 + b], acc);
     return acc;
-  }, g);
+  }, [](double v, int) { return v; }, g);
   double t0 = 0.0, uw[NT], duw[NT];
 #pragma unroll
   for (int st = 0; st < NT; ++st) { uw[st] = 0.0; duw[st] = 0.0; }
@@ -210,7 +204,7 @@ __device__ __forceinline__ void second_order_terms(const MechView& M, void* dwv,
     yd[i] = x;
   }
   g.sync();
-  const ScalT<DT> scd = eval_jac<DT>(M, dw, Ld, yd, p, g);
+  const ScalT<DT> scd = eval_jac(M, dw, Ld, yd, p, g);
   vjp_tangents<NT>(M, dw + Ld.S, dw + Ld.u, dw + Ld.v, Ws, tmp, reinterpret_cast<double*>(dw + Ld.part), g);
   for (int i = g.lane; i < M.m; i += g.size) LAM[i] += tmp[i];
   g.sync();
@@ -232,15 +226,14 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
   double* LAM = ws + A.LAM; double* G = ws + A.G; double* Y3 = ws + A.Y3; double* Y4 = ws + A.Y4;
   const double* UY = jr + A.UY; const double* VY = jr + A.VY; double* ZT = ws + A.ZT;
   const double* LUg = jr + A.LUG;
-  double* X = s + L.U3;      // shared scratch of the transposed solves
-  double* a = s + L.ytmp;    // shared scratch of the parameter terms (n <= m)
+  const SPtr X = shared_ptr(s + L.U3);      // shared scratch of the transposed solves
+  const SPtr a = shared_ptr(s + L.ytmp);    // shared scratch of the parameter terms (n <= m)
   // ---- the step's factor (kept by the recompute) into shared memory for the first solves
   vset(s + L.LU, LUg, M.nnz_LU + m, g);
-  const double* LUs = s + L.LU;
-  const double* dinvs = s + L.dinv;
+  const SPtr LUs = shared_ptr(s + L.LU);
   // transposed Sherman-Morrison vector zt = A^-T v
   vset(X, VY, m, g);
-  lu_solveT(M, LUs, dinvs, X, g);
+  lu_solveT(M, LUs, X, g);
   double uz = 0.0;
   for (int i = g.lane; i < m; i += g.size) uz = fma(UY[i], X[i], uz);
   uz = gsum(g, uz);
@@ -262,15 +255,15 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
     // the factor back into shared memory where a stage Jacobian took its region
     if (st == 2 || st == 1) vset(s + L.LU, LUg, M.nnz_LU + m, g);
     vset(X, MUv[st], m, g);
-    smT_solve(M, LUs, dinvs, UY, ZT, X, idenT, g);
+    smT_solve(M, LUs, UY, ZT, X, idenT, g);
     double* W = Wv[st];
     vset(W, X, m, g);
     if (st >= 2) {
       // stage 4: r4 = f(Y4) + (c41 U1 + c42 U2 + c43 U3)/h, Y4 = y + a41 U1 + a43 U3;
       // stage 3: r3 = f(Y3) + (c31 U1 + c32 U2)/h,          Y3 = y + a31 U1
-      const ScalT<double> sc = eval_jac<double>(M, s, L, st == 3 ? Y4 : Y3, p, g);
+      const ScalT<double> sc = eval_jac(M, s, L, st == 3 ? Y4 : Y3, p, g);
       theta_terms(M, s + L.hRT, s + L.q, sc.T, sc.rho, sc.cp, sc.irho, W, a, GA, GE, g);
-      vjp<double>(M, s + L.S, s + L.u, s + L.v, W, G, s + L.part, g);
+      vjp(M, s + L.S, s + L.u, s + L.v, W, G, s + L.part, g);
       if (st == 3) {
         for (int i = g.lane; i < m; i += g.size) {
           MU1[i] = fma(C41 * ih, W4[i], fma(A41, G[i], MU1[i]));
@@ -293,7 +286,7 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
   double* WS = ws + A.WS;
   for (int i = g.lane; i < m; i += g.size) WS[i] = W1[i] + W2[i];
   g.sync();
-  vjp<double>(M, jr + A.SY, UY, VY, WS, G, s + L.part, g);
+  vjp(M, jr + A.SY, UY, VY, (const double*)WS, G, s + L.part, g);
   for (int i = g.lane; i < m; i += g.size) LAM[i] += G[i];
   g.sync();
   theta_terms(M, jr + A.HY, jr + A.QY, jr[A.SC], jr[A.SC + 1], jr[A.SC + 2], jr[A.SC + 3], WS, a, GA, GE, g);
@@ -327,7 +320,7 @@ __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, doubl
     for (int nn = n0; nn < n1; ++nn) {
       double* jr = ws + A.JREC + (size_t)(nn - n0) * A.jstride;
       vset(s + L.y, seg + (size_t)(nn - n0) * m, m, g);
-      const ScalT<double> sy = eval_jac<double>(M, s, L, s + L.y, p, g);
+      const ScalT<double> sy = eval_jac(M, s, L, s + L.y, p, g);
       vset(jr + A.SY, s + L.S, M.nnz_S, g);
       vset(jr + A.UY, s + L.u, m, g);
       vset(jr + A.VY, s + L.v, m, g);
@@ -336,7 +329,7 @@ __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, doubl
       if (g.lane == 0) {
         jr[A.SC] = sy.T; jr[A.SC + 1] = sy.rho; jr[A.SC + 2] = sy.cp; jr[A.SC + 3] = sy.irho;
       }
-      const StepOut so = ros_attempt(M, s, L, p, rec_h[(size_t)nn * N + cell], o.rtol, o.atol, g);
+      const StepOut so = ros_attempt(M, s, L, p, rec_h[(size_t)nn * N + cell], o.rtol, o.atol, g, 0, false);
       if (!so.good) return false;   // also a singular factor (cannot happen for a step the forward pass accepted)
       vset(jr + A.LUG, s + L.LU, M.nnz_LU + m, g);
       double* u4 = ust + (size_t)(nn - n0) * 4 * m;

@@ -576,14 +576,19 @@ chem_status chem_create(const chem_mech_desc* desc, int device, chem_handle* out
   const int n_jp = (int)hm.jpass.size() / 4;
   if (n_jp > kMaxJPass) { delete h; return fail(CHEM_EUNSUPPORTED, "too many Jacobian passes"); }
   constexpr int kMaxG = 3 + kMaxJPass;
-  size_t o_g[kNumGroups][kMaxG][2], o_lops[kNumGroups], o_sops[kNumGroups], o_tops[kNumGroups];
+  size_t o_g[kNumGroups][kMaxG][2], o_p[kNumGroups][4][2];
+  HostFma progs[kNumGroups][4];   // elimination, substitution for all and for half the lanes, transposed
   const HostGather* gs[kNumGroups][kMaxG];
   for (int w = 0; w < kNumGroups; ++w) {
     const HostProg& P = hm.prog[w];
     gs[w][0] = &P.g_omega; gs[w][1] = &P.g_row; gs[w][2] = &P.g_col;
     for (int i = 0; i < n_jp; ++i) gs[w][3 + i] = &P.g_jac[i];
     for (int i = 0; i < 3 + n_jp; ++i) { o_g[w][i][0] = put(buf, gs[w][i]->ops); o_g[w][i][1] = put(buf, gs[w][i]->comb); }
-    o_lops[w] = put(buf, P.lu_ops); o_sops[w] = put(buf, P.sv_ops); o_tops[w] = put(buf, P.svT_ops);
+    progs[w][0] = device_program(P.lu_ops, P.lu_kind, P.width, P.width, hm.nnz_LU, true);
+    progs[w][1] = device_program(P.sv_ops, P.sv_kind, P.width, P.width, hm.nnz_LU, false);
+    progs[w][2] = device_program(P.sv_ops, P.sv_kind, P.width, P.width / 2, hm.nnz_LU, false);
+    progs[w][3] = device_program(P.svT_ops, P.svT_kind, P.width, P.width, hm.nnz_LU, false);
+    for (int i = 0; i < 4; ++i) { o_p[w][i][0] = put(buf, progs[w][i].ops); o_p[w][i][1] = put(buf, progs[w][i].head); }
   }
   if ((e = cudaMalloc(&h->blob, buf.size())) != cudaSuccess) { delete h; return fail(CHEM_ENOMEM, "cudaMalloc of mechanism tables failed"); }
   if ((e = cudaMemcpy(h->blob, buf.data(), buf.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
@@ -607,9 +612,9 @@ chem_status chem_create(const chem_mech_desc* desc, int device, chem_handle* out
     V.entry_row = (const int*)(b + o_er); V.entry_col = (const int*)(b + o_ec);
     V.entry_wratio = (const double*)(b + o_ew);
     V.lu_src = (const int*)(b + o_lsrc); V.lu_diag = (const int*)(b + o_ldiag);
-    V.lu_ops = (const ElimOp*)(b + o_lops[w]); V.lu_steps = (int)P.lu_kind.size();
-    V.sv_ops = (const ElimOp*)(b + o_sops[w]); V.sv_steps = (int)P.sv_kind.size();
-    V.svT_ops = (const ElimOp*)(b + o_tops[w]); V.svT_steps = (int)P.svT_kind.size();
+    FmaProgram* vp[4] = {&V.lu, &V.sv, &V.sv2, &V.svT};
+    for (int i = 0; i < 4; ++i)
+      *vp[i] = FmaProgram{(const FmaOp*)(b + o_p[w][i][0]), (const int*)(b + o_p[w][i][1]), (int)progs[w][i].head.size()};
     V.s_out = (const int*)(b + o_sout);
     V.rx_order = (const int*)(b + o_rxo);
     V.n_jpass = n_jp;
@@ -619,7 +624,7 @@ chem_status chem_create(const chem_mech_desc* desc, int device, chem_handle* out
     for (int i = 0; i < n_jp; ++i) vg[3 + i] = &V.g_jac[i];
     for (int i = 0; i < 3 + n_jp; ++i) {
       vg[i]->ops = (const GatherOp*)(b + o_g[w][i][0]);
-      vg[i]->steps = gs[w][i]->steps;
+      vg[i]->blocks = gs[w][i]->steps / kProgBlock;
       vg[i]->n_partial = gs[w][i]->n_partial;
       vg[i]->comb = (const int*)(b + o_g[w][i][1]);
       vg[i]->n_comb = (int)gs[w][i]->comb.size() / 3;

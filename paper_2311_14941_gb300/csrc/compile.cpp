@@ -42,10 +42,10 @@ int enc_nu(int nu) {
 // groups[g] = list of (a, b) terms summed into output g.  Terms are dealt to the 32 lanes so that the
 // longest lane is as short as possible: a group longer than the per-lane target is split into pieces
 // whose partial sums are combined afterwards; pieces go to lanes largest first (LPT).  With skip_empty,
-// outputs without terms are left untouched (programs that accumulate into their outputs); otherwise
-// they are written with 0.
+// outputs without terms are left untouched; otherwise they are written with 0.  adds: the program adds to its
+// outputs.
 bool build_gather(const std::vector<std::vector<std::pair<int, int>>>& groups, HostGather& G, std::string& err,
-                  int width, bool skip_empty = false) {
+                  int width, bool skip_empty = false, bool adds = false) {
   G = HostGather();
   long total = 0;
   for (auto& g : groups) total += skip_empty ? (long)g.size() : (long)std::max<size_t>(g.size(), 1);
@@ -77,19 +77,40 @@ bool build_gather(const std::vector<std::vector<std::pair<int, int>>>& groups, H
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(),
                    [&](int x, int y) { return std::max(pieces[x].count, 1) > std::max(pieces[y].count, 1); });
-  std::vector<std::vector<int>> lane(width);
-  std::vector<long> load(width, 0);
+  // Two ways to deal the pieces, largest first: each to the lane with the least load (fewest steps), or in rounds
+  // of one piece per lane whose last terms fall on one step.  A program that adds to its outputs pays an FP64
+  // addition in every step in which some lane ends a piece: there the rounds, with one such step each, cost less.
+  auto len = [&](int pi) { return std::max(pieces[pi].count, 1); };
+  std::vector<std::vector<std::pair<int, int>>> lane(width);   // per lane: (first step, piece)
+  std::vector<int> load(width, 0);
+  std::set<int> ends;
   for (int pi : order) {
-    int l = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-    lane[l].push_back(pi);
-    load[l] += std::max(pieces[pi].count, 1);
+    const int l = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    lane[l].push_back({load[l], pi});
+    load[l] += len(pi);
+    ends.insert(load[l]);
   }
-  G.steps = (int)*std::max_element(load.begin(), load.end());
+  G.steps = *std::max_element(load.begin(), load.end());
+  if (adds) {
+    int steps = 0, rounds = 0;
+    for (size_t i = 0; i < order.size(); i += width, ++rounds) steps += len(order[i]);
+    if (steps + rounds < G.steps + (int)ends.size()) {
+      G.steps = steps;
+      for (auto& l : lane) l.clear();
+      int at = 0;
+      for (size_t i = 0; i < order.size(); i += width) {
+        at += len(order[i]);
+        for (size_t j = i; j < std::min(i + width, order.size()); ++j)
+          lane[j - i].push_back({at - len(order[j]), order[j]});
+      }
+    }
+  }
+  G.steps = (G.steps + kProgBlock - 1) / kProgBlock * kProgBlock;
   G.ops.assign((size_t)G.steps * width, GatherOp{0, 0, DST_NONE, 1});
   for (int l = 0; l < width; ++l) {
-    int s = 0;
-    for (int pi : lane[l]) {
-      const Piece& P = pieces[pi];
+    for (auto& fp : lane[l]) {
+      const Piece& P = pieces[fp.second];
+      int s = fp.first;
       const auto& terms = groups[P.g];
       const int cnt = std::max(P.count, 1);
       for (int t = 0; t < cnt; ++t, ++s) {
@@ -218,6 +239,103 @@ std::vector<int> min_degree_order(int m, const std::vector<std::vector<char>>& a
 }
 
 }  // namespace
+
+HostFma device_program(const std::vector<ElimOp>& ops, const std::vector<uint8_t>& kinds, int prog_width, int width,
+                       int nnz, bool elimination) {
+  // the ops in program order, with what they read and write: locations of v, and in the elimination the
+  // reciprocals behind them
+  struct Op {
+    FmaOp f;
+    bool recip;
+    int w, rd[2], nrd;
+    std::vector<int> succ;
+    int npred = 0, prio = 0;
+  };
+  std::vector<Op> v;
+  for (size_t st = 0; st < kinds.size(); ++st)
+    for (int l = 0; l < prog_width; ++l) {
+      const ElimOp& e = ops[st * prog_width + l];
+      if (e.t == OP_IDLE) continue;
+      Op o;
+      o.recip = kinds[st] == K_RECIP;
+      if (o.recip) {
+        o.f = FmaOp{(uint16_t)(nnz + e.t), e.a, 0, 0};
+        o.w = nnz + e.t; o.rd[0] = e.a; o.nrd = 1;
+      } else if (kinds[st] == K_SCALE) {
+        o.f = FmaOp{e.t, (uint16_t)(nnz + e.a), e.t, FM_MUL};
+        o.w = e.t; o.nrd = 0;
+        if (elimination) o.rd[o.nrd++] = nnz + e.a;
+      } else {
+        o.f = FmaOp{e.t, e.a, e.b, 0};
+        o.w = e.t; o.nrd = 0;
+        if (elimination) o.rd[o.nrd++] = e.a;
+        o.rd[o.nrd++] = e.b;
+      }
+      v.push_back(o);
+    }
+  // dependences of the program order: a read after the last write of its location, a write after the reads and
+  // the write before it
+  {
+    std::map<int, int> last_write;
+    std::map<int, std::vector<int>> reads;
+    auto edge = [&](int from, int to) { v[from].succ.push_back(to); v[to].npred++; };
+    for (int i = 0; i < (int)v.size(); ++i) {
+      for (int k = 0; k < v[i].nrd; ++k) {
+        auto it = last_write.find(v[i].rd[k]);
+        if (it != last_write.end()) edge(it->second, i);
+        reads[v[i].rd[k]].push_back(i);
+      }
+      auto it = last_write.find(v[i].w);
+      if (it != last_write.end()) edge(it->second, i);
+      for (int r : reads[v[i].w]) if (r != i) edge(r, i);
+      reads[v[i].w].clear();
+      last_write[v[i].w] = i;
+    }
+  }
+  for (int i = (int)v.size() - 1; i >= 0; --i) {
+    int best = 0;
+    for (int s : v[i].succ) best = std::max(best, v[s].prio);
+    v[i].prio = best + (v[i].recip ? 3 : 1);   // a reciprocal takes about three steps' time
+  }
+  HostFma P;
+  std::vector<std::vector<int>> steps;   // of the open block
+  const int slots = kProgBlock + (elimination ? 1 : 0);
+  auto put = [&](const std::vector<int>& ids) {
+    for (int l = 0; l < width; ++l) P.ops.push_back(l < (int)ids.size() ? v[ids[l]].f : FmaOp{0, 0, 0, FM_IDLE});
+  };
+  auto close = [&](const std::vector<int>& recips) {
+    if (steps.empty() && recips.empty()) return;
+    P.head.push_back((int)steps.size() | (recips.empty() ? 0 : 256));
+    for (int u = 0; u < kProgBlock - (int)steps.size(); ++u) put({});
+    for (auto& s : steps) put(s);
+    if (slots > kProgBlock) put(recips);
+    steps.clear();
+  };
+  std::vector<int> ready;
+  for (int i = 0; i < (int)v.size(); ++i) if (v[i].npred == 0) ready.push_back(i);
+  while (!ready.empty()) {
+    std::stable_sort(ready.begin(), ready.end(), [&](int a, int b) {
+      return v[a].prio != v[b].prio ? v[a].prio > v[b].prio : a < b;
+    });
+    const bool recip = v[ready[0]].recip;
+    std::vector<int> step, keep;
+    for (int i : ready) (v[i].recip == recip && (int)step.size() < width ? step : keep).push_back(i);
+    for (int i : step)
+      for (int s : v[i].succ) if (--v[s].npred == 0) keep.push_back(s);
+    ready.swap(keep);
+    if (recip) { close(step); continue; }
+    steps.push_back(step);
+    if ((int)steps.size() == kProgBlock) {
+      // a step of reciprocals that is due next belongs to this block
+      const bool next_recip = !ready.empty() && v[*std::min_element(ready.begin(), ready.end(), [&](int a, int b) {
+        return v[a].prio != v[b].prio ? v[a].prio > v[b].prio : a < b;
+      })].recip;
+      if (!next_recip) close({});
+    }
+  }
+  close({});
+  return P;
+}
 
 chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string& err) {
   hm = HostMech();
@@ -684,7 +802,7 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
         }
       }
       for (HostProg& Pg : hm.prog)
-        if (!build_gather(gj, Pg.g_jac[p], err, Pg.width, true)) return CHEM_EUNSUPPORTED;
+        if (!build_gather(gj, Pg.g_jac[p], err, Pg.width, true, p > 0)) return CHEM_EUNSUPPORTED;
     }
   }
   return CHEM_OK;

@@ -41,6 +41,15 @@ struct HostMech {
   long long lu_flops = 0;              // multiply-adds of one factorisation (algorithmic)
 };
 
+// A device program (see FmaOp) of an elimination or substitution program: rescheduled for `width` lanes, every
+// target's updates in the order of the given program.  nnz: entries of the factor.
+struct HostFma {
+  std::vector<FmaOp> ops;
+  std::vector<int> head;
+};
+HostFma device_program(const std::vector<ElimOp>& ops, const std::vector<uint8_t>& kinds, int prog_width, int width,
+                       int nnz, bool elimination);
+
 // Validates and compiles; returns CHEM_OK or an error code with a message in err.
 chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string& err);
 

@@ -66,6 +66,16 @@ struct GrpH {
   __device__ __forceinline__ void sync() const { __syncwarp(mask); }
 };
 
+// Ordering among the lanes of half a group (both halves run the same steps, so a barrier of the whole warp will do;
+// the halves of two warps are the warps themselves).
+struct SyncMask {
+  unsigned mask;
+  __device__ __forceinline__ void sync() const { __syncwarp(mask); }
+};
+__device__ __forceinline__ SyncMask half_sync(const Grp1&) { return SyncMask{0xffffffffu}; }
+__device__ __forceinline__ SyncMask half_sync(const Grp2&) { return SyncMask{0xffffffffu}; }
+__device__ __forceinline__ SyncMask half_sync(const GrpH& g) { return SyncMask{g.mask}; }
+
 __device__ __forceinline__ double gsum(const Grp1&, double v) { return warp_sum(v); }
 __device__ __forceinline__ double gsum(const GrpH& g, double v) {
 #pragma unroll
@@ -208,8 +218,9 @@ constexpr double R4_C51 = 7.496443313967647, R4_C52 = -10.24680431464352, R4_C53
                  R4_C54 = 11.70890893206160;
 constexpr double R4_C61 = 8.083246795921522, R4_C62 = -7.981132988064893, R4_C63 = -31.52159432874371,
                  R4_C64 = 16.31930543123136, R4_C65 = -6.058818238834054;
-// The same coefficients as tables for the stage loop (row k - 2 of stage k; constant memory, read
-// with warp-uniform indices).
+// The three methods as tables for one stage loop (constant memory, read with warp-uniform indices).  Row k - 2 of
+// stage k: the point y + sum_j a_kj U_j in ascending j (zero coefficients are skipped) and the coefficient sum
+// sum_j c_kj U_j in descending j.  RODAS3's stage 2 has no point of its own (a21 = 0: f(y) again).
 static __constant__ double kR4A[4][4] = {{R4_A21, 0.0, 0.0, 0.0},
                                          {R4_A31, R4_A32, 0.0, 0.0},
                                          {R4_A41, R4_A42, R4_A43, 0.0},
@@ -219,25 +230,137 @@ static __constant__ double kR4C[5][5] = {{R4_C21, 0.0, 0.0, 0.0, 0.0},
                                          {R4_C41, R4_C42, R4_C43, 0.0, 0.0},
                                          {R4_C51, R4_C52, R4_C53, R4_C54, 0.0},
                                          {R4_C61, R4_C62, R4_C63, R4_C64, R4_C65}};
+// methods 0 (RODAS3) and 1 (ROS2)
+static __constant__ double kRosA[2][3][3] = {{{0.0, 0.0, 0.0}, {A31, 0.0, 0.0}, {A41, 0.0, A43}},
+                                             {{R2_A21, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}}};
+static __constant__ double kRosC[2][3][3] = {{{C21, 0.0, 0.0}, {C31, C32, 0.0}, {C41, C42, C43}},
+                                             {{R2_C21, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}}};
+__device__ __forceinline__ double stage_a(int method, int k, int j) {   // a of stage k + 1 and U_(j+1)
+  return method == 2 ? kR4A[k - 1][j] : kRosA[method][k - 1][j];
+}
+__device__ __forceinline__ double stage_c(int method, int k, int j) {
+  return method == 2 ? kR4C[k - 1][j] : kRosC[method][k - 1][j];
+}
 
 constexpr double kInvLn10 = 0.43429448190325182765;
 constexpr double kLn10 = 2.30258509299404568402;
 
 
-__device__ __forceinline__ GatherOp ld_gop(const GatherOp* p) {
-  uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+// ---- doubles in shared memory by 32-bit address.  The compiler carries a pointer into shared memory as a 64-bit
+// number and rebuilds addresses in 64 bits; a step of a substitution takes 166 cycles with plain pointers and 130
+// with these.  The accesses are volatile: they keep their order among themselves and around barriers, which the
+// rate code, with many independent loads in flight, would pay for: it keeps plain pointers.
+struct SRef {
+  uint32_t a;
+  __device__ __forceinline__ operator double() const {
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a));
+    return v;
+  }
+  __device__ __forceinline__ SRef& operator=(double v) {
+    asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v));
+    return *this;
+  }
+  __device__ __forceinline__ SRef& operator=(const SRef& o) { return *this = (double)o; }
+  __device__ __forceinline__ SRef& operator+=(double v) { return *this = (double)*this + v; }
+  __device__ __forceinline__ SRef& operator*=(double v) { return *this = (double)*this * v; }
+};
+struct SPtr {
+  uint32_t a;
+  __device__ __forceinline__ SRef operator[](int i) const { return SRef{a + (uint32_t)i * 8u}; }
+  __device__ __forceinline__ SPtr operator+(int i) const { return SPtr{a + (uint32_t)i * 8u}; }
+  __device__ __forceinline__ SPtr operator-(int i) const { return SPtr{a - (uint32_t)i * 8u}; }
+};
+__device__ __forceinline__ SPtr shared_ptr(const double* p) { return SPtr{(uint32_t)__cvta_generic_to_shared(p)}; }
+// The number type behind a pointer (the routines below take plain pointers too: dual numbers and the adjoint's
+// records live in global memory).
+template <class P>
+struct pointee;
+template <>
+struct pointee<SPtr> {
+  using type = double;
+};
+template <class T>
+struct pointee<T*> {
+  using type = T;
+};
+template <class T>
+struct pointee<const T*> {
+  using type = T;
+};
+template <class P>
+using num = typename pointee<P>::type;
+
+// ---- running the warp programs.  A program is tens of kilobytes, more than the L1 that the cells' shared memory
+// leaves, so every step's ops come from L2, 300 to 600 cycles away.  The steps are therefore taken in blocks of
+// kProgBlock: a lane loads its ops of the next block (independent loads) before it executes the current one.  A
+// step has no branch (a divergent branch costs about 60 cycles, as much as its FP64 instruction): idle lanes take
+// part and do not store.  A step of the elimination so takes 125 to 155 cycles, of which 64 are the FP64
+// instruction; reading two steps ahead in a loop over kinds it took 640.
+__device__ __forceinline__ GatherOp as_gop(uint2 v) {
   GatherOp o;
   o.a = (uint16_t)(v.x & 0xFFFF); o.b = (uint16_t)(v.x >> 16);
   o.dst = (uint16_t)(v.y & 0xFFFF); o.flags = (uint16_t)(v.y >> 16);
   return o;
 }
 
-__device__ __forceinline__ ElimOp ld_eop(const ElimOp* p) {
-  uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
-  ElimOp o;
-  o.t = (uint16_t)(v.x & 0xFFFF); o.a = (uint16_t)(v.x >> 16);
-  o.b = (uint16_t)(v.y & 0xFFFF); o.kind = (uint16_t)(v.y >> 16);
-  return o;
+// v <- the program's result.  A: the factor; lane of width: this lane's place among the program's lanes.  RECIP:
+// elimination (v = A), false if a reciprocal is not finite.
+template <bool RECIP, class Sy>
+__device__ __forceinline__ bool run_fma(const FmaProgram& P, SPtr A, SPtr v, int lane, int width, const Sy& sy) {
+  constexpr int slots = kProgBlock + (RECIP ? 1 : 0);
+  bool ok = true;
+  if (P.blocks <= 0) return ok;
+  const uint2* op = reinterpret_cast<const uint2*>(P.ops) + lane;
+  uint2 cur[slots], nxt[slots];
+#pragma unroll
+  for (int u = 0; u < slots; ++u) nxt[u] = __ldg(op + u * width);
+  int head = RECIP ? __ldg(P.head) : 0;
+  auto step = [&](uint2 w) {
+    const int t = w.x & 0xFFFF, a = w.x >> 16, b = w.y & 0xFFFF;
+    const double old = v[t], c = A[a], x = v[b];
+    const double r = fma(-c, x, (w.y & (FM_MUL << 16)) ? -0.0 : old);
+    if (!(w.y & (FM_IDLE << 16))) v[t] = r;
+    sy.sync();
+  };
+#pragma unroll 1
+  for (int blk = 0; blk < P.blocks; ++blk) {
+    const int h = head;
+#pragma unroll
+    for (int u = 0; u < slots; ++u) cur[u] = nxt[u];
+    if (blk + 1 < P.blocks) {
+      op += slots * width;
+      if (RECIP) head = __ldg(P.head + blk + 1);
+#pragma unroll
+      for (int u = 0; u < slots; ++u) nxt[u] = __ldg(op + u * width);
+    }
+    if (!RECIP) {   // whole blocks (the first slots of the first one may be idle)
+#pragma unroll
+      for (int u = 0; u < kProgBlock; ++u) step(cur[u]);
+    } else {
+      switch (h & 255) {
+        case 8: step(cur[0]);   // fall through: the last h & 255 slots
+        case 7: step(cur[1]);
+        case 6: step(cur[2]);
+        case 5: step(cur[3]);
+        case 4: step(cur[4]);
+        case 3: step(cur[5]);
+        case 2: step(cur[6]);
+        case 1: step(cur[7]);
+        default: break;
+      }
+    }
+    if (RECIP && (h & 256)) {
+      const uint2 w = cur[slots - 1];
+      const double r = rcp_rn(v[w.x >> 16]);
+      if (!(w.y & (FM_IDLE << 16))) {
+        ok = ok && finite_bits(r);   // 1/0 is infinite
+        v[w.x & 0xFFFF] = -r;
+      }
+      sy.sync();
+    }
+  }
+  return ok;
 }
 
 // Per-cell scalars shared by all lanes (every lane holds the same values).  tj, ttau: interval and local
@@ -288,35 +411,76 @@ __device__ __forceinline__ double nu_of(int b) { return __hiloint2double(b << 16
 
 // -------------------------------------------------------------------------------------- gathers
 // out[g] = sum over the group's terms of val(a, b); partial sums of split groups are combined after.
-// ACC: out[g] += sum instead (outputs without terms in the program are left as they are).
-template <bool ACC = false, class Sc, class F, class Gp, class GT>
-__device__ __forceinline__ void run_gather(const GT& G, Sc* out, Sc* part, F valf, const Gp& g) {
+// add: out[g] += sum instead (outputs without terms in the program are left as they are).  ld(a, b) reads a term's
+// operands, fin(operands, b) multiplies them.  The operands of a block's steps are read before its sums, which are
+// a chain of FP64 instructions with nothing to wait for.
+template <class P, class PP, class Ld, class Fin, class Gp, class GT>
+__device__ __forceinline__ void run_gather(const GT& G, P out, PP part, Ld ld, Fin fin, const Gp& g,
+                                           bool add = false) {
+  using Sc = num<P>;
   Sc acc = Sc(0.0);
-  const GatherOp* op = G.ops + g.lane;
-  const int NS = G.steps;
-  const GatherOp idle{0, 0, DST_NONE, 1};
-  GatherOp n1 = NS > 0 ? ld_gop(op) : idle;
-  GatherOp n2 = NS > 1 ? ld_gop(op + g.size) : idle;
-  for (int s = 0; s < NS; ++s) {
-    const GatherOp o = n1;
-    n1 = n2;
-    if (s + 2 < NS) n2 = ld_gop(op + (size_t)(s + 2) * g.size);
-    if (!(o.flags & 1)) acc += valf(o.a, o.b);
-    if (o.dst != DST_NONE) {
-      if (o.dst & PARTIAL_BIT) part[o.dst & 0x7FFF] = acc;
-      else if (ACC) out[o.dst] += acc;
-      else out[o.dst] = acc;
-      acc = Sc(0.0);
+  const uint2* op = reinterpret_cast<const uint2*>(G.ops) + g.lane;
+  uint2 nxt[kProgBlock];
+  if (G.blocks > 0) {
+#pragma unroll
+    for (int u = 0; u < kProgBlock; ++u) nxt[u] = __ldg(op + u * g.size);
+  }
+#pragma unroll 1
+  for (int blk = 0; blk < G.blocks; ++blk) {
+    uint2 cur[kProgBlock];
+    decltype(ld(0, 0)) x[kProgBlock];
+#pragma unroll
+    for (int u = 0; u < kProgBlock; ++u) {
+      cur[u] = nxt[u];
+      x[u] = ld((int)(cur[u].x & 0xFFFF), (int)(cur[u].x >> 16));
+    }
+    if (blk + 1 < G.blocks) {
+      op += kProgBlock * g.size;
+#pragma unroll
+      for (int u = 0; u < kProgBlock; ++u) nxt[u] = __ldg(op + u * g.size);
+    }
+#pragma unroll
+    for (int u = 0; u < kProgBlock; ++u) {
+      const GatherOp o = as_gop(cur[u]);
+      const Sc sum = acc + fin(x[u], (int)o.b);
+      if (!(o.flags & 1)) acc = sum;
+      if (add) {
+        if (o.dst != DST_NONE) {
+          if (o.dst & PARTIAL_BIT) part[o.dst & 0x7FFF] = acc;
+          else out[o.dst] += acc;
+          acc = Sc(0.0);
+        }
+      } else {
+        if (o.dst < PARTIAL_BIT) out[o.dst] = acc;
+        if (o.dst >= PARTIAL_BIT && o.dst != DST_NONE) part[o.dst & 0x7FFF] = acc;
+        if (o.dst != DST_NONE) acc = Sc(0.0);
+      }
     }
   }
   g.sync();
   for (int c = g.lane; c < G.n_comb; c += g.size) {
     const int dst = __ldg(G.comb + 3 * c), f = __ldg(G.comb + 3 * c + 1), cnt = __ldg(G.comb + 3 * c + 2);
-    Sc s = Sc(0.0);
-    for (int i = 0; i < cnt; ++i) s += part[f + i];
-    if (ACC) out[dst] += s; else out[dst] = s;
+    Sc s = part[f];
+    for (int i = 1; i < cnt; ++i) s += part[f + i];
+    if (add) out[dst] += s; else out[dst] = s;
   }
   g.sync();
+}
+// sum of nu x[a] (b encodes nu), and of x[a] y[b]
+template <class P, class PP, class Q, class Gp, class GT>
+__device__ __forceinline__ void gather_nu(const GT& G, P out, PP part, Q x, const Gp& g, bool add = false) {
+  using Sc = num<P>;
+  run_gather(G, out, part, [&](int a, int) { return Sc(x[a]); }, [](const Sc& v, int b) { return nu_of(b) * v; }, g, add);
+}
+template <class T1, class T2>
+struct Pair {
+  T1 x;
+  T2 y;
+};
+template <class P, class PP, class Q1, class Q2, class Gp, class GT>
+__device__ __forceinline__ void gather_xy(const GT& G, P out, PP part, Q1 x, Q2 y, const Gp& g) {
+  using Pr = Pair<num<Q1>, num<Q2>>;
+  run_gather(G, out, part, [&](int a, int b) { return Pr{x[a], y[b]}; }, [](const Pr& v, int) { return v.x * v.y; }, g);
 }
 
 // -------------------------------------------------------------------------------------- thermo
@@ -326,9 +490,9 @@ struct SpOut {
   Sc cpR, hRT, eg, emg, yw, dcp;
 };
 
-template <class Sc, bool DERIV, class MV>
-__device__ __forceinline__ SpOut<Sc> species_item(const MV& M, int k, const Sc* y, Sc T, Sc lnT, Sc invT,
-                                                  int tj, double ttau) {
+template <class Sc, class MV, class Q>
+__device__ __forceinline__ SpOut<Sc> species_item(const MV& M, int k, Q y, Sc T, Sc lnT, Sc invT,
+                                                  int tj, double ttau, bool deriv) {
   const double* t = M.sp + k;
   const double iw = __ldg(t);
   const double* cb = t + (size_t)(4 + (less_pos(val(T), __ldg(t + 2 * M.n)) ? 0 : SP_RANGE)) * M.n;
@@ -353,15 +517,17 @@ __device__ __forceinline__ SpOut<Sc> species_item(const MV& M, int k, const Sc* 
     o.emg = srcp(o.eg);
   }
   o.yw = y[1 + k] * iw;
-  o.dcp = DERIV ? sfma(T, sfma(T, Sc(c(17)) * T + Sc(c(16)), Sc(c(15))), a1) : Sc(0.0);
+  o.dcp = Sc(0.0);
+  if (deriv) o.dcp = sfma(T, sfma(T, Sc(c(17)) * T + Sc(c(16)), Sc(c(15))), a1);
   return o;
 }
 
 // NASA-7 at T for every species, one species per lane at a time; fills C, hRT, eg = exp(g), emg = 1/eg, cpR.
 // A lane's consecutive species enter the sum of Y/W in pairs (first the pair, then the running sum).
-template <class Sc, bool DERIV, class Gp, class MV, class LT>
-__device__ __forceinline__ ScalT<Sc> eval_species(const MV& M, Sc* s, const LT& L, const Sc* y,
-                                                  double p, const Gp& g) {
+template <class P, class Q, class Gp, class MV, class LT>
+__device__ __forceinline__ ScalT<num<P>> eval_species(const MV& M, P s, const LT& L, Q y, double p, const Gp& g,
+                                                      bool deriv) {
+  using Sc = num<P>;
   ScalT<Sc> sc;
   sc.T = y[0];
   sc.lnT = slog(sc.T);
@@ -372,23 +538,23 @@ __device__ __forceinline__ ScalT<Sc> eval_species(const MV& M, Sc* s, const LT& 
   const Sc T = sc.T;
   Sc sig = Sc(0.0), cps = Sc(0.0), dcps = Sc(0.0), first = Sc(0.0);
   bool odd = false;
-  Sc* __restrict__ hRT = s + L.hRT;
-  Sc* __restrict__ egv = s + L.eg;
-  Sc* __restrict__ emg = s + L.emg;
-  Sc* __restrict__ cpv = s + L.cpR;
-  Sc* __restrict__ C = s + L.C;
+  const P hRT = s + L.hRT;
+  const P egv = s + L.eg;
+  const P emg = s + L.emg;
+  const P cpv = s + L.cpR;
+  const P C = s + L.C;
 #pragma unroll 1
   for (int k = g.lane; k < M.n; k += g.size) {
-    const SpOut<Sc> a = species_item<Sc, DERIV>(M, k, y, T, sc.lnT, sc.invT, sc.tj, sc.ttau);
+    const SpOut<Sc> a = species_item<Sc>(M, k, y, T, sc.lnT, sc.invT, sc.tj, sc.ttau, deriv);
     if (odd) sig += first + a.yw;
     else first = a.yw;
     odd = !odd;
     cps = sfma(a.yw, a.cpR, cps);
-    if (DERIV) dcps = sfma(a.yw, a.dcp, dcps);
+    if (deriv) dcps = sfma(a.yw, a.dcp, dcps);
     hRT[k] = a.hRT; egv[k] = a.eg; emg[k] = a.emg; cpv[k] = a.cpR; C[k] = a.yw;
   }
   if (odd) sig += first;
-  if (DERIV) gsum3(g, sig, cps, dcps);
+  if (deriv) gsum3(g, sig, cps, dcps);
   else gsum2(g, sig, cps);
   sc.Wbar = srcp(sig);
   sc.ctot = p * sc.invT * (1.0 / kRu);
@@ -439,29 +605,27 @@ __device__ __forceinline__ Sc rx_kf(const MV& M, int r, const RxIn& x, const Sca
 // from s[d_off + so] on).  The FP64 pipe takes one warp instruction per 64 cycles and is what bounds this code:
 // with it and the tables as structures of arrays, the source term of 65,536 cells of 53 species / 325 reactions
 // went from 2999 to 2667 us, the Jacobian of 8,191 cells from 1236 to 1071 us.
-template <class Sc, bool DERIV, class MV, class LT>
-__device__ __forceinline__ void rx_simple(const MV& M, int r, const RxIn& in, Sc* s, const LT& L, const ScalT<Sc>& sc,
-                                          bool valid, int dq_off, int d_off) {
+template <class Sc, class P, class MV, class LT>
+__device__ __forceinline__ void rx_simple(const MV& M, int r, const RxIn& in, P s, const LT& L, const ScalT<Sc>& sc,
+                                          bool valid, int dq_off, int d_off, bool deriv) {
   const int r0 = in.i.r01 & 0xffff, r1 = in.i.r01 >> 16, p0 = in.i.r2p0 >> 16, p1 = in.i.p12 & 0xffff;
-  const Sc* C = s + L.C;
-  const Sc* eg = s + L.eg;
-  const Sc* emg = s + L.emg;
+  const P C = s + L.C, eg = s + L.eg, emg = s + L.emg;
   Sc lnk;
   const Sc kf = rx_kf(M, r, in, sc, lnk);
   const Sc cr0 = C[r0], cr1 = C[r1], cp0 = C[p0], cp1 = C[p1];
-  Sc ik = eg[p0] * emg[r0];
-  ik *= eg[p1];
-  ik *= emg[r1];
+  Sc ik = Sc(eg[p0]) * Sc(emg[r0]);
+  ik *= Sc(eg[p1]);
+  ik *= Sc(emg[r1]);
   const Sc kr = kf * ik;
   const Sc q = sfma(kf, cr0 * cr1, -(kr * (cp0 * cp1)));
   if (valid) s[L.q + r] = q;
-  if constexpr (DERIV) {
-    const Sc* hRT = s + L.hRT;
+  if (deriv) {
+    const P hRT = s + L.hRT;
     const int so = __ldg(M.rxi + (size_t)r * RX_I + 13);
     const Sc dlnkf = sfma(Sc(in.Ta), sc.invT, Sc(in.b)) * sc.invT;
-    Sc sh = hRT[p0] - hRT[r0];
-    sh += hRT[p1];
-    sh -= hRT[r1];
+    Sc sh = Sc(hRT[p0]) - Sc(hRT[r0]);
+    sh += Sc(hRT[p1]);
+    sh -= Sc(hRT[r1]);
     const Sc dlnKc = smul(sh, sc.invT);
     Sc s0 = kf * cr1, s1 = kf * cr0, s2 = kr * cp1, s3 = kr * cp0;
     const Sc qf = s1 * cr1, qr = s3 * cp1;
@@ -476,7 +640,7 @@ __device__ __forceinline__ void rx_simple(const MV& M, int r, const RxIn& in, Sc
     }
     if (valid) {
       s[dq_off + r] = dq;
-      Sc* d = s + d_off + so;
+      const P d = s + (d_off + so);
       d[0] = s0; d[1] = s1; d[2] = s2; d[3] = s3;
     }
   }
@@ -492,10 +656,9 @@ struct RxCore {
 
 // Rate of progress of reaction r, specialised on the reaction type (0 elementary, 1 third-body,
 // 2 Troe).  Branch-free in the participant counts: absent occurrences read index 0 and count as 1.
-template <class Sc, int TYPE, bool DERIV, class MV>
-__device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in, const Sc* __restrict__ C,
-                                              const Sc* __restrict__ eg, const Sc* __restrict__ emg,
-                                              const Sc* __restrict__ hRT, const ScalT<Sc>& sc) {
+template <class Sc, int TYPE, class P, class MV>
+__device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in, P C, P eg, P emg, P hRT,
+                                              const ScalT<Sc>& sc, bool deriv) {
   const int* I = M.rxi + (size_t)r * RX_I;
   const double* D = M.rxd + r;
   auto par = [&](int f) { return __ldg(D + f * M.R); };
@@ -506,15 +669,17 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in
   RxCore<Sc> x;
   Sc lnkinf;
   Sc kf = rx_kf(M, r, in, sc, lnkinf);
-  x.cr0 = C[r0]; x.cr1 = nro > 1 ? C[r1] : Sc(1.0); x.cr2 = nro > 2 ? C[r2] : Sc(1.0);
-  x.cp0 = C[p0]; x.cp1 = npo > 1 ? C[p1] : Sc(1.0); x.cp2 = npo > 2 ? C[p2] : Sc(1.0);
+  auto at = [](P v, bool there, int i, double other) { return there ? Sc(v[i]) : Sc(other); };
+  x.cr0 = C[r0]; x.cr1 = at(C, nro > 1, r1, 1.0); x.cr2 = at(C, nro > 2, r2, 1.0);
+  x.cp0 = C[p0]; x.cp1 = at(C, npo > 1, p1, 1.0); x.cp2 = at(C, npo > 2, p2, 1.0);
   const Sc Pf = x.cr0 * x.cr1 * x.cr2, Pb = x.cp0 * x.cp1 * x.cp2;
   Sc Mv = sc.ctot;
   if (TYPE != 0) {
     const int eo = __ldg(I + 11), ec = __ldg(I + 12);
-    for (int i = 0; i < ec; ++i) Mv = sfma(Sc(__ldg(M.eff_am1 + eo + i)), C[__ldg(M.eff_sp + eo + i)], Mv);
+    for (int i = 0; i < ec; ++i) Mv = sfma(Sc(__ldg(M.eff_am1 + eo + i)), Sc(C[__ldg(M.eff_sp + eo + i)]), Mv);
   }
-  x.dlnkf_dT = DERIV ? sfma(Ta, sc.invT, bb) * sc.invT : Sc(0.0);
+  x.dlnkf_dT = Sc(0.0);
+  if (deriv) x.dlnkf_dT = sfma(Ta, sc.invT, bb) * sc.invT;
   x.dlnk_dlnM = Sc(0.0);
   x.iM = Sc(0.0);
   if (TYPE == 2) {
@@ -528,7 +693,7 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in
     bool tfc = false;
     if constexpr (is_real<Sc>()) tfc = sc.tj >= 0 && M.tab_deg[3] > 0;
     Sc e3 = Sc(0.0), e1 = Sc(0.0), e2 = Sc(0.0), Fc;
-    if (!tfc || DERIV) {
+    if (!tfc || deriv) {
       e3 = sexp(-sc.T * par(8));
       e1 = sexp(-sc.T * par(9));
       e2 = less_pos(0.0, T2) ? sexp(-T2 * sc.invT) : Sc(0.0);
@@ -554,7 +719,7 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in
     const Sc F = sexp(Lc * ib * kLn10);
     const Sc ipr1 = den * S2 * R;
     kf = kf * (Pr * ipr1) * F;
-    if (DERIV) {
+    if (deriv) {
       const Sc dlnk0_dT = sfma(Sc(par(5)), sc.invT, Sc(par(4))) * sc.invT;
       const Sc dlnPr_dT = dlnk0_dT - x.dlnkf_dT;
       const Sc dFc_dT = -(par(6) * par(8)) * e3 - (par(7) * par(9)) * e1 +
@@ -572,18 +737,18 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in
   }
   // reverse rate: k_r = k_f * prod exp(g)^nu'' * prod exp(-g)^nu' * (Ru T/p0)^(sum nu)
   const int dn = npo - nro;
-  Sc ik = eg[p0] * emg[r0];
-  ik *= (npo > 1 ? eg[p1] : Sc(1.0)) * (npo > 2 ? eg[p2] : Sc(1.0));
-  ik *= (nro > 1 ? emg[r1] : Sc(1.0)) * (nro > 2 ? emg[r2] : Sc(1.0));
+  Sc ik = Sc(eg[p0]) * Sc(emg[r0]);
+  ik *= at(eg, npo > 1, p1, 1.0) * at(eg, npo > 2, p2, 1.0);
+  ik *= at(emg, nro > 1, r1, 1.0) * at(emg, nro > 2, r2, 1.0);
   const Sc fp = dn > 0 ? sc.rtp : sc.irtp;
   const int adn = dn < 0 ? -dn : dn;
   ik *= (adn >= 1 ? fp : Sc(1.0)) * (adn >= 2 ? fp : Sc(1.0)) * (adn >= 3 ? fp : Sc(1.0));
   x.kr = rev ? kf * ik : Sc(0.0);
   x.kf = kf;
-  if (DERIV) {
-    Sc sh = hRT[p0] - hRT[r0];
-    sh += (npo > 1 ? hRT[p1] : Sc(0.0)) + (npo > 2 ? hRT[p2] : Sc(0.0));
-    sh -= (nro > 1 ? hRT[r1] : Sc(0.0)) + (nro > 2 ? hRT[r2] : Sc(0.0));
+  if (deriv) {
+    Sc sh = Sc(hRT[p0]) - Sc(hRT[r0]);
+    sh += at(hRT, npo > 1, p1, 0.0) + at(hRT, npo > 2, p2, 0.0);
+    sh -= at(hRT, nro > 1, r1, 0.0) + at(hRT, nro > 2, r2, 0.0);
     const double dnd = dn == 0 ? 0.0 : dn == 1 ? 1.0 : dn == -1 ? -1.0 : dn == 2 ? 2.0 : dn == -2 ? -2.0 :
                        dn == 3 ? 3.0 : -3.0;
     x.dlnKc_dT = rev ? (sh - dnd) * sc.invT : Sc(0.0);
@@ -593,19 +758,23 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in
   x.Mfac = (TYPE == 1) ? Mv : Sc(1.0);
   x.qn = sfma(kf, Pf, -(x.kr * Pb));
   x.q = x.Mfac * x.qn;
-  x.so = DERIV ? __ldg(I + 13) : 0;
-  x.scn = DERIV ? __ldg(I + 14) : 0;
+  x.so = 0;
+  x.scn = 0;
+  if (deriv) {
+    x.so = __ldg(I + 13);
+    x.scn = __ldg(I + 14);
+  }
   return x;
 }
 
-// Store q (and with DERIV: dq/dT at fixed C into s[dq_off + r], and the derivative slots dq/dC_j into
+// Store q (and with deriv: dq/dT at fixed C into s[dq_off + r], and the derivative slots dq/dC_j into
 // s[d_off + slot]) of reaction r.
-template <class Sc, int TYPE, bool DERIV, class MV, class LT>
-__device__ __forceinline__ void rx_store(const MV& M, int r, const RxCore<Sc>& x, Sc* s, const LT& L,
-                                         const ScalT<Sc>& sc, bool valid, int dq_off, int d_off) {
+template <class Sc, int TYPE, class P, class MV, class LT>
+__device__ __forceinline__ void rx_store(const MV& M, int r, const RxCore<Sc>& x, P s, const LT& L,
+                                         const ScalT<Sc>& sc, bool valid, int dq_off, int d_off, bool deriv) {
   if (!valid) return;
   s[L.q + r] = x.q;
-  if (!DERIV) return;
+  if (!deriv) return;
   const Sc kfM = x.kf * x.Mfac, krM = x.kr * x.Mfac;
   const Sc qf = kfM * x.cr0 * x.cr1 * x.cr2, qr = krM * x.cp0 * x.cp1 * x.cp2;
   Sc dqdM = Sc(0.0);
@@ -645,22 +814,19 @@ __device__ __forceinline__ void rx_store(const MV& M, int r, const RxCore<Sc>& x
 // segment has warp-uniform control flow; the elementary ones go in rounds of one reaction per lane, and a round
 // whose reactions are all simple takes the short form (every lane of a round's warp takes part: lanes past the
 // end repeat the last reaction and store nothing).
-template <class Sc, bool DERIV, class Gp, class MV, class LT>
-__device__ __forceinline__ void eval_reactions(const MV& M, Sc* s, const LT& L, const ScalT<Sc>& sc,
-                                               const Gp& g, int rb, int re, int dq_off = 0, int d_off = 0) {
-  const Sc* C = s + L.C;
-  const Sc* eg = s + L.eg;
-  const Sc* emg = s + L.emg;
-  const Sc* hRT = s + L.hRT;
+template <class Sc, class P, class Gp, class MV, class LT>
+__device__ __forceinline__ void eval_reactions(const MV& M, P s, const LT& L, const ScalT<Sc>& sc,
+                                               const Gp& g, int rb, int re, int dq_off, int d_off, bool deriv) {
+  const P C = s + L.C, eg = s + L.eg, emg = s + L.emg, hRT = s + L.hRT;
   const int t1 = min(re, M.n_troe), e0 = M.n_troe + M.n_tb, b1 = min(re, e0);
 #pragma unroll 1
   for (int r = rb + g.lane; r < t1; r += g.size)
-    rx_store<Sc, 2, DERIV>(M, r, rx_core<Sc, 2, DERIV>(M, r, ld_rx(M, r), C, eg, emg, hRT, sc), s, L, sc, true, dq_off,
-                           d_off);
+    rx_store<Sc, 2>(M, r, rx_core<Sc, 2, P>(M, r, ld_rx(M, r), C, eg, emg, hRT, sc, deriv), s, L, sc, true, dq_off, d_off,
+                     deriv);
 #pragma unroll 1
   for (int r = max(rb, M.n_troe) + g.lane; r < b1; r += g.size)
-    rx_store<Sc, 1, DERIV>(M, r, rx_core<Sc, 1, DERIV>(M, r, ld_rx(M, r), C, eg, emg, hRT, sc), s, L, sc, true, dq_off,
-                           d_off);
+    rx_store<Sc, 1>(M, r, rx_core<Sc, 1, P>(M, r, ld_rx(M, r), C, eg, emg, hRT, sc, deriv), s, L, sc, true, dq_off, d_off,
+                     deriv);
   const int r0 = max(rb, e0);
   if (r0 < re) {
     RxIn next = ld_rx(M, min(r0 + g.lane, re - 1));
@@ -671,75 +837,79 @@ __device__ __forceinline__ void eval_reactions(const MV& M, Sc* s, const LT& L, 
       const RxIn in = next;
       if (base + g.size < re) next = ld_rx(M, min(base + g.size + g.lane, re - 1));
       if (wall(g, (in.i.flags & RXF_SIMPLE) != 0))
-        rx_simple<Sc, DERIV>(M, r, in, s, L, sc, valid, dq_off, d_off);
+        rx_simple<Sc>(M, r, in, s, L, sc, valid, dq_off, d_off, deriv);
       else
-        rx_store<Sc, 0, DERIV>(M, r, rx_core<Sc, 0, DERIV>(M, r, in, C, eg, emg, hRT, sc), s, L, sc, valid, dq_off,
-                               d_off);
+        rx_store<Sc, 0>(M, r, rx_core<Sc, 0, P>(M, r, in, C, eg, emg, hRT, sc, deriv), s, L, sc, valid, dq_off, d_off,
+                     deriv);
     }
   }
   g.sync();
 }
 
 // -------------------------------------------------------------------------------------- f and J
-// f(y) into out[m].  Uses C/hRT/eg/emg/cpR/q scratch.  Returns the scalars of the evaluation.
-template <class Sc, class Gp, class MV, class LT>
-__device__ __forceinline__ ScalT<Sc> eval_f(const MV& M, Sc* s, const LT& L, const Sc* y, double p,
-                                            Sc* out, const Gp& g) {
-  ScalT<Sc> sc = eval_species<Sc, false>(M, s, L, y, p, g);
-  eval_reactions<Sc, false>(M, s, L, sc, g, 0, M.R);
-  const Sc* q = s + L.q;
-  Sc* part = s + L.part;
-  Sc* w = out + 1;   // production rates written in place, then scaled
-  run_gather(M.g_omega, w, part, [&](int a, int b) { return nu_of(b) * q[a]; }, g);
+// The rates at y: C, h/RT, the rates of progress q and the production rates w_k into w[n].  With deriv also the
+// Y block of S (Dtil) and w_T in the T-column slots of S.  For those the reactions run in passes (see
+// MechView::jpass): each pass leaves dq/dT and the derivative slots of its reactions in the region D, and its
+// gather adds them into S.  deriv is a run-time flag so that a kernel that needs both holds the code once.
+template <class P, class Q, class Gp, class MV, class LT>
+__device__ __forceinline__ ScalT<num<P>> eval_rates(const MV& M, P s, const LT& L, Q y, double p, P w, const Gp& g,
+                                                    bool deriv) {
+  using Sc = num<P>;
+  const ScalT<Sc> sc = eval_species(M, s, L, y, p, g, deriv);
+  const P S = s + L.S, part = s + L.part;
+  if (deriv)
+    for (int e = g.lane; e < M.nY + M.n; e += g.size) S[e] = Sc(0.0);
+  const int passes = deriv ? M.n_jpass : 1;
+#pragma unroll 1
+  for (int ps = 0; ps < passes; ++ps) {
+    const int rb = deriv ? M.jpass[ps][JP_RB] : 0, re = deriv ? M.jpass[ps][JP_RE] : M.R;
+    const int cnt = M.jpass[ps][JP_CNT];
+    eval_reactions<Sc>(M, s, L, sc, g, rb, re, L.D - rb, L.D + cnt - M.jpass[ps][JP_SB], deriv);
+    if (deriv) gather_nu(M.g_jac[ps], S, part, s + L.D, g, ps > 0);
+  }
+  gather_nu(M.g_omega, w, part, s + L.q, g);
+  return sc;
+}
+
+// f from the production rates, in place: out[1 + k] holds w_k on entry.
+template <class Sc, class P, class Gp, class MV, class LT>
+__device__ __forceinline__ void finish_f(const MV& M, P s, const LT& L, const ScalT<Sc>& sc, P out, const Gp& g) {
+  const P w = out + 1;
   Sc Qs = Sc(0.0);
   for (int k = g.lane; k < M.n; k += g.size) {
     const Sc om = w[k];
-    Qs = sfma(s[L.hRT + k], om, Qs);
+    Qs = sfma(Sc(s[L.hRT + k]), om, Qs);
     w[k] = om * __ldg(M.sp + M.n + k) * sc.irho;
   }
   Qs = gsum(g, Qs);
   if (g.lane == 0) out[0] = sdiv(-kRu * sc.T * Qs, sc.rho * sc.cp);
   g.sync();
+}
+
+// f(y) into out[m].  Uses C/hRT/eg/emg/cpR/q scratch.  Returns the scalars of the evaluation.
+template <class P, class Q, class Gp, class MV, class LT>
+__device__ __forceinline__ ScalT<num<P>> eval_f(const MV& M, P s, const LT& L, Q y, double p, P out, const Gp& g) {
+  const ScalT<num<P>> sc = eval_rates(M, s, L, y, p, out + 1, g, false);
+  finish_f(M, s, L, sc, out, g);
   return sc;
 }
 
-// f(y) into f0[m], S[nnz_S] (internal order), u[m], v[m].  Scratch: C.., q, the pass region D, x (w),
-// U1 (g), U2 (t).  The reactions run in passes (see MechView::jpass): each pass leaves dq/dT and the
-// derivative slots of its reactions in the region, and its gather adds them into the Y block of S
-// (Dtil) and into the T-column slots of S, which hold w_T until the T column is formed below.
-template <class Sc, class Gp, class MV, class LT>
-__device__ __forceinline__ ScalT<Sc> eval_jac(const MV& M, Sc* s, const LT& L, const Sc* y, double p,
-                                              const Gp& g) {
-  ScalT<Sc> sc = eval_species<Sc, true>(M, s, L, y, p, g);
-  Sc* part = s + L.part;
-  Sc* w = s + L.x;      // w_k
-  Sc* gk = s + L.U1;
-  Sc* tk = s + L.U2;
-  Sc* S = s + L.S;
-  Sc* wT = S + M.nY;    // w_T,k, until overwritten by the T column
-  const Sc* C = s + L.C;
-  const Sc* hRT = s + L.hRT;
-  const Sc* reg = s + L.D;
-  for (int e = g.lane; e < M.nY + M.n; e += g.size) S[e] = Sc(0.0);
-  for (int ps = 0; ps < M.n_jpass; ++ps) {
-    const int rb = M.jpass[ps][JP_RB], cnt = M.jpass[ps][JP_CNT];
-    eval_reactions<Sc, true>(M, s, L, sc, g, rb, M.jpass[ps][JP_RE], L.D - rb, L.D + cnt - M.jpass[ps][JP_SB]);
-    run_gather<true>(M.g_jac[ps], S, part, [&](int a, int b) { return nu_of(b) * reg[a]; }, g);
-  }
-  const Sc* q = s + L.q;
-  run_gather(M.g_omega, w, part, [&](int a, int b) { return nu_of(b) * q[a]; }, g);
-  run_gather(M.g_row, gk, part, [&](int a, int b) { return S[a] * C[b]; }, g);
-  run_gather(M.g_col, tk, part, [&](int a, int b) { return S[a] * hRT[b]; }, g);
-  Sc* f = s + L.f0;
-  Sc* u = s + L.u;
-  Sc* v = s + L.v;
+// f(y) into f0[m], S[nnz_S] (internal order), u[m], v[m] from what eval_rates with deriv left: w_k in x, Dtil and
+// w_T in S (the T column takes w_T's place).  Scratch: U1 (g), U2 (t).
+template <class Sc, class P, class Gp, class MV, class LT>
+__device__ __forceinline__ void finish_jac(const MV& M, P s, const LT& L, const ScalT<Sc>& sc, const Gp& g) {
+  const P w = s + L.x, gk = s + L.U1, tk = s + L.U2, S = s + L.S, wT = s + (L.S + M.nY);
+  const P C = s + L.C, hRT = s + L.hRT;
+  gather_xy(M.g_row, gk, s + L.part, S, C, g);
+  gather_xy(M.g_col, tk, s + L.part, S, hRT, g);
+  const P f = s + L.f0, u = s + L.u, v = s + L.v;
   const Sc T = sc.T;
   // f, u and the T column; partial sums for the T row scalars
   Sc Qs = Sc(0.0), A1 = Sc(0.0), A2 = Sc(0.0);
   for (int k = g.lane; k < M.n; k += g.size) {
     const double Wk = __ldg(M.sp + M.n + k);
     const Sc om = w[k], g = gk[k];
-    const Sc dwT = sfma(-g, sc.invT, wT[k]);   // read before the T column overwrites w_T
+    const Sc dwT = sfma(-g, sc.invT, Sc(wT[k]));   // read before the T column overwrites w_T
     const Sc fk = Wk * om * sc.irho;
     f[1 + k] = fk;
     u[1 + k] = Wk * sc.irho * (om - g);
@@ -747,7 +917,7 @@ __device__ __forceinline__ ScalT<Sc> eval_jac(const MV& M, Sc* s, const LT& L, c
     v[1 + k] = sc.Wbar * __ldg(M.sp + k);
     const Sc h = hRT[k];
     Qs = sfma(h, om, Qs);
-    A1 = sfma(s[L.cpR + k], om, sfma(T * h, dwT, A1));
+    A1 = sfma(Sc(s[L.cpR + k]), om, sfma(T * h, dwT, A1));
     A2 = sfma(h, g, A2);
   }
   gsum3(g, Qs, A1, A2);
@@ -756,7 +926,7 @@ __device__ __forceinline__ ScalT<Sc> eval_jac(const MV& M, Sc* s, const LT& L, c
   // T row: S_Tj for species j, then S_TT; u_T; v_T
   for (int j = g.lane; j < M.n; j += g.size) {
     const double iw = __ldg(M.sp + j);
-    S[M.nY + M.n + 1 + j] = sdiv(-kRu * sfma(T, tk[j], fT * s[L.cpR + j]) * iw, sc.cp);
+    S[M.nY + M.n + 1 + j] = sdiv(-kRu * sfma(T, Sc(tk[j]), fT * Sc(s[L.cpR + j])) * iw, sc.cp);
   }
   if (g.lane == 0) {
     f[0] = fT;
@@ -768,6 +938,13 @@ __device__ __forceinline__ ScalT<Sc> eval_jac(const MV& M, Sc* s, const LT& L, c
   // species block: S_kj = (W_k / W_j) Dtil_kj (after the row and column sums used Dtil)
   for (int e = g.lane; e < M.nY; e += g.size) S[e] *= __ldg(M.entry_wratio + e);
   g.sync();
+}
+
+// f(y) into f0[m], S[nnz_S] (internal order), u[m], v[m].  Scratch: C.., q, the pass region D, x, U1, U2.
+template <class P, class Q, class Gp, class MV, class LT>
+__device__ __forceinline__ ScalT<num<P>> eval_jac(const MV& M, P s, const LT& L, Q y, double p, const Gp& g) {
+  const ScalT<num<P>> sc = eval_rates(M, s, L, y, p, s + L.x, g, true);
+  finish_jac(M, s, L, sc, g);
   return sc;
 }
 
@@ -775,92 +952,42 @@ __device__ __forceinline__ ScalT<Sc> eval_jac(const MV& M, Sc* s, const LT& L, c
 // LU of A = I/(h gamma) - S, in place, by the precomputed elimination program.  false if a pivot is 0
 // or not finite.
 template <class Gp, class MV, class LT>
-__device__ __forceinline__ bool lu_build_factor(const MV& M, double* s, const LT& L, double gh,
+__device__ __forceinline__ bool lu_build_factor(const MV& M, SPtr s, const LT& L, double gh,
                                                 const Gp& g) {
-  double* LU = s + L.LU;
-  double* dinv = s + L.dinv;
-  const double* S = s + L.S;
+  const SPtr LU = s + L.LU;   // followed by the negated reciprocal pivots (L.dinv)
+  const SPtr S = s + L.S;
   for (int l = g.lane; l < M.nnz_LU; l += g.size) {
     const int src = __ldg(M.lu_src + l);
-    LU[l] = src >= 0 ? -S[src] : 0.0;
+    const double v = S[max(src, 0)];
+    LU[l] = src >= 0 ? -v : 0.0;
   }
   g.sync();
   for (int i = g.lane; i < M.m; i += g.size) LU[__ldg(M.lu_diag + i)] += gh;
   g.sync();
-  bool ok = true;
-  const ElimOp* op = M.lu_ops + g.lane;
-  const int NS = M.lu_steps;
-  ElimOp n1 = NS > 0 ? ld_eop(op) : ElimOp{OP_IDLE, 0, 0, 0};
-  ElimOp n2 = NS > 1 ? ld_eop(op + g.size) : ElimOp{OP_IDLE, 0, 0, 0};
-  for (int st = 0; st < NS; ++st) {
-    const ElimOp o = n1;
-    n1 = n2;
-    if (st + 2 < NS) n2 = ld_eop(op + (size_t)(st + 2) * g.size);
-    const int kind = o.kind;
-    if (o.t != OP_IDLE) {
-      if (kind == K_UPDATE) {
-        LU[o.t] = fma(-LU[o.a], LU[o.b], LU[o.t]);
-      } else if (kind == K_SCALE) {
-        LU[o.t] *= dinv[o.a];
-      } else {
-        const double d = LU[o.a];
-        const double r = rcp_rn(d);
-        ok = ok && finite_bits(r);   // 1/0 is infinite
-        dinv[o.t] = r;
-      }
-    }
-    g.sync();
-  }
-  return gall(g, ok);
+  return gall(g, run_fma<true>(M.lu, LU, LU, g.lane, g.size, g));
 }
 
 // x <- A^{-1} x (forward and backward substitution by the precomputed program; state-order vector).
-// With x2 != nullptr the same program solves a second right-hand side in the same steps.
-template <bool TWO, class Gp, class MV, class LT>
-__device__ __forceinline__ void lu_solve_impl(const MV& M, const double* s, const LT& L, double* x,
-                                              double* x2, const Gp& g) {
-  const double* LU = s + L.LU;
-  const double* dinv = s + L.dinv;
-  const ElimOp* op = M.sv_ops + g.lane;
-  const int S = M.sv_steps;
-  // the factor does not change during the solve: each step's coefficient (L/U entry or 1/pivot; idle
-  // ops read entry 0) is loaded one step ahead, off the step-to-step dependence through x
-  auto coef = [&](const ElimOp& o) { return (o.kind == K_UPDATE ? LU : dinv)[o.a]; };
-  ElimOp n1 = S > 0 ? ld_eop(op) : ElimOp{OP_IDLE, 0, 0, K_SCALE};
-  ElimOp n2 = S > 1 ? ld_eop(op + g.size) : ElimOp{OP_IDLE, 0, 0, K_SCALE};
-  double c1 = coef(n1);
-  for (int st = 0; st < S; ++st) {
-    const ElimOp o = n1;
-    const double c = c1;
-    n1 = n2;
-    c1 = coef(n1);
-    if (st + 2 < S) n2 = ld_eop(op + (size_t)(st + 2) * g.size);
-    if (o.t != OP_IDLE) {
-      if (o.kind == K_UPDATE) {
-        x[o.t] = fma(-c, x[o.b], x[o.t]);
-        if (TWO) x2[o.t] = fma(-c, x2[o.b], x2[o.t]);
-      } else {
-        x[o.t] *= c;
-        if (TWO) x2[o.t] *= c;
-      }
-    }
-    g.sync();
-  }
+template <class Gp, class MV, class LT>
+__device__ __forceinline__ void lu_solve(const MV& M, SPtr s, const LT& L, SPtr x, const Gp& g) {
+  run_fma<false>(M.sv, s + L.LU, x, g.lane, g.size, g);
 }
 
+// The same for two right-hand sides: half of the group's lanes take each (a step of the program has about ten ops,
+// so half the lanes need few more steps, and an FP64 instruction costs the same for 16 lanes as for 32).
 template <class Gp, class MV, class LT>
-__device__ __forceinline__ void lu_solve(const MV& M, const double* s, const LT& L, double* x,
-                                         const Gp& g) {
-  lu_solve_impl<false>(M, s, L, x, nullptr, g);
+__device__ __forceinline__ void lu_solve2(const MV& M, SPtr s, const LT& L, SPtr x1, SPtr x2, const Gp& g) {
+  constexpr int half = Gp::size / 2;
+  const bool second = g.lane >= half;
+  run_fma<false>(M.sv2, s + L.LU, second ? x2 : x1, second ? g.lane - half : g.lane, half, half_sync(g));
+  g.sync();
 }
 
 // x <- M^{-1} x with M = A - u v^T:  x = A^-1 x + z (v . A^-1 x) / (1 - v . z),  z = A^-1 u
 template <class Gp, class MV, class LT>
-__device__ __forceinline__ void sm_solve(const MV& M, const double* s, const LT& L, double* x,
-                                         double iden, const Gp& g) {
+__device__ __forceinline__ void sm_solve(const MV& M, SPtr s, const LT& L, SPtr x, double iden, const Gp& g) {
   lu_solve(M, s, L, x, g);
-  const double* v = s + L.v;
-  const double* z = s + L.z;
+  const SPtr v = s + L.v, z = s + L.z;
   double d = 0.0;
   for (int i = g.lane; i < M.m; i += g.size) d = fma(v[i], x[i], d);
   d = gsum(g, d) * iden;
@@ -874,211 +1001,113 @@ struct StepOut {
   double err;
 };
 
-// One RODAS3 attempt of size h from y (f0, S, u, v already evaluated at y).  ynew into ytmp, err into
-// the return value.  U1..U4, x, z, LU are scratch.
+// One attempt of size h from y with method 0 RODAS3, 1 ROS2 or 2 RODAS4; need_jac: f0, S, u, v are evaluated at y
+// first (otherwise they hold that already).  ynew into ytmp, err into the return value.  U1..U4, x, z, LU are
+// scratch: RODAS4's U5 lives in the Jacobian's w_k vector (x), its stage 6 gathers the coefficient sum into U1 and
+// takes U2's place, both dead by then.
+// All stages of all methods, the Jacobian included, go through one loop with one copy of the rates and of the
+// solve.  Written out, the kernel held four copies of the rates and nine of the solve and waited on instruction
+// fetch.
 template <class Gp, class MV, class LT>
-__device__ __forceinline__ StepOut ros_attempt(const MV& M, double* s, const LT& L, double p, double h,
-                                               double rtol, double atol, const Gp& g) {
+__device__ __forceinline__ StepOut ros_attempt(const MV& M, double* sd, const LT& L, double p, double h,
+                                               double rtol, double atol, const Gp& g, int method, bool need_jac) {
   StepOut so{false, 0.0};
   const int m = M.m;
+  const SPtr s = shared_ptr(sd);
   const double ih = rcp_rn(h);
-  if (!lu_build_factor(M, s, L, ih * (1.0 / RG), g)) return so;
-  double* y = s + L.y;
-  double* yt = s + L.ytmp;
-  double* f0 = s + L.f0;
-  double* U1 = s + L.U1;
-  double* U2 = s + L.U2;
-  double* U3 = s + L.U3;
-  double* U4 = s + L.U4;
-  double* z = s + L.z;
-  const double* u = s + L.u;
-  const double* v = s + L.v;
-  // z = A^-1 u (the Sherman-Morrison vector) and stage 1's A^-1 f0, in one pass of the solve program
-  for (int i = g.lane; i < m; i += g.size) { z[i] = u[i]; U1[i] = f0[i]; }
-  g.sync();
-  lu_solve_impl<true>(M, s, L, z, U1, g);
-  double vz = 0.0, vx = 0.0;
-  for (int i = g.lane; i < m; i += g.size) { vz = fma(v[i], z[i], vz); vx = fma(v[i], U1[i], vx); }
-  gsum2(g, vz, vx);
-  const double den = 1.0 - vz;
-  if ((__double_as_longlong(den) << 1) == 0 || !finite_bits(den)) return so;
-  const double iden = rcp_rn(den);
-  // stage 1: Sherman-Morrison correction of A^-1 f0
-  vx *= iden;
-  for (int i = g.lane; i < m; i += g.size) U1[i] = fma(z[i], vx, U1[i]);
-  g.sync();
-  // stage 2 (a21 = 0: f(y) again)
-  for (int i = g.lane; i < m; i += g.size) U2[i] = fma(C21 * ih, U1[i], f0[i]);
-  g.sync();
-  sm_solve(M, s, L, U2, iden, g);
-  // stage 3
-  for (int i = g.lane; i < m; i += g.size) yt[i] = fma(A31, U1[i], y[i]);
-  g.sync();
-  eval_f<double>(M, s, L, yt, p, U3, g);
-  for (int i = g.lane; i < m; i += g.size) U3[i] = fma(ih, fma(C31, U1[i], C32 * U2[i]), U3[i]);
-  g.sync();
-  sm_solve(M, s, L, U3, iden, g);
-  // stage 4
-  for (int i = g.lane; i < m; i += g.size) yt[i] = fma(A43, U3[i], fma(A41, U1[i], y[i]));
-  g.sync();
-  eval_f<double>(M, s, L, yt, p, U4, g);
-  for (int i = g.lane; i < m; i += g.size) U4[i] = fma(ih, fma(C41, U1[i], fma(C42, U2[i], C43 * U3[i])), U4[i]);
-  g.sync();
-  sm_solve(M, s, L, U4, iden, g);
-  // solution, embedded error, scaled RMS norm
-  double e2 = 0.0;
-  bool fin = true;
-  for (int i = g.lane; i < m; i += g.size) {
-    const double yn = fma(M4, U4[i], fma(M3, U3[i], fma(M1, U1[i], y[i])));
-    yt[i] = yn;
-    const double sc = fma(rtol, max_mag(y[i], yn), atol);
-    const double e = div_rn(U4[i], sc);
-    e2 = fma(e, e, e2);
-    fin = fin && finite_bits(yn);
-  }
-  e2 = gsum(g, e2);
-  fin = gall(g, fin);
-  g.sync();
-  so.err = sqrt(div_rn(e2, (double)m));
-  so.good = fin;
-  return so;
-}
-
-// One ROS2 attempt of size h from y (f0, S, u, v already evaluated at y); ynew into ytmp.
-template <class Gp, class MV, class LT>
-__device__ __forceinline__ StepOut ros2_attempt(const MV& M, double* s, const LT& L, double p, double h,
-                                                double rtol, double atol, const Gp& g) {
-  StepOut so{false, 0.0};
-  const int m = M.m;
-  const double ih = rcp_rn(h);
-  if (!lu_build_factor(M, s, L, ih * (1.0 / RG2), g)) return so;
-  double* y = s + L.y;
-  double* yt = s + L.ytmp;
-  double* f0 = s + L.f0;
-  double* U1 = s + L.U1;
-  double* U2 = s + L.U2;
-  double* z = s + L.z;
-  const double* u = s + L.u;
-  const double* v = s + L.v;
-  for (int i = g.lane; i < m; i += g.size) { z[i] = u[i]; U1[i] = f0[i]; }
-  g.sync();
-  lu_solve_impl<true>(M, s, L, z, U1, g);
-  double vz = 0.0, vx = 0.0;
-  for (int i = g.lane; i < m; i += g.size) { vz = fma(v[i], z[i], vz); vx = fma(v[i], U1[i], vx); }
-  gsum2(g, vz, vx);
-  const double den = 1.0 - vz;
-  if ((__double_as_longlong(den) << 1) == 0 || !finite_bits(den)) return so;
-  const double iden = rcp_rn(den);
-  vx *= iden;
-  for (int i = g.lane; i < m; i += g.size) U1[i] = fma(z[i], vx, U1[i]);
-  g.sync();
-  // stage 2
-  for (int i = g.lane; i < m; i += g.size) yt[i] = fma(R2_A21, U1[i], y[i]);
-  g.sync();
-  eval_f<double>(M, s, L, yt, p, U2, g);
-  for (int i = g.lane; i < m; i += g.size) U2[i] = fma(R2_C21 * ih, U1[i], U2[i]);
-  g.sync();
-  sm_solve(M, s, L, U2, iden, g);
-  double e2 = 0.0;
-  bool fin = true;
-  for (int i = g.lane; i < m; i += g.size) {
-    const double yn = fma(R2_M2, U2[i], fma(R2_M1, U1[i], y[i]));
-    yt[i] = yn;
-    const double sc = fma(rtol, max_mag(y[i], yn), atol);
-    const double e = div_rn(R2_E * (U1[i] + U2[i]), sc);
-    e2 = fma(e, e, e2);
-    fin = fin && finite_bits(yn);
-  }
-  e2 = gsum(g, e2);
-  fin = gall(g, fin);
-  g.sync();
-  so.err = sqrt(div_rn(e2, (double)m));
-  so.good = fin;
-  return so;
-}
-
-// One RODAS4 attempt of size h from y (f0, S, u, v already evaluated at y); ynew into ytmp.  U5 lives in
-// the Jacobian's w_k vector (x), which is scratch until the next Jacobian evaluation; stage 6's
-// coefficient sum is gathered into U1 and its solution U6 takes U2's place, so the attempt needs no
-// shared memory beyond RODAS3's.
-template <class Gp, class MV, class LT>
-__device__ __forceinline__ StepOut ros4_attempt(const MV& M, double* s, const LT& L, double p, double h,
-                                                double rtol, double atol, const Gp& g) {
-  StepOut so{false, 0.0};
-  const int m = M.m;
-  const double ih = rcp_rn(h);
-  if (!lu_build_factor(M, s, L, ih * (1.0 / RG4), g)) return so;
-  double* y = s + L.y;
-  double* yt = s + L.ytmp;
-  double* f0 = s + L.f0;
-  double* U1 = s + L.U1;
-  double* U2 = s + L.U2;
-  double* U3 = s + L.U3;
-  double* U4 = s + L.U4;
-  double* U5 = s + L.x;
-  double* z = s + L.z;
-  const double* u = s + L.u;
-  const double* v = s + L.v;
-  // z = A^-1 u and stage 1's A^-1 f0 in one pass of the solve program, then the Sherman-Morrison
-  // correction of stage 1
-  for (int i = g.lane; i < m; i += g.size) { z[i] = u[i]; U1[i] = f0[i]; }
-  g.sync();
-  lu_solve_impl<true>(M, s, L, z, U1, g);
-  double vz = 0.0, vx = 0.0;
-  for (int i = g.lane; i < m; i += g.size) { vz = fma(v[i], z[i], vz); vx = fma(v[i], U1[i], vx); }
-  gsum2(g, vz, vx);
-  const double den = 1.0 - vz;
-  if ((__double_as_longlong(den) << 1) == 0 || !finite_bits(den)) return so;
-  const double iden = rcp_rn(den);
-  vx *= iden;
-  for (int i = g.lane; i < m; i += g.size) U1[i] = fma(z[i], vx, U1[i]);
-  g.sync();
-  // stages 2..6 in one loop (one copy of the right-hand side and solve code: the six stages written out
-  // overflowed the instruction cache).  Stage k's point is y + sum_j a_kj U_j (stage 6: stage 5's point
-  // plus U5), its vector solves A U_k = f(point) + (1/h) sum_j c_kj U_j; the coefficient sums are formed
-  // in the order of the written-out stages, so the arithmetic is unchanged.
-  double* Us[5] = {U1, U2, U3, U4, U5};
+  const SPtr y = s + L.y, yt = s + L.ytmp, f0 = s + L.f0, U1 = s + L.U1, U2 = s + L.U2, z = s + L.z;
+  const SPtr u = s + L.u, v = s + L.v;
+  // U1..U4 are consecutive vectors, U5 is x
+  auto U = [&](int j) { return j < 4 ? U1 + j * (L.U2 - L.U1) : s + L.x; };
+  const int stages = method == 0 ? 4 : method == 1 ? 2 : 6;
+  double iden = 0.0;
 #pragma unroll 1
-  for (int k = 1; k < 6; ++k) {   // stage k + 1
-    double* out = k < 5 ? Us[k] : U2;   // stage 6's vector overwrites U2, dead by then
-    if (k < 5) {
-      for (int i = g.lane; i < m; i += g.size) {
-        double acc = y[i];
-        for (int j = 0; j < k; ++j) acc = fma(kR4A[k - 1][j], Us[j][i], acc);
-        yt[i] = acc;
+  for (int k = 0; k < stages; ++k) {   // stage k + 1
+    const SPtr out = k == 0 ? s + (L.x - 1) : k < 5 ? U(k) : U2;   // stage 1: the production rates go to x
+    const bool rates = k == 0 ? need_jac : (method != 0 || k > 1);   // RODAS3's stage 2 takes f(y) again (a21 = 0)
+    if (k > 0 && rates) {
+      if (k < 5) {
+        for (int i = g.lane; i < m; i += g.size) {
+          double acc = y[i];
+          for (int j = 0; j < k; ++j) {
+            const double a = stage_a(method, k, j);
+            if (__double2hiint(a) != 0) acc = fma(a, U(j)[i], acc);
+          }
+          yt[i] = acc;
+        }
+      } else {   // RODAS4's stage 6: stage 5's point plus U5; the coefficient sum goes into U1
+        for (int i = g.lane; i < m; i += g.size) {
+          yt[i] += U(4)[i];
+          double acc = kR4C[4][4] * U(4)[i];
+          for (int j = 3; j >= 0; --j) acc = fma(kR4C[4][j], U(j)[i], acc);
+          U1[i] = ih * acc;
+        }
       }
-    } else {   // stage 6: the coefficient sum of U1..U5 goes into U1 (not read afterwards)
-      for (int i = g.lane; i < m; i += g.size) {
-        yt[i] += U5[i];
-        double acc = kR4C[4][4] * U5[i];
-        for (int j = 3; j >= 0; --j) acc = fma(kR4C[4][j], Us[j][i], acc);
-        U1[i] = ih * acc;
-      }
+      g.sync();
     }
-    g.sync();
-    eval_f<double>(M, s, L, yt, p, out, g);
-    if (k == 1) {
-      for (int i = g.lane; i < m; i += g.size) out[i] = fma(R4_C21 * ih, U1[i], out[i]);
-    } else if (k < 5) {
-      for (int i = g.lane; i < m; i += g.size) {
-        double acc = kR4C[k - 1][k - 1] * Us[k - 1][i];
-        for (int j = k - 2; j >= 0; --j) acc = fma(kR4C[k - 1][j], Us[j][i], acc);
-        out[i] = fma(ih, acc, out[i]);
+    if (rates) {
+      double* to = sd + (k == 0 ? L.x - 1 : k < 4 ? L.U1 + k * (L.U2 - L.U1) : k == 4 ? L.x : L.U2);
+      const Scal sc = eval_rates(M, sd, L, sd + (k == 0 ? L.y : L.ytmp), p, to + 1, g, k == 0);
+      if (k == 0) finish_jac(M, sd, L, sc, g);
+      else finish_f(M, sd, L, sc, to, g);
+    }
+    if (k == 0) {
+      if (!lu_build_factor(M, s, L, ih * (method == 1 ? 1.0 / RG2 : method == 2 ? 1.0 / RG4 : 1.0 / RG), g)) return so;
+      // z = A^-1 u (the Sherman-Morrison vector) and stage 1's A^-1 f0 together, then stage 1's correction
+      for (int i = g.lane; i < m; i += g.size) { z[i] = u[i]; U1[i] = f0[i]; }
+      g.sync();
+      lu_solve2(M, s, L, z, U1, g);
+      double vz = 0.0, vx = 0.0;
+      for (int i = g.lane; i < m; i += g.size) { vz = fma(v[i], z[i], vz); vx = fma(v[i], U1[i], vx); }
+      gsum2(g, vz, vx);
+      const double den = 1.0 - vz;
+      if ((__double_as_longlong(den) << 1) == 0 || !finite_bits(den)) return so;
+      iden = rcp_rn(den);
+      vx *= iden;
+      for (int i = g.lane; i < m; i += g.size) U1[i] = fma(z[i], vx, U1[i]);
+      g.sync();
+      continue;
+    }
+    for (int i = g.lane; i < m; i += g.size) {
+      const double f = (rates ? out : f0)[i];
+      if (k == 1) {
+        out[i] = fma(stage_c(method, 1, 0) * ih, U1[i], f);
+      } else if (k < 5) {
+        int j = k - 2;
+        double acc = stage_c(method, k, k - 1) * U(k - 1)[i];
+        if (method == 0 && k == 3) {   // c42 = -1: one rounding with the product before it
+          acc = fma(C43, U(2)[i], -(double)U(1)[i]);
+          j = 0;
+        }
+        for (; j >= 0; --j) acc = fma(stage_c(method, k, j), U(j)[i], acc);
+        out[i] = fma(ih, acc, f);
+      } else {
+        out[i] = f + U1[i];
       }
-    } else {
-      for (int i = g.lane; i < m; i += g.size) out[i] += U1[i];
     }
     g.sync();
     sm_solve(M, s, L, out, iden, g);
   }
-  // solution = stage 6's point + U6, error estimate U6, scaled RMS norm
+  // solution, embedded error, scaled RMS norm (RODAS3: the error is U4; RODAS4: the solution is stage 6's point plus
+  // U6, which is the error)
+  const SPtr U3 = U(2), U4 = U(3);
   double e2 = 0.0;
   bool fin = true;
   for (int i = g.lane; i < m; i += g.size) {
-    const double yn = yt[i] + U2[i];
+    double yn, ei;
+    if (method == 0) {
+      yn = fma(M4, U4[i], fma(M3, U3[i], fma(M1, U1[i], y[i])));
+      ei = U4[i];
+    } else if (method == 1) {
+      yn = fma(R2_M2, U2[i], fma(R2_M1, U1[i], y[i]));
+      ei = R2_E * (U1[i] + U2[i]);
+    } else {
+      yn = yt[i] + U2[i];
+      ei = U2[i];
+    }
     yt[i] = yn;
     const double sc = fma(rtol, max_mag(y[i], yn), atol);
-    const double e = div_rn(U2[i], sc);
+    const double e = div_rn(ei, sc);
     e2 = fma(e, e, e2);
     fin = fin && finite_bits(yn);
   }
@@ -1115,13 +1144,14 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // Adaptive integration of the cell whose state sits in y (shared memory) over [0, dt].
 template <class Gp, class MV, class LT>
-__device__ __forceinline__ void integrate_cell(const MV& M, double* s, const LT& L, double p, double dt,
+__device__ __forceinline__ void integrate_cell(const MV& M, double* sd, const LT& L, double p, double dt,
                                                double& h_io, int& nsub, int& nacc, int& status, const IntOpts& o,
                                                const Gp& g, int cell) {
-  double* y = s + L.y;
+  const SPtr s = shared_ptr(sd), y = s + L.y;
   const int m = M.m;
   // input check
-  bool ok = isfinite(p) && p > 0.0 && isfinite(dt) && dt >= 0.0 && isfinite(y[0]) && y[0] > 0.0;
+  const double T0 = y[0];
+  bool ok = isfinite(p) && p > 0.0 && isfinite(dt) && dt >= 0.0 && isfinite(T0) && T0 > 0.0;
   double sig = 0.0;
   for (int k = g.lane; k < M.n; k += g.size) {
     const double yk = y[1 + k];
@@ -1155,13 +1185,8 @@ __device__ __forceinline__ void integrate_cell(const MV& M, double* s, const LT&
     const double hu = last ? dt - t : h;
     if (less_pos(hu, o.h_min)) { st = kCellHmin; break; }
     ++ns;
-    if (needJ) {
-      eval_jac<double>(M, s, L, y, p, g);
-      needJ = false;
-    }
-    const StepOut so = o.method == 1   ? ros2_attempt(M, s, L, p, hu, o.rtol, o.atol, g)
-                       : o.method == 2 ? ros4_attempt(M, s, L, p, hu, o.rtol, o.atol, g)
-                                       : ros_attempt(M, s, L, p, hu, o.rtol, o.atol, g);
+    const StepOut so = ros_attempt(M, sd, L, p, hu, o.rtol, o.atol, g, o.method, needJ);
+    needJ = false;
     if (o.trace && g.lane == 0 && ns <= o.trace_cap)
       o.trace[(size_t)(ns - 1) * o.N + cell] = (so.good && finite_bits(so.err) && leq_pos(so.err, 1.0)) ? hu : -hu;
     if (!so.good || !finite_bits(so.err)) {
@@ -1177,7 +1202,7 @@ __device__ __forceinline__ void integrate_cell(const MV& M, double* s, const LT&
     if (leq_pos(so.err, 1.0)) {
       t = last ? dt : t + hu;
       ++na;
-      const double* yt = s + L.ytmp;
+      const SPtr yt = s + L.ytmp;
       for (int i = g.lane; i < m; i += g.size) y[i] = yt[i];
       g.sync();
       if (o.rec_h && na <= o.rec_cap) {

@@ -24,6 +24,8 @@
 namespace chemgb {
 
 #ifdef __CUDACC__
+// the hardware's sequence, out of line: the usual case does not reach it
+static __device__ __noinline__ double slow_div(double a, double b) { return a / b; }
 CHEM_DEV unsigned long long dbits(double x) { return (unsigned long long)__double_as_longlong(x); }
 CHEM_DEV double bitsd(unsigned long long x) { return __longlong_as_double((long long)x); }
 CHEM_DEV float f_of_bits(unsigned x) { return __uint_as_float(x); }
@@ -35,6 +37,7 @@ CHEM_DEV float rcp_seed(float x) {
   return y;
 }
 #else
+inline double slow_div(double a, double b) { return a / b; }
 CHEM_DEV unsigned long long dbits(double x) { unsigned long long u; std::memcpy(&u, &x, 8); return u; }
 CHEM_DEV double bitsd(unsigned long long u) { double x; std::memcpy(&x, &u, 8); return x; }
 CHEM_DEV float f_of_bits(unsigned u) { float x; std::memcpy(&x, &u, 4); return x; }
@@ -70,7 +73,7 @@ CHEM_DEV unsigned long long recip63(unsigned long long X) {
 CHEM_DEV double rcp_rn(double d) {
   const unsigned long long b = dbits(d);
   const unsigned ed = (unsigned)(b >> 52) & 0x7ffu;
-  if (ed - 1u >= 2044u) return 1.0 / d;
+  if (ed - 1u >= 2044u) return slow_div(1.0, d);
   const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
   unsigned long long q = (recip63(m << 11) + 512u) >> 10;   // 2^105 / m within one
   const long long r = -(long long)(q * m);                  // 2^105 - q m, exact modulo 2^64
@@ -88,7 +91,7 @@ CHEM_DEV double div_rn(double a, double d) {
   const bool less = ma < md;
   const int B = 1023 + ea - ed - (less ? 1 : 0);   // biased exponent of the quotient
   const bool zero = (ba << 1) == 0;
-  if (ed - 1u >= 2046u || (!zero && (ea - 1u >= 2046u || B - 1u >= 2045u))) return a / d;
+  if (ed - 1u >= 2046u || (!zero && (ea - 1u >= 2046u || B - 1u >= 2045u))) return slow_div(a, d);
   const unsigned long long h = mul_hi64(ma << 11, recip63(md << 11));   // ma/md 2^62
   unsigned long long q = (h + (less ? 256u : 512u)) >> (less ? 9 : 10);
   const long long r = (long long)((ma << (less ? 53 : 52)) - q * md);

@@ -96,7 +96,7 @@ __global__ void k_integrate_plain(MV M, LT L, int N, double* __restrict__ T, con
   double h = h_io[c];
   int ns = 0, na = 0, st = 0;
   integrate_cell(M, s, L, p[c], dt[c], h, ns, na, st, with_deadline(o, stamp, budget_ns), g, c);
-  const double* y = s + L.y;
+  const SPtr y = shared_ptr(s) + L.y;
   for (int i = g.lane; i < M.m; i += g.size) {
     if (i == 0) T[c] = y[0];
     else Y[(size_t)(i - 1) * N + c] = y[i];
@@ -154,7 +154,7 @@ __global__ void k_integrate_persistent(MV M, LT L, int N, double* __restrict__ T
       double h = h_io[c];
       int ns = 0, na = 0, st = 0;
       integrate_cell(M, s, L, p[c], dt[c], h, ns, na, st, oo, g, c);
-      const double* y = s + L.y;
+      const SPtr y = shared_ptr(s) + L.y;
       for (int i = g.lane; i < M.m; i += g.size) {
         if (i == 0) T[c] = y[0];
         else Y[(size_t)(i - 1) * N + c] = y[i];

@@ -15,7 +15,7 @@ __global__ void k_rates(MechView M, CellLayout L, int N, const double* __restric
   if (c >= N) return;
   const Grp1 g{lane};
   double* f = s + L.f0;
-  Scal sc = eval_f<double>(M, s, L, s + L.y, p[c], f, g);
+  const Scal sc = eval_f(M, s, L, s + L.y, p[c], f, g);
   for (int i = lane; i < M.m; i += kWarp) {
     if (i == 0) dTdt[c] = f[0];
     else dYdt[(size_t)(i - 1) * N + c] = f[i];
@@ -35,7 +35,7 @@ __global__ void k_jacobian(MechView M, CellLayout L, int N, const double* __rest
   load_tile(smem, L, M.m, N, c0, wpb, T, Y);
   const int c = c0 + w;
   if (c >= N) return;
-  eval_jac<double>(M, s, L, s + L.y, p[c], Grp1{lane});
+  eval_jac(M, s, L, s + L.y, p[c], Grp1{lane});
   for (int e = lane; e < M.nnz_S; e += kWarp) Sv[(size_t)__ldg(M.s_out + e) * N + c] = s[L.S + e];
   for (int i = lane; i < M.m; i += kWarp) {
     u[(size_t)i * N + c] = s[L.u + i];

@@ -65,8 +65,10 @@ struct alignas(16) RxRec {
 enum : int { RXF_REV = 1, RXF_SIMPLE = 32, RXF_REP = 64 };
 
 // ---- warp programs, compiled for a group of `width` lanes (one warp per cell: 32, two: 64, half: 16)
+// The device reads every program in blocks of kProgBlock steps, a block ahead.
+constexpr int kProgBlock = 8;
 // Gather ("flattened segmented reduction"): step s, lane l executes op[s*width + l]:
-//   acc = fma(value(a, b), acc); if dst != NONE: out[dst] = acc, acc = 0.
+//   acc = fma(value(a, b), acc); if dst != NONE: out[dst] = acc, acc = 0.  Padded to whole blocks of steps.
 // dst >= PARTIAL_BIT selects the partial-sum buffer; a combine list then adds partials into outputs.
 struct GatherOp {
   uint16_t a, b, dst, flags;   // flags bit 0: padding (no accumulation)
@@ -84,9 +86,26 @@ struct ElimOp {
 constexpr uint16_t OP_IDLE = 0xFFFF;
 enum : int { K_RECIP = 0, K_SCALE = 1, K_UPDATE = 2 };
 
+// The same programs as the device runs them.  v = the factor's entries followed by the negated reciprocals of its
+// pivots for the elimination, the right-hand side for a substitution (whose factor is A, as above); an op is
+//   v[t] = fma(-A[a], v[b], FM_MUL ? -0 : v[t]),
+// an update or (b = t, a = a negated reciprocal) a scaling: fma(x, y, -0) is x y rounded, signed zeros included.
+// One form for both needs no branch in a step and lets them share a step.  Updates of one target keep the order
+// of the program above, so the results are its results.  A block is up to kProgBlock steps, right-aligned, then
+// in the elimination at most one step of reciprocals, v[t] = -1/v[a], in slot kProgBlock.
+struct FmaOp {
+  uint16_t t, a, b, flags;
+};
+enum : int { FM_MUL = 1, FM_IDLE = 2 };
+struct FmaProgram {
+  const FmaOp* ops;   // [blocks * (kProgBlock + recip) * width]
+  const int* head;    // [blocks] steps of the block, + 256 with a step of reciprocals
+  int blocks;
+};
+
 struct Gather {
-  const GatherOp* ops;   // [steps * 32]
-  int steps;
+  const GatherOp* ops;   // [blocks * kProgBlock * width]
+  int blocks;
   int n_partial;
   const int* comb;       // [n_comb * 3]: dst, first partial, count
   int n_comb;
@@ -127,12 +146,10 @@ struct MechView {
   Gather g_col;              // species i <- sum_k h_k Dtil_ki (a = entry, b = species k)
   const int* lu_src;         // [nnz_LU] S index feeding the slot (-1: fill)
   const int* lu_diag;        // [m] LU slot of the diagonal of state index s (natural order)
-  const ElimOp* lu_ops;      // [lu_steps * width]
-  int lu_steps;
-  const ElimOp* sv_ops;      // forward + backward substitution program, vector indices in state order
-  int sv_steps;
-  const ElimOp* svT_ops;     // transposed substitution program (A^T x = b)
-  int svT_steps;
+  FmaProgram lu;             // elimination
+  FmaProgram sv;             // forward + backward substitution, vector indices in state order
+  FmaProgram sv2;            // the same for half of the group's lanes (two right-hand sides at once)
+  FmaProgram svT;            // transposed substitution (A^T x = b)
   const int* rx_order;       // [R] compiled reaction -> description index
   const int* s_out;          // [nnz_S] position of internal S entry in the CSR output order
   // tabulated temperature functions (an opt-in approximation; tab_on == 0: every function exact):

@@ -18,6 +18,11 @@ __device__ __forceinline__ double double_of_int(int k) {
   return __hiloint2double(a ? (int)hi : 0, (int)(f << 20));
 }
 
+// The library functions that take over outside the ranges of the table-driven ones and of the integer division;
+// not inlined, so that the code of the usual case stays together.
+static __device__ __noinline__ double slow_exp(double x) { return exp(x); }
+static __device__ __noinline__ double slow_log(double x) { return log(x); }
+
 // e^x by table-driven reduction (Tang, ACM TOMS 15(2), 1989), in a variant with 256 table entries:
 //   k = nearest integer to 256 x / ln2, read from the low word of x * 256/ln2 + 1.5 * 2^52;
 //   r = x - k ln2/256 in two fused steps (the first is exact because k * kExpCHi is), |r| <= ln2/512;
@@ -26,7 +31,7 @@ __device__ __forceinline__ double double_of_int(int k) {
 // Eight FP64 operations; error about one ulp.  |x| >= 704 (results near overflow or in the subnormal
 // range) and NaN take the library exp.
 __device__ __forceinline__ double fast_exp(double x) {
-  if ((__double2hiint(x) & 0x7fffffff) >= 0x40860000) return exp(x);
+  if ((__double2hiint(x) & 0x7fffffff) >= 0x40860000) return slow_exp(x);
   constexpr double kShift = 0x1.8p52;
   const double t = fma(x, kExpInvC, kShift);
   const int k = __double2loint(t);
@@ -192,7 +197,7 @@ __device__ __forceinline__ DualN<K> smul(const DualN<K>& a, const DualN<K>& b) {
 // Zero, negative, subnormal, infinite and NaN arguments take the library log.
 __device__ __forceinline__ double fast_log(double x) {
   const int hx = __double2hiint(x);
-  if (hx < 0x00100000 || hx >= 0x7ff00000) return log(x);
+  if (hx < 0x00100000 || hx >= 0x7ff00000) return slow_log(x);
   const int k = (hx >> 20) - 1023;
   const int j = (hx >> 12) & 0xff;
   const double y = __hiloint2double((hx & 0x000fffff) | 0x3ff00000, __double2loint(x));
