@@ -120,7 +120,7 @@ template <int NT>
 __device__ __forceinline__ void vjp_tangents(const MechView& M, const DualN<NT>* S, const DualN<NT>* u,
                                              const DualN<NT>* v, const double* const* Ws, double* out, double* part,
                                              const Grp1& g) {
-  run_gather(M.g_col, out + 1, part, [&](int a, int b) {
+  run_gather<false>(M.g_col, out + 1, part, [&](int a, int b) {
     double acc = 0.0;
 #pragma unroll
     for (int st = 0; st < NT; ++st) acc = fma(S[a].d[st], Ws[st][1 + b], acc);
@@ -263,7 +263,7 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
       // stage 3: r3 = f(Y3) + (c31 U1 + c32 U2)/h,          Y3 = y + a31 U1
       const ScalT<double> sc = eval_jac(M, s, L, st == 3 ? Y4 : Y3, p, g);
       theta_terms(M, s + L.hRT, s + L.q, sc.T, sc.rho, sc.cp, sc.irho, W, a, GA, GE, g);
-      vjp(M, s + L.S, s + L.u, s + L.v, W, G, s + L.part, g);
+      vjp(M, s + L.S, s + L.u, s + L.v, W, G, shared_ptr(s + L.part), g);
       if (st == 3) {
         for (int i = g.lane; i < m; i += g.size) {
           MU1[i] = fma(C41 * ih, W4[i], fma(A41, G[i], MU1[i]));
@@ -286,7 +286,7 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
   double* WS = ws + A.WS;
   for (int i = g.lane; i < m; i += g.size) WS[i] = W1[i] + W2[i];
   g.sync();
-  vjp(M, jr + A.SY, UY, VY, (const double*)WS, G, s + L.part, g);
+  vjp(M, jr + A.SY, UY, VY, (const double*)WS, G, shared_ptr(s + L.part), g);
   for (int i = g.lane; i < m; i += g.size) LAM[i] += G[i];
   g.sync();
   theta_terms(M, jr + A.HY, jr + A.QY, jr[A.SC], jr[A.SC + 1], jr[A.SC + 2], jr[A.SC + 3], WS, a, GA, GE, g);

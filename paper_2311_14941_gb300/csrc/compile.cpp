@@ -134,6 +134,11 @@ bool build_gather(const std::vector<std::vector<std::pair<int, int>>>& groups, H
       }
     }
   }
+  for (int st = 0; st < G.steps; ++st) {
+    GatherOp* o = &G.ops[(size_t)st * width];
+    if (std::any_of(o, o + width, [](const GatherOp& x) { return x.dst != DST_NONE; }))
+      for (int l = 0; l < width; ++l) o[l].flags |= GF_END;
+  }
   return true;
 }
 
@@ -456,9 +461,10 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
     for (size_t i = 0; i < x.ro.size(); ++i) I[4 + i] = x.ro[i];
     for (size_t i = 0; i < x.po.size(); ++i) I[7 + i] = x.po[i];
     I[10] = (int)x.po.size() - (int)x.ro.size();
-    I[11] = (int)hm.eff_sp.size();
+    I[11] = (int)hm.eff.size();
     I[12] = (int)x.eff.size();
-    for (auto& e : x.eff) { hm.eff_sp.push_back(e.first); hm.eff_am1.push_back(e.second - 1.0); }
+    I[15] = I[11];
+    for (auto& e : x.eff) hm.eff.push_back(EffRec{e.second - 1.0, e.first, 0});
     for (int s : x.ro) netmap[r][s] -= 1;
     for (int s : x.po) netmap[r][s] += 1;
     // distinct column species: reactants, products, listed colliders
@@ -475,9 +481,7 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
       for (size_t i = 0; i < x.po.size(); ++i) if (x.po[i] == s) mask |= 1 << (3 + i);
       double am1 = 0.0;
       if (x.type != 0) for (auto& e : x.eff) if (e.first == s) am1 = e.second - 1.0;
-      hm.dslot_sp.push_back(s);
-      hm.dslot_mask.push_back(mask);
-      hm.dslot_am1.push_back(am1);
+      hm.dslot.push_back(SlotRec{am1, mask, 0});
       hm.n_dslot++;
     }
     slots_sp[r] = cols;
@@ -750,7 +754,8 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
       rec[r] = RxRec{sp_of(x.ro, 0) | sp_of(x.ro, 1) << 16, sp_of(x.ro, 2) | sp_of(x.po, 0) << 16,
                      sp_of(x.po, 1) | sp_of(x.po, 2) << 16,
                      (uint32_t)((x.rev ? RXF_REV : 0) | x.ro.size() << 1 | x.po.size() << 3 | (simple ? RXF_SIMPLE : 0) |
-                                (rep(x.ro) || rep(x.po) ? RXF_REP : 0))};
+                                (rep(x.ro) || rep(x.po) ? RXF_REP : 0) |
+                                (uint32_t)hm.rxi[(size_t)r * RX_I + 13] << 16)};
     }
     std::vector<int> at(R), pos(R);   // at[i]: reaction placed at i; pos: its inverse
     std::iota(at.begin(), at.end(), 0);

@@ -28,9 +28,11 @@ struct HostProg {
 struct HostMech {
   int n = 0, R = 0, m = 0, n_troe = 0, n_tb = 0, nY = 0, nnz_S = 0, nnz_LU = 0, n_dslot = 0;
   std::vector<int> rx_order;           // compiled reaction index -> description index
-  std::vector<double> sp, rxd, eff_am1, dslot_am1, entry_wratio;
+  std::vector<double> sp, rxd, entry_wratio;
   std::vector<RxRec> rxr;
-  std::vector<int> rxi, eff_sp, dslot_sp, dslot_mask, entry_row, entry_col;
+  std::vector<EffRec> eff;
+  std::vector<SlotRec> dslot;
+  std::vector<int> rxi, entry_row, entry_col;
   HostProg prog[kNumGroups];           // prog[g]: programs for lane group g (widths kGroupWidth)
   std::vector<int> jpass;              // [passes * 4]: first reaction, end reaction, first slot, reactions
   int jreg = 0;                        // doubles of the largest pass (dq/dT values + derivative slots)

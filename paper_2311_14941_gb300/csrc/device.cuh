@@ -272,6 +272,20 @@ struct SPtr {
   __device__ __forceinline__ SPtr operator-(int i) const { return SPtr{a - (uint32_t)i * 8u}; }
 };
 __device__ __forceinline__ SPtr shared_ptr(const double* p) { return SPtr{(uint32_t)__cvta_generic_to_shared(p)}; }
+// A cell's memory as the programs address it: shared memory for doubles, global memory for dual numbers.
+__device__ __forceinline__ SPtr prog_ptr(double* p) { return shared_ptr(p); }
+template <class T>
+__device__ __forceinline__ T* prog_ptr(T* p) { return p; }
+// Stores under a predicate, as one predicated instruction (the compiler makes a branch of an if, at about 60 cycles
+// when lanes disagree).
+__device__ __forceinline__ void store_if(const SPtr& p, int i, double v, bool yes) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.shared.f64 [%0], %1;\n\t}" ::"r"(p.a + (uint32_t)i * 8u),
+               "d"(v), "r"((int)yes));
+}
+template <class T>
+__device__ __forceinline__ void store_if(T* p, int i, const T& v, bool yes) {
+  if (yes) p[i] = v;
+}
 // The number type behind a pointer (the routines below take plain pointers too: dual numbers and the adjoint's
 // records live in global memory).
 template <class P>
@@ -411,12 +425,13 @@ __device__ __forceinline__ double nu_of(int b) { return __hiloint2double(b << 16
 
 // -------------------------------------------------------------------------------------- gathers
 // out[g] = sum over the group's terms of val(a, b); partial sums of split groups are combined after.
-// add: out[g] += sum instead (outputs without terms in the program are left as they are).  ld(a, b) reads a term's
-// operands, fin(operands, b) multiplies them.  The operands of a block's steps are read before its sums, which are
-// a chain of FP64 instructions with nothing to wait for.
-template <class P, class PP, class Ld, class Fin, class Gp, class GT>
-__device__ __forceinline__ void run_gather(const GT& G, P out, PP part, Ld ld, Fin fin, const Gp& g,
-                                           bool add = false) {
+// ADD: out[g] += sum instead (outputs without terms in the program are left as they are; its pieces end on common
+// steps, marked in every lane's op).  ld(a, b) reads a term's operands, fin(operands, b) multiplies them.
+//
+// Doubles: a block of steps at a time.  The operands of the block are read before its sums, which are a chain of
+// FP64 instructions with nothing to wait for.
+template <bool ADD, class P, class PP, class Ld, class Fin, class Gp, class GT>
+__device__ __forceinline__ void gather_blocks(const GT& G, P out, PP part, Ld ld, Fin fin, const Gp& g) {
   using Sc = num<P>;
   Sc acc = Sc(0.0);
   const uint2* op = reinterpret_cast<const uint2*>(G.ops) + g.lane;
@@ -443,34 +458,65 @@ __device__ __forceinline__ void run_gather(const GT& G, P out, PP part, Ld ld, F
     for (int u = 0; u < kProgBlock; ++u) {
       const GatherOp o = as_gop(cur[u]);
       const Sc sum = acc + fin(x[u], (int)o.b);
-      if (!(o.flags & 1)) acc = sum;
-      if (add) {
-        if (o.dst != DST_NONE) {
-          if (o.dst & PARTIAL_BIT) part[o.dst & 0x7FFF] = acc;
-          else out[o.dst] += acc;
-          acc = Sc(0.0);
+      if (!(o.flags & GF_IDLE)) acc = sum;
+      const bool end = o.dst != DST_NONE, partial = (o.dst & PARTIAL_BIT) != 0;
+      if (ADD) {
+        if (o.flags & GF_END) {
+          if (end && !partial) out[o.dst] += acc;
+          if (end && partial) part[o.dst & 0x7FFF] = acc;
+          if (end) acc = Sc(0.0);
         }
       } else {
-        if (o.dst < PARTIAL_BIT) out[o.dst] = acc;
-        if (o.dst >= PARTIAL_BIT && o.dst != DST_NONE) part[o.dst & 0x7FFF] = acc;
-        if (o.dst != DST_NONE) acc = Sc(0.0);
+        store_if(out, o.dst, acc, !partial);
+        store_if(part, o.dst & 0x7FFF, acc, end && partial);
+        if (end) acc = Sc(0.0);
       }
     }
   }
+}
+// Dual numbers: step by step (a step is long, and the operands of a block would spill).
+template <bool ADD, class P, class PP, class Ld, class Fin, class Gp, class GT>
+__device__ __forceinline__ void gather_steps(const GT& G, P out, PP part, Ld ld, Fin fin, const Gp& g) {
+  using Sc = num<P>;
+  Sc acc = Sc(0.0);
+  const uint2* op = reinterpret_cast<const uint2*>(G.ops) + g.lane;
+  const int steps = G.blocks * kProgBlock;
+  const uint2 idle = make_uint2(0u, (GF_IDLE << 16) | DST_NONE);
+  uint2 n1 = steps > 0 ? __ldg(op) : idle, n2 = steps > 1 ? __ldg(op + g.size) : idle;
+#pragma unroll 1
+  for (int st = 0; st < steps; ++st) {
+    const GatherOp o = as_gop(n1);
+    n1 = n2;
+    if (st + 2 < steps) n2 = __ldg(op + (size_t)(st + 2) * g.size);
+    if (!(o.flags & GF_IDLE)) acc += fin(ld(o.a, o.b), (int)o.b);
+    if (o.dst != DST_NONE) {
+      if (o.dst & PARTIAL_BIT) part[o.dst & 0x7FFF] = acc;
+      else if (ADD) out[o.dst] += acc;
+      else out[o.dst] = acc;
+      acc = Sc(0.0);
+    }
+  }
+}
+template <bool ADD, class P, class PP, class Ld, class Fin, class Gp, class GT>
+__device__ __forceinline__ void run_gather(const GT& G, P out, PP part, Ld ld, Fin fin, const Gp& g) {
+  using Sc = num<P>;
+  if constexpr (is_real<Sc>()) gather_blocks<ADD>(G, out, part, ld, fin, g);
+  else gather_steps<ADD>(G, out, part, ld, fin, g);
   g.sync();
   for (int c = g.lane; c < G.n_comb; c += g.size) {
     const int dst = __ldg(G.comb + 3 * c), f = __ldg(G.comb + 3 * c + 1), cnt = __ldg(G.comb + 3 * c + 2);
     Sc s = part[f];
     for (int i = 1; i < cnt; ++i) s += part[f + i];
-    if (add) out[dst] += s; else out[dst] = s;
+    if (ADD) out[dst] += s; else out[dst] = s;
   }
   g.sync();
 }
 // sum of nu x[a] (b encodes nu), and of x[a] y[b]
-template <class P, class PP, class Q, class Gp, class GT>
-__device__ __forceinline__ void gather_nu(const GT& G, P out, PP part, Q x, const Gp& g, bool add = false) {
+template <bool ADD, class P, class PP, class Q, class Gp, class GT>
+__device__ __forceinline__ void gather_nu(const GT& G, P out, PP part, Q x, const Gp& g) {
   using Sc = num<P>;
-  run_gather(G, out, part, [&](int a, int) { return Sc(x[a]); }, [](const Sc& v, int b) { return nu_of(b) * v; }, g, add);
+  run_gather<ADD>(G, out, part, [&](int a, int) { return Sc(x[a]); }, [](const Sc& v, int b) { return nu_of(b) * v; },
+                  g);
 }
 template <class T1, class T2>
 struct Pair {
@@ -480,7 +526,8 @@ struct Pair {
 template <class P, class PP, class Q1, class Q2, class Gp, class GT>
 __device__ __forceinline__ void gather_xy(const GT& G, P out, PP part, Q1 x, Q2 y, const Gp& g) {
   using Pr = Pair<num<Q1>, num<Q2>>;
-  run_gather(G, out, part, [&](int a, int b) { return Pr{x[a], y[b]}; }, [](const Pr& v, int) { return v.x * v.y; }, g);
+  run_gather<false>(G, out, part, [&](int a, int b) { return Pr{x[a], y[b]}; },
+                    [](const Pr& v, int) { return v.x * v.y; }, g);
 }
 
 // -------------------------------------------------------------------------------------- thermo
@@ -491,11 +538,11 @@ struct SpOut {
 };
 
 template <class Sc, class MV, class Q>
-__device__ __forceinline__ SpOut<Sc> species_item(const MV& M, int k, Q y, Sc T, Sc lnT, Sc invT,
+__device__ __forceinline__ SpOut<Sc> species_item(const MV& M, int k, double tmid, Q y, Sc T, Sc lnT, Sc invT,
                                                   int tj, double ttau, bool deriv) {
   const double* t = M.sp + k;
   const double iw = __ldg(t);
-  const double* cb = t + (size_t)(4 + (less_pos(val(T), __ldg(t + 2 * M.n)) ? 0 : SP_RANGE)) * M.n;
+  const double* cb = t + (size_t)(4 + (less_pos(val(T), tmid) ? 0 : SP_RANGE)) * M.n;
   auto c = [&](int f) { return __ldg(cb + f * M.n); };
   const Sc a0 = c(0), a1 = c(1), a2 = c(2), a3 = c(3), a4 = c(4);
   SpOut<Sc> o;
@@ -543,9 +590,12 @@ __device__ __forceinline__ ScalT<num<P>> eval_species(const MV& M, P s, const LT
   const P emg = s + L.emg;
   const P cpv = s + L.cpR;
   const P C = s + L.C;
+  double tmid = __ldg(M.sp + 2 * M.n + min(g.lane, M.n - 1));   // the range decides which coefficients to read
 #pragma unroll 1
   for (int k = g.lane; k < M.n; k += g.size) {
-    const SpOut<Sc> a = species_item<Sc>(M, k, y, T, sc.lnT, sc.invT, sc.tj, sc.ttau, deriv);
+    const double tm = tmid;
+    tmid = __ldg(M.sp + 2 * M.n + min(k + g.size, M.n - 1));
+    const SpOut<Sc> a = species_item<Sc>(M, k, tm, y, T, sc.lnT, sc.invT, sc.tj, sc.ttau, deriv);
     if (odd) sig += first + a.yw;
     else first = a.yw;
     odd = !odd;
@@ -621,7 +671,7 @@ __device__ __forceinline__ void rx_simple(const MV& M, int r, const RxIn& in, P 
   if (valid) s[L.q + r] = q;
   if (deriv) {
     const P hRT = s + L.hRT;
-    const int so = __ldg(M.rxi + (size_t)r * RX_I + 13);
+    const int so = (int)(in.i.flags >> 16);
     const Sc dlnkf = sfma(Sc(in.Ta), sc.invT, Sc(in.b)) * sc.invT;
     Sc sh = Sc(hRT[p0]) - Sc(hRT[r0]);
     sh += Sc(hRT[p1]);
@@ -646,6 +696,19 @@ __device__ __forceinline__ void rx_simple(const MV& M, int r, const RxIn& in, P 
   }
 }
 
+// Table records of listed colliders and derivative slots are read in batches (one by one for dual numbers): each read is a trip to L2, and
+// one after the other they took as long as the reaction's exponentials.
+template <class Sc>
+__host__ __device__ constexpr int batch_of() { return is_real<Sc>() ? 4 : 1; }
+__device__ __forceinline__ EffRec ld_rec(const EffRec* p) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  return EffRec{__hiloint2double(v.y, v.x), v.z, 0};
+}
+__device__ __forceinline__ SlotRec ld_rec(const SlotRec* p) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  return SlotRec{__hiloint2double(v.y, v.x), v.z, 0};
+}
+
 // Per-reaction quantities of the rate evaluation that the derivative part needs afterwards.
 template <class Sc>
 struct RxCore {
@@ -654,14 +717,19 @@ struct RxCore {
   int so, scn;
 };
 
-// Rate of progress of reaction r, specialised on the reaction type (0 elementary, 1 third-body,
-// 2 Troe).  Branch-free in the participant counts: absent occurrences read index 0 and count as 1.
-template <class Sc, int TYPE, class P, class MV>
-__device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in, P C, P eg, P emg, P hRT,
+// Rate of progress of reaction r of any type (0 elementary, 1 third-body, 2 Troe).  Branch-free in the participant
+// counts: absent occurrences read index 0 and count as 1.
+template <class Sc, class P, class MV>
+__device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, int type, const RxIn& in, P C, P eg, P emg, P hRT,
                                               const ScalT<Sc>& sc, bool deriv) {
-  const int* I = M.rxi + (size_t)r * RX_I;
-  const double* D = M.rxd + r;
-  auto par = [&](int f) { return __ldg(D + f * M.R); };
+  // everything that is read from the tables is asked for before the first exponential
+  int4 w = make_int4(0, 0, 0, 0);   // efficiency count, slot offset, slot count, efficiency offset
+  if (type != 0 || deriv) w = __ldg(reinterpret_cast<const int4*>(M.rxi + (size_t)r * RX_I) + 3);
+  double par[11];
+  if (type == 2) {
+#pragma unroll
+    for (int f = 3; f < 11; ++f) par[f] = __ldg(M.rxd + r + f * M.R);
+  }
   const int rev = in.i.flags & RXF_REV, nro = (in.i.flags >> 1) & 3, npo = (in.i.flags >> 3) & 3;
   const int r0 = in.i.r01 & 0xffff, r1 = in.i.r01 >> 16, r2 = in.i.r2p0 & 0xffff;
   const int p0 = in.i.r2p0 >> 16, p1 = in.i.p12 & 0xffff, p2 = in.i.p12 >> 16;
@@ -674,34 +742,43 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in
   x.cp0 = C[p0]; x.cp1 = at(C, npo > 1, p1, 1.0); x.cp2 = at(C, npo > 2, p2, 1.0);
   const Sc Pf = x.cr0 * x.cr1 * x.cr2, Pb = x.cp0 * x.cp1 * x.cp2;
   Sc Mv = sc.ctot;
-  if (TYPE != 0) {
-    const int eo = __ldg(I + 11), ec = __ldg(I + 12);
-    for (int i = 0; i < ec; ++i) Mv = sfma(Sc(__ldg(M.eff_am1 + eo + i)), Sc(C[__ldg(M.eff_sp + eo + i)]), Mv);
+  if (type != 0) {
+    constexpr int kBatch = batch_of<Sc>();
+    for (int i = 0; i < w.x; i += kBatch) {   // a batch of listed colliders is read at once
+      EffRec e[kBatch];
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) e[j] = ld_rec(M.eff + w.w + min(i + j, w.x - 1));
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j) {
+        const Sc c = C[e[j].sp];
+        if (i + j < w.x) Mv = sfma(Sc(e[j].am1), c, Mv);
+      }
+    }
   }
   x.dlnkf_dT = Sc(0.0);
   if (deriv) x.dlnkf_dT = sfma(Ta, sc.invT, bb) * sc.invT;
   x.dlnk_dlnM = Sc(0.0);
   x.iM = Sc(0.0);
-  if (TYPE == 2) {
-    const Sc lnk0 = sfma(-Sc(par(5)), sc.invT, sfma(Sc(par(4)), sc.lnT, Sc(par(3))));
+  if (type == 2) {
+    const Sc lnk0 = sfma(-Sc(par[5]), sc.invT, sfma(Sc(par[4]), sc.lnT, Sc(par[3])));
     const Sc lnM = slog(Mv);
     const Sc lnPr = lnk0 - lnkinf + lnM;
     const Sc Pr = sexp(lnPr);
-    const double T2 = par(10);
+    const double T2 = par[10];
     // the Troe centre: tabulated (Troe reactions are the first compiled ones), or from its three
     // exponentials, which the Jacobian's temperature derivative needs in any case
     bool tfc = false;
     if constexpr (is_real<Sc>()) tfc = sc.tj >= 0 && M.tab_deg[3] > 0;
     Sc e3 = Sc(0.0), e1 = Sc(0.0), e2 = Sc(0.0), Fc;
     if (!tfc || deriv) {
-      e3 = sexp(-sc.T * par(8));
-      e1 = sexp(-sc.T * par(9));
+      e3 = sexp(-sc.T * par[8]);
+      e1 = sexp(-sc.T * par[9]);
       e2 = less_pos(0.0, T2) ? sexp(-T2 * sc.invT) : Sc(0.0);
     }
     if constexpr (is_real<Sc>()) {
       if (tfc) Fc = tab_poly(M.tab[3] + ((size_t)sc.tj * M.n_troe + r) * (M.tab_deg[3] + 1), M.tab_deg[3], sc.ttau);
     }
-    if (!tfc) Fc = sfma(Sc(par(6)), e3, sfma(Sc(par(7)), e1, e2));
+    if (!tfc) Fc = sfma(Sc(par[6]), e3, sfma(Sc(par[7]), e1, e2));
     const Sc Lc = slog(Fc) * kInvLn10;
     const Sc cc = sfma(Sc(-0.67), Lc, Sc(-0.4));
     const Sc nn = sfma(Sc(-1.27), Lc, Sc(0.75));
@@ -720,9 +797,9 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in
     const Sc ipr1 = den * S2 * R;
     kf = kf * (Pr * ipr1) * F;
     if (deriv) {
-      const Sc dlnk0_dT = sfma(Sc(par(5)), sc.invT, Sc(par(4))) * sc.invT;
+      const Sc dlnk0_dT = sfma(Sc(par[5]), sc.invT, Sc(par[4])) * sc.invT;
       const Sc dlnPr_dT = dlnk0_dT - x.dlnkf_dT;
-      const Sc dFc_dT = -(par(6) * par(8)) * e3 - (par(7) * par(9)) * e1 +
+      const Sc dFc_dT = -(par[6] * par[8]) * e3 - (par[7] * par[9]) * e1 +
                         T2 * sc.invT * sc.invT * e2;
       const Sc dLc_dT = dFc_dT / Fc * kInvLn10;
       const Sc dx_dT = sfma(dlnPr_dT, Sc(kInvLn10), -0.67 * dLc_dT);
@@ -755,22 +832,18 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, const RxIn& in
   } else {
     x.dlnKc_dT = Sc(0.0);
   }
-  x.Mfac = (TYPE == 1) ? Mv : Sc(1.0);
+  x.Mfac = type == 1 ? Mv : Sc(1.0);
   x.qn = sfma(kf, Pf, -(x.kr * Pb));
   x.q = x.Mfac * x.qn;
-  x.so = 0;
-  x.scn = 0;
-  if (deriv) {
-    x.so = __ldg(I + 13);
-    x.scn = __ldg(I + 14);
-  }
+  x.so = w.y;
+  x.scn = w.z;
   return x;
 }
 
 // Store q (and with deriv: dq/dT at fixed C into s[dq_off + r], and the derivative slots dq/dC_j into
 // s[d_off + slot]) of reaction r.
-template <class Sc, int TYPE, class P, class MV, class LT>
-__device__ __forceinline__ void rx_store(const MV& M, int r, const RxCore<Sc>& x, P s, const LT& L,
+template <class Sc, class P, class MV, class LT>
+__device__ __forceinline__ void rx_store(const MV& M, int r, int type, const RxCore<Sc>& x, P s, const LT& L,
                                          const ScalT<Sc>& sc, bool valid, int dq_off, int d_off, bool deriv) {
   if (!valid) return;
   s[L.q + r] = x.q;
@@ -778,69 +851,69 @@ __device__ __forceinline__ void rx_store(const MV& M, int r, const RxCore<Sc>& x
   const Sc kfM = x.kf * x.Mfac, krM = x.kr * x.Mfac;
   const Sc qf = kfM * x.cr0 * x.cr1 * x.cr2, qr = krM * x.cp0 * x.cp1 * x.cp2;
   Sc dqdM = Sc(0.0);
-  if (TYPE == 1) dqdM = x.qn;
-  if (TYPE == 2) dqdM = x.dlnk_dlnM * x.q * x.iM;
+  if (type == 1) dqdM = x.qn;
+  if (type == 2) dqdM = x.dlnk_dlnM * x.q * x.iM;
   // [M] depends on T through the total concentration p/(Ru T)
   s[dq_off + r] = sfma(x.dlnkf_dT, qf, -((x.dlnkf_dT - x.dlnKc_dT) * qr)) - dqdM * sc.ctot * sc.invT;
   // partial products: d(prod)/d(occurrence i) = product of the other occurrences
   const Sc dr0 = x.cr1 * x.cr2, dr1 = x.cr0 * x.cr2, dr2 = x.cr0 * x.cr1;
   const Sc dp0 = x.cp1 * x.cp2, dp1 = x.cp0 * x.cp2, dp2 = x.cp0 * x.cp1;
   const bool fin = finite_bits(val(kfM)) && finite_bits(val(krM));
-  for (int i = 0; i < x.scn; ++i) {
-    const int mask = __ldg(M.dslot_mask + x.so + i);
-    // elementary reactions list no colliders: their (efficiency - 1) is 0 and so is the [M] term
-    Sc v = TYPE == 0 ? Sc(0.0) : __ldg(M.dslot_am1 + x.so + i) * dqdM;
-    if (mask != 0 || !fin) {   // a participant (a species that only collides has no factor: the [M] term is all)
-      // the slot's factor on a side is the sum over the species' occurrences there, nearly always one: it is
-      // selected, and a second or third one added
-      Sc fr = (mask & 1) ? dr0 : (mask & 2) ? dr1 : (mask & 4) ? dr2 : Sc(0.0);
-      Sc fq = (mask & 8) ? dp0 : (mask & 16) ? dp1 : (mask & 32) ? dp2 : Sc(0.0);
-      if ((mask & 3) == 3 || (mask & 5) == 5 || (mask & 6) == 6) {
-        if ((mask & 3) == 3) fr += dr1;
-        if ((mask & 4) && (mask & 3)) fr += dr2;
+  constexpr int kBatch = batch_of<Sc>();
+  for (int i0 = 0; i0 < x.scn; i0 += kBatch) {
+    SlotRec rec[kBatch];
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) rec[j] = ld_rec(M.dslot + x.so + min(i0 + j, x.scn - 1));
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+      const int i = i0 + j, mask = rec[j].mask;
+      if (i >= x.scn) break;
+      // elementary reactions list no colliders: their (efficiency - 1) is 0 and so is the [M] term
+      Sc v = type == 0 ? Sc(0.0) : rec[j].am1 * dqdM;
+      if (mask != 0 || !fin) {   // a participant (a species that only collides has no factor: the [M] term is all)
+        // the slot's factor on a side is the sum over the species' occurrences there, nearly always one: it is
+        // selected, and a second or third one added
+        Sc fr = (mask & 1) ? dr0 : (mask & 2) ? dr1 : (mask & 4) ? dr2 : Sc(0.0);
+        Sc fq = (mask & 8) ? dp0 : (mask & 16) ? dp1 : (mask & 32) ? dp2 : Sc(0.0);
+        if ((mask & 3) == 3 || (mask & 5) == 5 || (mask & 6) == 6) {
+          if ((mask & 3) == 3) fr += dr1;
+          if ((mask & 4) && (mask & 3)) fr += dr2;
+        }
+        if ((mask & 24) == 24 || (mask & 40) == 40 || (mask & 48) == 48) {
+          if ((mask & 24) == 24) fq += dp1;
+          if ((mask & 32) && (mask & 24)) fq += dp2;
+        }
+        v = sfma(kfM, fr, v);
+        v = sfma(-krM, fq, v);
       }
-      if ((mask & 24) == 24 || (mask & 40) == 40 || (mask & 48) == 48) {
-        if ((mask & 24) == 24) fq += dp1;
-        if ((mask & 32) && (mask & 24)) fq += dp2;
-      }
-      v = sfma(kfM, fr, v);
-      v = sfma(-krM, fq, v);
+      s[d_off + x.so + i] = v;
     }
-    s[d_off + x.so + i] = v;
   }
 }
 
-// Rates of progress of reactions [rb, re).  Reactions are ordered Troe, third-body, elementary, so every
-// segment has warp-uniform control flow; the elementary ones go in rounds of one reaction per lane, and a round
-// whose reactions are all simple takes the short form (every lane of a round's warp takes part: lanes past the
-// end repeat the last reaction and store nothing).
+// Rates of progress of reactions [rb, re), in rounds of one reaction per lane.  A round whose reactions are all
+// simple takes the short form (every lane of a round's warp takes part: lanes past the end repeat the last reaction
+// and store nothing).  The other types stand first (Troe, third-body) and share their rounds: what a Troe or
+// third-body reaction needs beyond an elementary one is a branch that the round takes once.
 template <class Sc, class P, class Gp, class MV, class LT>
 __device__ __forceinline__ void eval_reactions(const MV& M, P s, const LT& L, const ScalT<Sc>& sc,
                                                const Gp& g, int rb, int re, int dq_off, int d_off, bool deriv) {
   const P C = s + L.C, eg = s + L.eg, emg = s + L.emg, hRT = s + L.hRT;
-  const int t1 = min(re, M.n_troe), e0 = M.n_troe + M.n_tb, b1 = min(re, e0);
+  if (rb < re) {
+    RxIn next = ld_rx(M, min(rb + g.lane, re - 1));
 #pragma unroll 1
-  for (int r = rb + g.lane; r < t1; r += g.size)
-    rx_store<Sc, 2>(M, r, rx_core<Sc, 2, P>(M, r, ld_rx(M, r), C, eg, emg, hRT, sc, deriv), s, L, sc, true, dq_off, d_off,
-                     deriv);
-#pragma unroll 1
-  for (int r = max(rb, M.n_troe) + g.lane; r < b1; r += g.size)
-    rx_store<Sc, 1>(M, r, rx_core<Sc, 1, P>(M, r, ld_rx(M, r), C, eg, emg, hRT, sc, deriv), s, L, sc, true, dq_off, d_off,
-                     deriv);
-  const int r0 = max(rb, e0);
-  if (r0 < re) {
-    RxIn next = ld_rx(M, min(r0 + g.lane, re - 1));
-#pragma unroll 1
-    for (int base = r0; base < re; base += g.size) {
+    for (int base = rb; base < re; base += g.size) {
       const int r = min(base + g.lane, re - 1);
       const bool valid = base + g.lane < re;
       const RxIn in = next;
       if (base + g.size < re) next = ld_rx(M, min(base + g.size + g.lane, re - 1));
-      if (wall(g, (in.i.flags & RXF_SIMPLE) != 0))
+      if (wall(g, (in.i.flags & RXF_SIMPLE) != 0)) {
         rx_simple<Sc>(M, r, in, s, L, sc, valid, dq_off, d_off, deriv);
-      else
-        rx_store<Sc, 0>(M, r, rx_core<Sc, 0, P>(M, r, in, C, eg, emg, hRT, sc, deriv), s, L, sc, valid, dq_off, d_off,
-                     deriv);
+      } else {
+        const int type = r < M.n_troe ? 2 : r < M.n_troe + M.n_tb ? 1 : 0;
+        rx_store<Sc>(M, r, type, rx_core<Sc, P>(M, r, type, in, C, eg, emg, hRT, sc, deriv), s, L, sc, valid, dq_off,
+                     d_off, deriv);
+      }
     }
   }
   g.sync();
@@ -856,7 +929,8 @@ __device__ __forceinline__ ScalT<num<P>> eval_rates(const MV& M, P s, const LT& 
                                                     bool deriv) {
   using Sc = num<P>;
   const ScalT<Sc> sc = eval_species(M, s, L, y, p, g, deriv);
-  const P S = s + L.S, part = s + L.part;
+  const P S = s + L.S;
+  const auto sp = prog_ptr(s);
   if (deriv)
     for (int e = g.lane; e < M.nY + M.n; e += g.size) S[e] = Sc(0.0);
   const int passes = deriv ? M.n_jpass : 1;
@@ -865,9 +939,10 @@ __device__ __forceinline__ ScalT<num<P>> eval_rates(const MV& M, P s, const LT& 
     const int rb = deriv ? M.jpass[ps][JP_RB] : 0, re = deriv ? M.jpass[ps][JP_RE] : M.R;
     const int cnt = M.jpass[ps][JP_CNT];
     eval_reactions<Sc>(M, s, L, sc, g, rb, re, L.D - rb, L.D + cnt - M.jpass[ps][JP_SB], deriv);
-    if (deriv) gather_nu(M.g_jac[ps], S, part, s + L.D, g, ps > 0);
+    if (deriv && ps == 0) gather_nu<false>(M.g_jac[0], sp + L.S, sp + L.part, sp + L.D, g);
+    if (deriv && ps > 0) gather_nu<true>(M.g_jac[ps], sp + L.S, sp + L.part, sp + L.D, g);
   }
-  gather_nu(M.g_omega, w, part, s + L.q, g);
+  gather_nu<false>(M.g_omega, prog_ptr(w), sp + L.part, sp + L.q, g);
   return sc;
 }
 
@@ -900,8 +975,9 @@ template <class Sc, class P, class Gp, class MV, class LT>
 __device__ __forceinline__ void finish_jac(const MV& M, P s, const LT& L, const ScalT<Sc>& sc, const Gp& g) {
   const P w = s + L.x, gk = s + L.U1, tk = s + L.U2, S = s + L.S, wT = s + (L.S + M.nY);
   const P C = s + L.C, hRT = s + L.hRT;
-  gather_xy(M.g_row, gk, s + L.part, S, C, g);
-  gather_xy(M.g_col, tk, s + L.part, S, hRT, g);
+  const auto sp = prog_ptr(s);
+  gather_xy(M.g_row, sp + L.U1, sp + L.part, sp + L.S, sp + L.C, g);
+  gather_xy(M.g_col, sp + L.U2, sp + L.part, sp + L.S, sp + L.hRT, g);
   const P f = s + L.f0, u = s + L.u, v = s + L.v;
   const Sc T = sc.T;
   // f, u and the T column; partial sums for the T row scalars
@@ -936,6 +1012,7 @@ __device__ __forceinline__ void finish_jac(const MV& M, P s, const LT& L, const 
   }
   g.sync();
   // species block: S_kj = (W_k / W_j) Dtil_kj (after the row and column sums used Dtil)
+#pragma unroll 8
   for (int e = g.lane; e < M.nY; e += g.size) S[e] *= __ldg(M.entry_wratio + e);
   g.sync();
 }
@@ -956,6 +1033,7 @@ __device__ __forceinline__ bool lu_build_factor(const MV& M, SPtr s, const LT& L
                                                 const Gp& g) {
   const SPtr LU = s + L.LU;   // followed by the negated reciprocal pivots (L.dinv)
   const SPtr S = s + L.S;
+#pragma unroll 8
   for (int l = g.lane; l < M.nnz_LU; l += g.size) {
     const int src = __ldg(M.lu_src + l);
     const double v = S[max(src, 0)];

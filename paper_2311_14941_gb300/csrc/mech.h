@@ -52,14 +52,25 @@ constexpr int RX_D = 12;
 //   [0] type (0 elementary, 1 third-body, 2 Troe)  [1] reversible  [2] reactant occurrences (1..3)
 //   [3] product occurrences (1..3)  [4..6] reactant species per occurrence (coefficient nu expands into
 //   nu occurrences)  [7..9] product occurrences  [10] sum of net coefficients  [11] efficiency offset
-//   [12] efficiency count  [13] derivative-slot offset  [14] derivative-slot count  [15] unused
+//   [12] efficiency count  [13] derivative-slot offset  [14] derivative-slot count  [15] efficiency offset again
+//   ([12..15] are read as one 16-byte word)
 constexpr int RX_I = 16;
 // one 16-byte record per reaction with what the rate of progress needs: six 16-bit species indices (reactant,
 // then product occurrences; absent ones are 0) and the flags below
 struct alignas(16) RxRec {
   uint32_t r01, r2p0, p12, flags;   // r0 | r1 << 16, r2 | p0 << 16, p1 | p2 << 16
 };
-// flags: bit 0 reversible, bits 1-2 reactant occurrences, bits 3-4 product occurrences, bit 5 simple
+// a listed efficiency (species and efficiency - 1), and a derivative slot: its species' (efficiency - 1), 0 if not
+// listed, and the occurrences that are this species (bits 0..2 reactants, 3..5 products)
+struct alignas(16) EffRec {
+  double am1;
+  int sp, pad;
+};
+struct alignas(16) SlotRec {
+  double am1;
+  int mask, pad;
+};
+// flags (bits 16-31: derivative-slot offset): bit 0 reversible, bits 1-2 reactant occurrences, bits 3-4 product occurrences, bit 5 simple
 // (elementary, reversible, two reactants and two products, all four different species), bit 6: a species
 // occurs more than once on one side
 enum : int { RXF_REV = 1, RXF_SIMPLE = 32, RXF_REP = 64 };
@@ -71,8 +82,10 @@ constexpr int kProgBlock = 8;
 //   acc = fma(value(a, b), acc); if dst != NONE: out[dst] = acc, acc = 0.  Padded to whole blocks of steps.
 // dst >= PARTIAL_BIT selects the partial-sum buffer; a combine list then adds partials into outputs.
 struct GatherOp {
-  uint16_t a, b, dst, flags;   // flags bit 0: padding (no accumulation)
+  uint16_t a, b, dst, flags;
 };
+// flags: padding (no accumulation); in every lane's op of a step in which some lane ends a piece
+enum : int { GF_IDLE = 1, GF_END = 2 };
 constexpr uint16_t DST_NONE = 0xFFFF;
 constexpr uint16_t PARTIAL_BIT = 0x8000;
 
@@ -128,11 +141,8 @@ struct MechView {
   const double* rxd;         // [RX_D * R]
   const int* rxi;            // [R * RX_I]
   const RxRec* rxr;          // [R]
-  const int* eff_sp;         // listed efficiencies
-  const double* eff_am1;     // alpha - 1
-  const int* dslot_sp;       // [n_dslot] column species of each derivative slot
-  const int* dslot_mask;     // [n_dslot] bits 0..2 reactant occurrences, 3..5 product occurrences equal
-  const double* dslot_am1;   // [n_dslot] (efficiency - 1) of the slot species, 0 if not listed
+  const EffRec* eff;         // listed efficiencies
+  const SlotRec* dslot;      // [n_dslot]
   const int* entry_row;      // [nY] species k of Y-block entry
   const int* entry_col;      // [nY] species j
   const double* entry_wratio;// [nY] W_k / W_j

@@ -84,7 +84,7 @@ constexpr const char* kKernelExpr[2] = {
     "chemgb::k_integrate_persistent<chemgb::Grp1, chemgb::SpecView, chemgb::SpecLayout>"};
 constexpr const char* kKernelTag[2] = {"plain", "persistent"};
 // The library's own integration kernels are built with the same register cap.
-constexpr const char* kOptions[] = {"--gpu-architecture=sm_103a", "-std=c++17", "-maxrregcount=168"};
+constexpr const char* kOptions[] = {"--gpu-architecture=sm_103a", "-std=c++17", "-maxrregcount=224"};
 constexpr int kNumOptions = sizeof(kOptions) / sizeof(kOptions[0]);
 
 uint64_t fnv1a(uint64_t h, const std::string& s) {
