@@ -20,12 +20,10 @@ LIB = os.path.join(OUT, "libchemgb.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 # kernel translation units besides capi.cu: the integration kernels per lane group, and the adjoint
-# Registers per thread of the integration kernels: with one or two warps per cell as many as they ask for (185;
-# shared memory allows nine warps per SM at 53 species, which 224 registers allow too).  Held to 168 or 128, the
-# programs' ops that are read ahead spill: a 4,096-cell jet field took 320 and 370 ms instead of 300.  Two cells
-# per warp are for small mechanisms, which need the 12 warps per SM of 168.
-REG_CAP = {"kern_fwd_warp": ["-maxrregcount=224"], "kern_fwd_warp_plain": ["-maxrregcount=224"],
-           "kern_fwd_pair": ["-maxrregcount=224"], "kern_fwd_half": ["-maxrregcount=168"]}
+# Registers per thread of the integration kernels: as many as they ask for (about 200; nine warps per SM, which
+# is what shared memory allows at 53 species).  Held to 168 or 128, the programs' ops that are read ahead spill: a
+# 4,096-cell jet field took 320 and 370 ms instead of 300, 6,000 small cells 371 (at 168) instead of 351.
+REG_CAP = {f: ["-maxrregcount=224"] for f in ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd_half")}
 CUDA_UNITS = ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd_half", "kern_rates",
               "kern_adjoint")
 HOST_UNITS = ("compile", "balance", "specialize")

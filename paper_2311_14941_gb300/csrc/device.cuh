@@ -55,16 +55,34 @@ struct GrpW<2> {
 using Grp1 = GrpW<1>;
 using Grp2 = GrpW<2>;
 
-// Half a warp: two cells share a warp, 16 lanes each (mechanisms with few species, whose loops and
-// sparse programs leave most of a warp's lanes idle).  Shared-memory ordering is a warp barrier over the
-// group's own lanes, and reductions are butterflies within them, so the two cells of a warp may also
-// run apart (different step sequences) without waiting for each other.
-struct GrpH {
+// Half a warp: two cells share a warp, 16 lanes each (mechanisms with few species, whose loops and sparse programs
+// leave most of a warp's lanes idle).  The two cells take every attempt together (see cell_step): an FP64
+// instruction takes the pipe for 64 cycles however many lanes it has, so run apart they would pay for each other
+// (6,000 cells of 10 species / 27 reactions: 368 ms apart, 346 together).
+// GrpH is such a half inside an attempt: the whole warp takes part in every barrier and vote.  GrpHs is the half by
+// itself (starting and finishing its cell).
+struct GrpHs {
   static constexpr int size = kWarp / 2;
   int lane;        // 0 .. 15
   unsigned mask;   // the lanes of this half of the warp
   __device__ __forceinline__ void sync() const { __syncwarp(mask); }
 };
+struct GrpH {
+  static constexpr int size = kWarp / 2;
+  int lane;        // 0 .. 15
+  unsigned mask;   // the lanes of this half of the warp
+  __device__ __forceinline__ void sync() const { __syncwarp(); }
+};
+__device__ __forceinline__ const Grp1& solo(const Grp1& g) { return g; }
+__device__ __forceinline__ const Grp2& solo(const Grp2& g) { return g; }
+__device__ __forceinline__ GrpHs solo(const GrpH& g) { return GrpHs{g.lane, g.mask}; }
+// Whether ok holds for one, for all of the cells of this warp (every lane of a cell passes the same value).
+__device__ __forceinline__ bool any_cell(const Grp1&, bool ok) { return ok; }
+__device__ __forceinline__ bool any_cell(const Grp2&, bool ok) { return ok; }
+__device__ __forceinline__ bool any_cell(const GrpH&, bool ok) { return __any_sync(0xffffffffu, ok); }
+__device__ __forceinline__ bool all_cells(const Grp1&, bool ok) { return ok; }
+__device__ __forceinline__ bool all_cells(const Grp2&, bool ok) { return ok; }
+__device__ __forceinline__ bool all_cells(const GrpH&, bool ok) { return __all_sync(0xffffffffu, ok); }
 
 // Ordering among the lanes of half a group (both halves run the same steps, so a barrier of the whole warp will do;
 // the halves of two warps are the warps themselves).
@@ -74,12 +92,17 @@ struct SyncMask {
 };
 __device__ __forceinline__ SyncMask half_sync(const Grp1&) { return SyncMask{0xffffffffu}; }
 __device__ __forceinline__ SyncMask half_sync(const Grp2&) { return SyncMask{0xffffffffu}; }
-__device__ __forceinline__ SyncMask half_sync(const GrpH& g) { return SyncMask{g.mask}; }
+__device__ __forceinline__ SyncMask half_sync(const GrpH&) { return SyncMask{0xffffffffu}; }
 
 __device__ __forceinline__ double gsum(const Grp1&, double v) { return warp_sum(v); }
-__device__ __forceinline__ double gsum(const GrpH& g, double v) {
+__device__ __forceinline__ double gsum(const GrpH&, double v) {   // exchanges stay within the half
 #pragma unroll
-  for (int o = GrpH::size / 2; o > 0; o >>= 1) v += __shfl_xor_sync(g.mask, v, o);
+  for (int o = GrpH::size / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double gsum(const GrpHs& g, double v) {
+#pragma unroll
+  for (int o = GrpHs::size / 2; o > 0; o >>= 1) v += __shfl_xor_sync(g.mask, v, o);
   return v;
 }
 __device__ __forceinline__ double gsum(const Grp2& g, double v) {
@@ -125,12 +148,12 @@ __device__ __forceinline__ void bfly3(unsigned mask, int lane, double& a, double
   c = __shfl_sync(mask, v, W / 4, W);
 }
 __device__ __forceinline__ void gsum2(const Grp1& g, double& a, double& b) { bfly2<kWarp>(0xffffffffu, g.lane, a, b); }
-__device__ __forceinline__ void gsum2(const GrpH& g, double& a, double& b) { bfly2<GrpH::size>(g.mask, g.lane, a, b); }
+__device__ __forceinline__ void gsum2(const GrpH& g, double& a, double& b) { bfly2<GrpH::size>(0xffffffffu, g.lane, a, b); }
 __device__ __forceinline__ void gsum3(const Grp1& g, double& a, double& b, double& c) {
   bfly3<kWarp>(0xffffffffu, g.lane, a, b, c);
 }
 __device__ __forceinline__ void gsum3(const GrpH& g, double& a, double& b, double& c) {
-  bfly3<GrpH::size>(g.mask, g.lane, a, b, c);
+  bfly3<GrpH::size>(0xffffffffu, g.lane, a, b, c);
 }
 __device__ __forceinline__ void gsum2(const Grp2& g, double& a, double& b) {
   bfly2<kWarp>(0xffffffffu, g.lane & (kWarp - 1), a, b);
@@ -157,7 +180,8 @@ template <class G, class Sc>
 __device__ __forceinline__ void gsum3(const G& g, Sc& a, Sc& b, Sc& c) { a = gsum(g, a); b = gsum(g, b); c = gsum(g, c); }
 
 __device__ __forceinline__ bool gall(const Grp1&, bool ok) { return __all_sync(0xffffffffu, ok); }
-__device__ __forceinline__ bool gall(const GrpH& g, bool ok) { return __all_sync(g.mask, ok); }
+__device__ __forceinline__ bool gall(const GrpHs& g, bool ok) { return __all_sync(g.mask, ok); }
+__device__ __forceinline__ bool gall(const GrpH& g, bool ok) { return (__ballot_sync(0xffffffffu, ok) & g.mask) == g.mask; }
 __device__ __forceinline__ bool gall(const Grp2& g, bool ok) {
   ok = __all_sync(0xffffffffu, ok);
   g.sync();
@@ -168,12 +192,12 @@ __device__ __forceinline__ bool gall(const Grp2& g, bool ok) {
 
 // Whether ok holds on all lanes of the group that share this thread's warp (all of them call it).
 __device__ __forceinline__ bool wall(const Grp1&, bool ok) { return __all_sync(0xffffffffu, ok); }
-__device__ __forceinline__ bool wall(const GrpH& g, bool ok) { return __all_sync(g.mask, ok); }
+__device__ __forceinline__ bool wall(const GrpH&, bool ok) { return __all_sync(0xffffffffu, ok); }
 __device__ __forceinline__ bool wall(const Grp2&, bool ok) { return __all_sync(0xffffffffu, ok); }
 
 // The value of lane 0, on every lane of the group.
 __device__ __forceinline__ long long gbcast(const Grp1&, long long v) { return __shfl_sync(0xffffffffu, v, 0); }
-__device__ __forceinline__ long long gbcast(const GrpH& g, long long v) { return __shfl_sync(g.mask, v, 0, GrpH::size); }
+__device__ __forceinline__ long long gbcast(const GrpHs& g, long long v) { return __shfl_sync(g.mask, v, 0, GrpHs::size); }
 __device__ __forceinline__ long long gbcast(const Grp2& g, long long v) {
   g.sync();
   if (g.lane == 0) g.xch[0] = __longlong_as_double(v);
@@ -1099,6 +1123,7 @@ __device__ __forceinline__ StepOut ros_attempt(const MV& M, double* sd, const LT
   auto U = [&](int j) { return j < 4 ? U1 + j * (L.U2 - L.U1) : s + L.x; };
   const int stages = method == 0 ? 4 : method == 1 ? 2 : 6;
   double iden = 0.0;
+  bool fine = true;   // (the other cell of the warp goes on when this one has failed)
 #pragma unroll 1
   for (int k = 0; k < stages; ++k) {   // stage k + 1
     const SPtr out = k == 0 ? s + (L.x - 1) : k < 5 ? U(k) : U2;   // stage 1: the production rates go to x
@@ -1130,7 +1155,8 @@ __device__ __forceinline__ StepOut ros_attempt(const MV& M, double* sd, const LT
       else finish_f(M, sd, L, sc, to, g);
     }
     if (k == 0) {
-      if (!lu_build_factor(M, s, L, ih * (method == 1 ? 1.0 / RG2 : method == 2 ? 1.0 / RG4 : 1.0 / RG), g)) return so;
+      fine = lu_build_factor(M, s, L, ih * (method == 1 ? 1.0 / RG2 : method == 2 ? 1.0 / RG4 : 1.0 / RG), g);
+      if (!any_cell(g, fine)) return so;
       // z = A^-1 u (the Sherman-Morrison vector) and stage 1's A^-1 f0 together, then stage 1's correction
       for (int i = g.lane; i < m; i += g.size) { z[i] = u[i]; U1[i] = f0[i]; }
       g.sync();
@@ -1139,7 +1165,8 @@ __device__ __forceinline__ StepOut ros_attempt(const MV& M, double* sd, const LT
       for (int i = g.lane; i < m; i += g.size) { vz = fma(v[i], z[i], vz); vx = fma(v[i], U1[i], vx); }
       gsum2(g, vz, vx);
       const double den = 1.0 - vz;
-      if ((__double_as_longlong(den) << 1) == 0 || !finite_bits(den)) return so;
+      fine = fine && (__double_as_longlong(den) << 1) != 0 && finite_bits(den);
+      if (!any_cell(g, fine)) return so;
       iden = rcp_rn(den);
       vx *= iden;
       for (int i = g.lane; i < m; i += g.size) U1[i] = fma(z[i], vx, U1[i]);
@@ -1193,7 +1220,7 @@ __device__ __forceinline__ StepOut ros_attempt(const MV& M, double* sd, const LT
   fin = gall(g, fin);
   g.sync();
   so.err = sqrt(div_rn(e2, (double)m));
-  so.good = fin;
+  so.good = fine && fin;
   return so;
 }
 
@@ -1220,13 +1247,21 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// Adaptive integration of the cell whose state sits in y (shared memory) over [0, dt].
-template <class Gp, class MV, class LT>
-__device__ __forceinline__ void integrate_cell(const MV& M, double* sd, const LT& L, double p, double dt,
-                                               double& h_io, int& nsub, int& nacc, int& status, const IntOpts& o,
-                                               const Gp& g, int cell) {
-  const SPtr s = shared_ptr(sd), y = s + L.y;
-  const int m = M.m;
+// A cell between two attempts.
+struct CellRun {
+  int cell = -1;   // -1: none
+  bool active = false, rejected_last = false, need_jac = true;
+  int nonfinite = 0, ns = 0, na = 0, status = kCellOk;
+  double p = 1e5, t = 0.0, dt = 0.0, h = 1.0;
+};
+
+// Start the cell whose state sits in y (shared memory); h_io: its proposed first step.
+template <class Gs, class MV, class LT>
+__device__ __forceinline__ void cell_start(const MV& M, double* sd, const LT& L, int cell, double p, double dt,
+                                           double h_io, const IntOpts& o, const Gs& g, CellRun& r) {
+  const SPtr y = shared_ptr(sd) + L.y;
+  r = CellRun();
+  r.cell = cell;
   // input check
   const double T0 = y[0];
   bool ok = isfinite(p) && p > 0.0 && isfinite(dt) && dt >= 0.0 && isfinite(T0) && T0 > 0.0;
@@ -1238,70 +1273,96 @@ __device__ __forceinline__ void integrate_cell(const MV& M, double* sd, const LT
   }
   sig = gsum(g, sig);
   ok = gall(g, ok) && sig > 0.0;
-  nsub = 0;
-  nacc = 0;
+  r.h = h_io;
   if (!ok) {
-    status = kCellBadInput;
+    r.status = kCellBadInput;
     if (o.rec_h && g.lane == 0) o.rec_n[cell] = -1;
     return;
   }
-  double h = (h_io > 0.0 && isfinite(h_io)) ? h_io : o.h_init;
-  if (dt > 0.0) h = fmin(h, dt);
-  const double dt_end = dt * (1.0 - 1e-14);
-  double t = 0.0;
-  bool rejected_last = false, needJ = true;
-  int nonfinite = 0, ns = 0, na = 0, st = kCellOk;
+  r.p = p;
+  r.dt = dt;
+  r.h = (h_io > 0.0 && isfinite(h_io)) ? h_io : o.h_init;
+  if (dt > 0.0) r.h = fmin(r.h, dt);
   if (o.rec_h)
-    for (int i = g.lane; i < m; i += g.size) o.rec_ck[(size_t)i * o.N + cell] = y[i];
-  while (less_pos(t, dt)) {
-    if (ns >= o.max_substeps) { st = kCellMaxSteps; break; }
-    if (o.deadline_ns) {
-      const unsigned long long now = (unsigned long long)gbcast(g, g.lane == 0 ? (long long)global_ns() : 0ll);
-      if (now > o.deadline_ns) { st = kCellTimeout; break; }
+    for (int i = g.lane; i < M.m; i += g.size) o.rec_ck[(size_t)i * o.N + cell] = y[i];
+  r.active = less_pos(r.t, dt);
+}
+
+// One attempt of every active cell of the warp (of this group's cell): the groups of a warp stay together.  r.active
+// falls when the cell has reached its dt or ends with another status.
+template <class Gp, class MV, class LT>
+__device__ __forceinline__ void cell_step(const MV& M, double* sd, const LT& L, const IntOpts& o, const Gp& g,
+                                          CellRun& r) {
+  const SPtr s = shared_ptr(sd), y = s + L.y;
+  const int m = M.m;
+  bool last = false;
+  double hu = r.h;
+  if (r.active) {
+    last = !less_pos(r.t + r.h, r.dt * (1.0 - 1e-14));
+    hu = last ? r.dt - r.t : r.h;
+    int st = kCellOk;
+    if (r.ns >= o.max_substeps) {
+      st = kCellMaxSteps;
+    } else if (o.deadline_ns) {
+      const auto gs = solo(g);
+      const unsigned long long now = (unsigned long long)gbcast(gs, gs.lane == 0 ? (long long)global_ns() : 0ll);
+      if (now > o.deadline_ns) st = kCellTimeout;
     }
-    const bool last = !less_pos(t + h, dt_end);
-    const double hu = last ? dt - t : h;
-    if (less_pos(hu, o.h_min)) { st = kCellHmin; break; }
-    ++ns;
-    const StepOut so = ros_attempt(M, sd, L, p, hu, o.rtol, o.atol, g, o.method, needJ);
-    needJ = false;
-    if (o.trace && g.lane == 0 && ns <= o.trace_cap)
-      o.trace[(size_t)(ns - 1) * o.N + cell] = (so.good && finite_bits(so.err) && leq_pos(so.err, 1.0)) ? hu : -hu;
-    if (!so.good || !finite_bits(so.err)) {
-      if (++nonfinite >= o.max_nonfinite) { st = kCellNonfinite; break; }
-      h = hu * 0.1;
-      rejected_last = true;
-      continue;
-    }
-    nonfinite = 0;
-    // step-size factor: err^(-1/(embedded order + 1)): 3 for RODAS3, 2 for ROS2, 4 for RODAS4
-    const double fac =
-        max_pos(0.2, 0.9 * pow(so.err, o.method == 1 ? -0.5 : o.method == 2 ? -0.25 : -1.0 / 3.0));
-    if (leq_pos(so.err, 1.0)) {
-      t = last ? dt : t + hu;
-      ++na;
-      const SPtr yt = s + L.ytmp;
-      for (int i = g.lane; i < m; i += g.size) y[i] = yt[i];
-      g.sync();
-      if (o.rec_h && na <= o.rec_cap) {
-        if (g.lane == 0) o.rec_h[(size_t)(na - 1) * o.N + cell] = hu;
-        if (na % o.rec_K == 0)
-          for (int i = g.lane; i < m; i += g.size) o.rec_ck[((size_t)(na / o.rec_K) * m + i) * o.N + cell] = y[i];
-      }
-      h = hu * min_pos(rejected_last ? 1.0 : 6.0, fac);
-      rejected_last = false;
-      needJ = true;
-    } else {
-      h = hu * min_pos(1.0, fac);
-      rejected_last = true;
+    if (st == kCellOk && less_pos(hu, o.h_min)) st = kCellHmin;
+    if (st != kCellOk) {
+      r.status = st;
+      r.active = false;
     }
   }
-  if (o.trace && g.lane == 0 && ns < o.trace_cap) o.trace[(size_t)ns * o.N + cell] = 0.0;
-  if (o.rec_h && g.lane == 0) o.rec_n[cell] = (na <= o.rec_cap && st == kCellOk) ? na : -1;
-  h_io = h;
-  nsub = ns;
-  nacc = na;
-  status = st;
+  if (!any_cell(g, r.active)) return;
+  const StepOut so = ros_attempt(M, sd, L, r.p, hu, o.rtol, o.atol, g, o.method, any_cell(g, r.active && r.need_jac));
+  bool accepted = false;
+  if (r.active) {
+    ++r.ns;
+    r.need_jac = false;
+    const bool numbers = so.good && finite_bits(so.err);
+    accepted = numbers && leq_pos(so.err, 1.0);
+    if (o.trace && g.lane == 0 && r.ns <= o.trace_cap)
+      o.trace[(size_t)(r.ns - 1) * o.N + r.cell] = accepted ? hu : -hu;
+    if (!numbers) {
+      if (++r.nonfinite >= o.max_nonfinite) {
+        r.status = kCellNonfinite;
+        r.active = false;
+      } else {
+        r.h = hu * 0.1;
+        r.rejected_last = true;
+      }
+    } else {
+      r.nonfinite = 0;
+      // step-size factor: err^(-1/(embedded order + 1)): 3 for RODAS3, 2 for ROS2, 4 for RODAS4
+      const double fac =
+          max_pos(0.2, 0.9 * pow(so.err, o.method == 1 ? -0.5 : o.method == 2 ? -0.25 : -1.0 / 3.0));
+      r.h = hu * min_pos(accepted && !r.rejected_last ? 6.0 : 1.0, fac);
+      r.rejected_last = !accepted;
+      if (accepted) {
+        r.t = last ? r.dt : r.t + hu;
+        ++r.na;
+        r.need_jac = true;
+        r.active = less_pos(r.t, r.dt);
+        const SPtr yt = s + L.ytmp;
+        for (int i = g.lane; i < m; i += g.size) y[i] = yt[i];
+      }
+    }
+  }
+  g.sync();
+  if (accepted && o.rec_h && r.na <= o.rec_cap) {
+    if (g.lane == 0) o.rec_h[(size_t)(r.na - 1) * o.N + r.cell] = hu;
+    if (r.na % o.rec_K == 0)
+      for (int i = g.lane; i < m; i += g.size) o.rec_ck[((size_t)(r.na / o.rec_K) * m + i) * o.N + r.cell] = y[i];
+  }
+}
+
+// What is left to record of a cell that has ended.
+template <class Gs>
+__device__ __forceinline__ void cell_end(const IntOpts& o, const Gs& g, const CellRun& r) {
+  if (g.lane != 0) return;
+  if (o.trace && r.status != kCellBadInput && r.ns < o.trace_cap) o.trace[(size_t)r.ns * o.N + r.cell] = 0.0;
+  if (o.rec_h && r.status != kCellBadInput) o.rec_n[r.cell] = (r.na <= o.rec_cap && r.status == kCellOk) ? r.na : -1;
 }
 
 }  // namespace chemgb

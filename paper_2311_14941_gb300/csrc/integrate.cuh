@@ -51,18 +51,6 @@ __device__ __forceinline__ Gp cell_group(const LT& L, double* smem, int& cell_in
   return make_group(static_cast<const Gp*>(nullptr), L, smem, cell_in_block, s);
 }
 
-// Cells taken per queue pull: a half-warp group pulls together with the other half of its warp (one
-// atomic per warp, the two halves take consecutive slots of the sorted queue, so the two cells that
-// share a warp have similar previous costs and run side by side); other groups pull alone.
-template <class Gp>
-struct PullOf {
-  static constexpr int groups = 1;   // lane groups per pulling unit
-};
-template <>
-struct PullOf<GrpH> {
-  static constexpr int groups = 2;
-};
-
 // Block-cooperative coalesced load of the block's consecutive cells: adjacent threads read adjacent
 // cells of the same state row (structure of arrays), then each lane group owns its cell's copy.
 template <class LT>
@@ -75,6 +63,31 @@ __device__ __forceinline__ void load_tile(double* smem, const LT& L, int m, int 
     if (c < N) smem[(size_t)w * L.total + L.y + row] = (row == 0) ? T[c] : Y[(size_t)(row - 1) * N + c];
   }
   __syncthreads();
+}
+
+// Write a cell that has ended back to global memory.
+template <class Gs, class MV, class LT>
+__device__ __forceinline__ void store_cell(const MV& M, double* s, const LT& L, int N, const Gs& g, const CellRun& r,
+                                           double* T, double* Y, double* h_io, int* nsub, int* status, int* nacc_out) {
+  const SPtr y = shared_ptr(s) + L.y;
+  const int c = r.cell;
+  for (int i = g.lane; i < M.m; i += g.size) {
+    if (i == 0) T[c] = y[0];
+    else Y[(size_t)(i - 1) * N + c] = y[i];
+  }
+  if (g.lane == 0) {
+    h_io[c] = r.h;
+    nsub[c] = r.ns;
+    status[c] = r.status;
+    if (nacc_out) nacc_out[c] = r.na;
+  }
+}
+
+// A state for a group that has no cell but shares its warp with one that has: the attempts it takes along must not
+// meet infinities and NaN, whose handling is slow.
+template <class Gp, class LT>
+__device__ __forceinline__ void idle_state(double* s, const LT& L, int m, const Gp& g) {
+  for (int i = g.lane; i < m; i += g.size) s[L.y + i] = i == 0 ? 1000.0 : 1.0 / (m - 1);
 }
 
 // Plain form: one lane group per cell, cells in index order, one launch.
@@ -92,37 +105,25 @@ __global__ void k_integrate_plain(MV M, LT L, int N, double* __restrict__ T, con
   const int c0 = blockIdx.x * cpb;
   load_tile(smem, L, M.m, N, c0, cpb, T, Y);
   const int c = c0 + w;
-  if (c >= N) return;
-  double h = h_io[c];
-  int ns = 0, na = 0, st = 0;
-  integrate_cell(M, s, L, p[c], dt[c], h, ns, na, st, with_deadline(o, stamp, budget_ns), g, c);
-  const SPtr y = shared_ptr(s) + L.y;
-  for (int i = g.lane; i < M.m; i += g.size) {
-    if (i == 0) T[c] = y[0];
-    else Y[(size_t)(i - 1) * N + c] = y[i];
-  }
-  if (g.lane == 0) {
-    h_io[c] = h;
-    nsub[c] = ns;
-    status[c] = st;
-    if (nacc_out) nacc_out[c] = na;
+  const IntOpts oo = with_deadline(o, stamp, budget_ns);
+  CellRun r;
+  if (c < N) cell_start(M, s, L, c, p[c], dt[c], h_io[c], oo, solo(g), r);
+  else idle_state(s, L, M.m, g);
+  g.sync();
+  while (any_cell(g, r.active)) cell_step(M, s, L, oo, g, r);
+  if (c < N) {
+    cell_end(oo, g, r);
+    store_cell(M, s, L, N, g, r, T, Y, h_io, nsub, status, nacc_out);
   }
 }
 
-// Persistent form: grid sized to the resident capacity; every lane group (every warp of two half-warp
-// groups) pulls `chunk` cells per group at a time from the sorted queue with one atomicAdd and
-// integrates them one after the other.  No block-wide barrier: warps of a block finish independently.
-template <class Gp>
-__device__ __forceinline__ long long queue_pull(const Gp& g, unsigned long long* head, int chunk) {
+// Persistent form: grid sized to the resident capacity; every lane group pulls `chunk` cells at a time from the
+// sorted queue with one atomicAdd and integrates them one after the other.  No block-wide barrier: warps of a
+// block finish independently; groups that share a warp take their attempts together and pull whenever they have
+// ended a cell.
+template <class Gs>
+__device__ __forceinline__ long long queue_pull(const Gs& g, unsigned long long* head, int chunk) {
   return gbcast(g, g.lane == 0 ? (long long)atomicAdd(head, (unsigned long long)chunk) : 0ll);
-}
-__device__ __forceinline__ long long queue_pull(const GrpH& g, unsigned long long* head, int chunk) {
-  // one pull for the warp; the upper half takes the second `chunk` cells
-  const unsigned lane = threadIdx.x & (kWarp - 1);
-  long long b = 0;
-  if (lane == 0) b = (long long)atomicAdd(head, 2ull * (unsigned long long)chunk);
-  b = __shfl_sync(0xffffffffu, b, 0);
-  return b + (lane >= (unsigned)GrpH::size ? chunk : 0);
 }
 
 template <class Gp, class MV = MechView, class LT = CellLayout>
@@ -138,34 +139,37 @@ __global__ void k_integrate_persistent(MV M, LT L, int N, double* __restrict__ T
   double* s = nullptr;
   const Gp g = cell_group<Gp>(L, smem, w, s);
   const IntOpts oo = with_deadline(o, stamp, budget_ns);
+  if (Gp::size < kWarp) idle_state(s, L, M.m, g);
+  CellRun r;
+  // 64-bit queue head: every pull adds `chunk`, including the last pulls past the end, so a 32-bit head could
+  // wrap for large N * lane groups * chunk
+  long long next = 0, end = 0;
+  bool more = true;
   while (true) {
-    // 64-bit queue head: every pull adds `chunk` per group, including the last pulls past the end, so a
-    // 32-bit head could wrap for large N * lane groups * chunk.  The half-warp pull is warp-wide: both
-    // halves leave the loop together (the first half's base decides), and a half whose share starts
-    // past the end integrates nothing in that round.
-    const long long base = queue_pull(g, head, chunk);
-    const long long base0 = PullOf<Gp>::groups == 2 ? base - ((threadIdx.x & (kWarp - 1)) >= GrpH::size ? chunk : 0)
-                                                    : base;
-    if (base0 >= N) break;
-    const int end = (int)min(base + (long long)chunk, (long long)N);
-    for (int j = (int)min(base, (long long)N); j < end; ++j) {
-      const int c = perm[j];
-      load_state(s + L.y, M.m, N, c, T, Y, g);
-      double h = h_io[c];
-      int ns = 0, na = 0, st = 0;
-      integrate_cell(M, s, L, p[c], dt[c], h, ns, na, st, oo, g, c);
-      const SPtr y = shared_ptr(s) + L.y;
-      for (int i = g.lane; i < M.m; i += g.size) {
-        if (i == 0) T[c] = y[0];
-        else Y[(size_t)(i - 1) * N + c] = y[i];
+    const auto gs = solo(g);
+    while (!r.active && more) {   // the next cell that has something to integrate
+      if (next >= end) {
+        next = queue_pull(gs, head, chunk);
+        end = min(next + (long long)chunk, (long long)N);
+        if (next >= N) { more = false; break; }
       }
-      if (g.lane == 0) {
-        h_io[c] = h;
-        nsub[c] = ns;
-        status[c] = st;
-        if (nacc_out) nacc_out[c] = na;
+      const int c = perm[next++];
+      load_state(s + L.y, M.m, N, c, T, Y, gs);
+      cell_start(M, s, L, c, p[c], dt[c], h_io[c], oo, gs, r);
+      if (!r.active) {
+        cell_end(oo, gs, r);
+        store_cell(M, s, L, N, gs, r, T, Y, h_io, nsub, status, nacc_out);
+        gs.sync();
       }
-      g.sync();
+    }
+    g.sync();
+    if (!any_cell(g, r.active)) break;
+    const bool was = r.active;
+    cell_step(M, s, L, oo, g, r);
+    if (was && !r.active) {
+      cell_end(oo, gs, r);
+      store_cell(M, s, L, N, gs, r, T, Y, h_io, nsub, status, nacc_out);
+      gs.sync();
     }
   }
 }
