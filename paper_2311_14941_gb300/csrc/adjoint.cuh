@@ -15,8 +15,8 @@
 // A shift of ln A_j scales reaction j's forward and reverse rates (both fall-off limits for Troe), so
 // d f / d lnA_j = e_j q_j with e_j = d f / d q_j, and d f / d Ea_j = -e_j q_j / (Ru T); w^T e_j is a
 // sum over the reaction's participants of a_k = W_k w_k / rho - w_T H_k / (rho c_p).
-// The Hessian and the mixed parameter terms use forward-mode dual numbers through the same rate and
-// Jacobian code (exact, no finite differences).
+// The Hessian and the mixed parameter terms use forward-mode dual numbers through the same rate code (exact, no
+// finite differences).
 #pragma once
 #include "device.cuh"
 
@@ -29,6 +29,11 @@ namespace chemgb {
 // factor), which the transposed solves and the products with J(y)^T read by index.
 struct AdjLayout {
   CellLayout L;        // shared memory: the forward layout
+  CellLayout Ld;       // the dual-number cell of the second-order terms, in dual numbers (contract)
+  int dual_bytes;      // its size; in the warp's shared memory, or (dual_shared 0) in its contraction workspace
+  int slots;           // contracted derivative slots and the partial sums of their gather
+  int dual_shared, slots_shared;   // slots_shared: doubles of them fit the Jacobian's place in the cell
+  int ctr;             // contraction workspace, doubles per warp
   int Y3, Y4, W1, W2, W3, W4, MU1, MU2, MU3, MU4, LAM, G, ZT, WS;   // m-vectors
   // step record, kept by the segment recompute for every step of the segment (offsets within a record):
   int SY;              // nnz_S: S at y (the step's own Jacobian)
@@ -62,6 +67,19 @@ __device__ __forceinline__ void vjp(const MechView& M, P S, P u, P v, const doub
   g.sync();
 }
 
+// sum of a over a reaction's product occurrences minus the sum over its reactant occurrences.
+template <class Sc, class P>
+__device__ __forceinline__ Sc net_of(const RxRec& r, P a) {
+  const int nro = (r.flags >> 1) & 3, npo = (r.flags >> 3) & 3;
+  Sc E = a[r.r2p0 >> 16];
+  if (npo > 1) E += Sc(a[r.p12 & 0xffff]);
+  if (npo > 2) E += Sc(a[r.p12 >> 16]);
+  E -= Sc(a[r.r01 & 0xffff]);
+  if (nro > 1) E -= Sc(a[r.r01 >> 16]);
+  if (nro > 2) E -= Sc(a[r.r2p0 & 0xffff]);
+  return E;
+}
+
 // dL/dtheta += w^T f_theta at an evaluated state: for reaction r, q_r * E_r with E_r = sum_products a_k -
 // sum_reactants a_k, a_k = W_k w_k / rho - w_T H_k / (rho c_p).  hRT, q: the evaluation's h/RT and rates
 // of progress; a: n doubles of scratch (shared memory, read by index).
@@ -75,11 +93,7 @@ __device__ __forceinline__ void theta_terms(const MechView& M, P hRT, P q, doubl
   g.sync();
   const double iRT = rcp_rn(kRu * T);
   for (int r = g.lane; r < M.R; r += g.size) {
-    const int* I = M.rxi + (size_t)r * RX_I;
-    const int nro = __ldg(I + 2), npo = __ldg(I + 3);
-    double E = 0.0;
-    for (int i = 0; i < npo; ++i) E += a[__ldg(I + 7 + i)];
-    for (int i = 0; i < nro; ++i) E -= a[__ldg(I + 4 + i)];
+    const double E = net_of<double>(ld_rx(M, r).i, a);
     const double qE = q[r] * E;
     GA[r] += qE;
     GE[r] += -(qE * iRT);
@@ -109,112 +123,181 @@ __device__ __forceinline__ void vset(P dst, Q src, int m, const Grp1& g) {
   g.sync();
 }
 
-// Tangents carried per dual-number evaluation of the Jacobian in the second-order terms: the four stages
-// take 4 / kTangentsPerPass passes (fewer live registers per dual number against a little more
-// arithmetic per pass).
+// ---- products with the Jacobian without the Jacobian.  With f_k = W_k w_k / rho, f_T = -sum H_k w_k / (rho c_p) and
+// a_k = W_k w_k(weight) / rho - w_T H_k / (rho c_p), the product w^T f is sum_r q_r E_r with E_r = sum_k nu_rk a_k,
+// and J^T w is its derivative at fixed weights:
+//   through the rates:  G_T = sum_r E_r dq_r/dT,  G_j = sum_r E_r dq_r/dC_j  (at fixed total concentration),
+//                       C_j = rho Y_j / W_j:  out_T += G_T - Q/T,  out_j += (rho G_j - Q Wbar) / W_j,  Q = sum_j G_j C_j;
+//   through a_k:        out_T += g/T - w_T Ru sum_k w_k cpR_k / (rho c_p) - w_T f_T Ru dcps / c_p,
+//                       out_j += (g Wbar - w_T f_T Ru cpR_j / c_p) / W_j,  g = sum_r q_r E_r.
+// So a reaction leaves one number per derivative slot, added up by column, where the Jacobian would add it to a row
+// for each of its species: at 53 species / 325 reactions 1,436 terms instead of 7,000, and no S, row and column
+// sums.  The parameter terms are q_r E_r itself.  In dual numbers the same code gives the derivative of J^T w
+// along the tangents: tangent st goes with weight st, and only the tangents of the results are kept.
+//
+// Tangents carried per dual-number evaluation: the four stages take 4 / kTangentsPerPass passes (fewer live registers
+// per dual number against a little more arithmetic per pass).
 constexpr int kTangentsPerPass = 2;
+using ContractDual = DualN<kTangentsPerPass>;
+using ContractVec = DualN<2 * kTangentsPerPass - 1>;   // a number pair (value, tangent) per weight
 
-// sum_st (d_st J)^T W_st into out (m), J = S + u v^T at the dual point (d_st: tangent st):
-//   d(J^T w) = dS^T w + dv (u . w) + v (du . w).
-template <int NT>
-__device__ __forceinline__ void vjp_tangents(const MechView& M, const DualN<NT>* S, const DualN<NT>* u,
-                                             const DualN<NT>* v, const double* const* Ws, double* out, double* part,
-                                             const Grp1& g) {
-  run_gather<false>(M.g_col, out + 1, part, [&](int a, int b) {
-    double acc = 0.0;
-#pragma unroll
-    for (int st = 0; st < NT; ++st) acc = fma(S[a].d[st], Ws[st][1 + b], acc);
-    return acc;
-  }, [](double v, int) { return v; }, g);
-  double t0 = 0.0, uw[NT], duw[NT];
-#pragma unroll
-  for (int st = 0; st < NT; ++st) { uw[st] = 0.0; duw[st] = 0.0; }
-  for (int k = g.lane; k < M.n; k += g.size)
-#pragma unroll
-    for (int st = 0; st < NT; ++st) t0 = fma(S[M.nY + k].d[st], Ws[st][1 + k], t0);
-  for (int i = g.lane; i < M.m; i += g.size)
-#pragma unroll
-    for (int st = 0; st < NT; ++st) {
-      uw[st] = fma(u[i].v, Ws[st][i], uw[st]);
-      duw[st] = fma(u[i].d[st], Ws[st][i], duw[st]);
-    }
-  t0 = gsum(g, t0);
-#pragma unroll
-  for (int st = 0; st < NT; ++st) { uw[st] = gsum(g, uw[st]); duw[st] = gsum(g, duw[st]); }
-  for (int c = g.lane; c < M.m; c += g.size) {
-    double acc = (c == 0) ? t0 : out[c];
-    const DualN<NT>& vc = v[c];
-    const DualN<NT>& sT = S[M.nY + M.n + c];
-#pragma unroll
-    for (int st = 0; st < NT; ++st)
-      acc += fma(vc.d[st], uw[st], fma(vc.v, duw[st], sT.d[st] * Ws[st][0]));
-    out[c] = acc;
+template <class Sc>
+struct Weights;
+template <>
+struct Weights<double> {   // one weight; results are values
+  static constexpr int n = 1;
+  using E = double;
+  using Vec = double;
+  static __device__ __forceinline__ double pick(double x, int) { return x; }
+  static __device__ __forceinline__ double get(double v, int) { return v; }
+  static __device__ __forceinline__ void set(double& v, int, double e) { v = e; }
+  static __device__ __forceinline__ double result(double e) { return e; }
+};
+template <>
+struct Weights<ContractDual> {   // one weight per tangent; results are tangents
+  static constexpr int n = kTangentsPerPass;
+  using E = Dual;
+  using Vec = ContractVec;
+  static __device__ __forceinline__ Dual pick(const ContractDual& x, int st) { return Dual(x.v, x.d[st]); }
+  static __device__ __forceinline__ Dual get(const ContractVec& v, int st) {
+    return st == 0 ? Dual(v.v, v.d[0]) : Dual(v.d[2 * st - 1], v.d[2 * st]);
   }
+  static __device__ __forceinline__ void set(ContractVec& v, int st, Dual e) {
+    if (st == 0) { v.v = e.v; v.d[0] = e.d; }
+    else { v.d[2 * st - 1] = e.v; v.d[2 * st] = e.d; }
+  }
+  static __device__ __forceinline__ double result(Dual e) { return e.d; }
+};
+
+// Takes a reaction's results as eval_reactions produces them.
+template <class Sc>
+struct ToContraction {
+  using W = Weights<Sc>;
+  using E = typename W::E;
+  using Vec = typename W::Vec;
+  const E* a;             // [weights][n]
+  const Sc* hRT;
+  const Sc* cpR;
+  Vec* slots;
+  double* GA;
+  double* GE;
+  int n;
+  E iRT[W::n], e[W::n], G_T[W::n], g[W::n];
+  Sc sh, scp;             // sum_r q_r times the reaction's change of h/RT and of cp/R
+  __device__ __forceinline__ void rate(int r, const RxRec& rec, const Sc& q) {
+    double dA = 0.0, dE = 0.0;
+#pragma unroll
+    for (int st = 0; st < W::n; ++st) {
+      e[st] = net_of<E>(rec, a + st * n);
+      const E qe = W::pick(q, st) * e[st];
+      dA += W::result(qe);
+      dE += W::result(-(qe * iRT[st]));
+      g[st] += qe;
+    }
+    GA[r] += dA;
+    GE[r] += dE;
+    sh = sfma(q, net_of<Sc>(rec, hRT), sh);
+    scp = sfma(q, net_of<Sc>(rec, cpR), scp);
+  }
+  __device__ __forceinline__ void dT(int, const Sc& v) {
+#pragma unroll
+    for (int st = 0; st < W::n; ++st) G_T[st] += e[st] * W::pick(v, st);
+  }
+  __device__ __forceinline__ void slot(int i, const Sc& v) {
+    Vec x;
+#pragma unroll
+    for (int st = 0; st < W::n; ++st) W::set(x, st, e[st] * W::pick(v, st));
+    slots[i] = x;
+  }
+};
+
+// out (m) = J(y)^T w, or for dual numbers the sum over the weights of the tangents of J(y)^T w_st; GA, GE += the
+// parameter terms.  s: the cell (layout L, numbers Sc: y .. cpR, U1 for a, U2 for the column sums); slots: M.n_dslot
+// numbers and the partial sums of their gather.
+template <class Sc>
+__device__ __forceinline__ void contract(const MechView& M, Sc* s, const CellLayout& L, const Sc* y, double p,
+                                         const double* const* ws, typename Weights<Sc>::Vec* slots, double* out,
+                                         double* GA, double* GE, const Grp1& g) {
+  using W = Weights<Sc>;
+  using E = typename W::E;
+  using Vec = typename W::Vec;
+  const ScalT<Sc> sc = eval_species(M, s, L, y, p, g, true);
+  E* a = reinterpret_cast<E*>(s + L.U1);
+  Vec* col = reinterpret_cast<Vec*>(s + L.U2);
+  const Sc* hRT = s + L.hRT;
+  const Sc* cpR = s + L.cpR;
+  const Sc* C = s + L.C;
+  ToContraction<Sc> to{a, hRT, cpR, slots, GA, GE, M.n, {}, {}, {}, {}, Sc(0.0), Sc(0.0)};
+#pragma unroll
+  for (int st = 0; st < W::n; ++st) {
+    const double* w = ws[st];
+    const E c1 = sdiv(E((w[0] * kRu) * W::pick(sc.T, st)), E(W::pick(sc.rho, st) * W::pick(sc.cp, st)));
+    const E irho = W::pick(sc.irho, st);
+    for (int k = g.lane; k < M.n; k += g.size)
+      a[st * M.n + k] = sfma(E(__ldg(M.sp + M.n + k) * w[1 + k]), irho, -(c1 * W::pick(hRT[k], st)));
+    to.iRT[st] = srcp(E(kRu * W::pick(sc.T, st)));
+    to.G_T[st] = E(0.0);
+    to.g[st] = E(0.0);
+  }
+  g.sync();
+  eval_reactions<Sc>(M, s, L, sc, g, 0, M.R, true, to);
+  {
+    auto ld = [&](int i, int) { return slots[i]; };
+    auto fin = [](const Vec& v, int) { return v; };
+    run_gather<false>(M.g_slot, col, slots + M.n_dslot, ld, fin, g);
+  }
+  const Sc sh = gsum(g, to.sh), scp = gsum(g, to.scp);
+  E gq[W::n], cT[W::n];   // g - Q, and w_T f_T Ru / c_p
+  double res_T = 0.0;
+#pragma unroll
+  for (int st = 0; st < W::n; ++st) {
+    E Q = E(0.0);
+    for (int j = g.lane; j < M.n; j += g.size) Q = sfma(W::get(col[j], st), W::pick(C[j], st), Q);
+    Q = gsum(g, Q);
+    const E gt = gsum(g, to.g[st]), GT = gsum(g, to.G_T[st]);
+    const E T = W::pick(sc.T, st), cp = W::pick(sc.cp, st), rcp = W::pick(sc.rho, st) * cp;
+    const double wR = ws[st][0] * kRu;
+    gq[st] = gt - Q;
+    const E ircp = srcp(rcp);
+    cT[st] = sdiv(E(wR * (-kRu * T * W::pick(sh, st) * ircp)), cp);
+    res_T += W::result(GT + gq[st] * W::pick(sc.invT, st) - wR * W::pick(scp, st) * ircp - cT[st] * W::pick(sc.dcps, st));
+  }
+  for (int j = g.lane; j < M.n; j += g.size) {
+    double res = 0.0;
+#pragma unroll
+    for (int st = 0; st < W::n; ++st)
+      res += W::result(sfma(W::pick(sc.rho, st), W::get(col[j], st),
+                            gq[st] * W::pick(sc.Wbar, st) - cT[st] * W::pick(cpR[j], st)));
+    out[1 + j] = res * __ldg(M.sp + j);
+  }
+  if (g.lane == 0) out[0] = res_T;
   g.sync();
 }
 
-template <int NT>
-__device__ __forceinline__ Dual tangent_of(const DualN<NT>& x, int st) { return Dual(x.v, x.d[st]); }
-
-// The mixed parameter terms of the stages of this pass: GA_r, GE_r += sum_st d_st [q_r E_r(W_st)] with
-// the parameter contraction of theta_terms evaluated in the dual number of tangent st.
-template <int NT>
-__device__ __forceinline__ void theta_tangents(const MechView& M, const DualN<NT>* s, const CellLayout& L,
-                                               const ScalT<DualN<NT>>& sc, const double* const* Ws, Dual* a,
-                                               double* GA, double* GE, const Grp1& g) {
-#pragma unroll
-  for (int st = 0; st < NT; ++st) {
-    const double* w = Ws[st];
-    const Dual T = tangent_of(sc.T, st), rho = tangent_of(sc.rho, st), cp = tangent_of(sc.cp, st);
-    const Dual irho = tangent_of(sc.irho, st);
-    const Dual c1 = (w[0] * kRu) * T / (rho * cp);
-    for (int k = g.lane; k < M.n; k += g.size)
-      a[k] = sfma(Dual(__ldg(M.sp + M.n + k) * w[1 + k]), irho, -(c1 * tangent_of(s[L.hRT + k], st)));
-    g.sync();
-    const Dual iRT = 1.0 / (kRu * T);
-    for (int r = g.lane; r < M.R; r += g.size) {
-      const int* I = M.rxi + (size_t)r * RX_I;
-      const int nro = __ldg(I + 2), npo = __ldg(I + 3);
-      Dual E = Dual(0.0);
-      for (int i = 0; i < npo; ++i) E += a[__ldg(I + 7 + i)];
-      for (int i = 0; i < nro; ++i) E -= a[__ldg(I + 4 + i)];
-      const Dual qE = tangent_of(s[L.q + r], st) * E;
-      GA[r] += qE.d;
-      GE[r] += (-(qE * iRT)).d;
-    }
-    g.sync();
-  }
-}
-
-// Second-order terms of NT stages of one step: the Jacobian at y differentiated along their U_i at once,
-// then the state part into LAM and the parameter part into GA, GE.  dwv: the dual workspace (the cell
-// layout in DualN<NT>); tmp: m doubles of scratch.
-template <int NT>
-__device__ __forceinline__ void second_order_terms(const MechView& M, void* dwv, const CellLayout& Ld,
-                                                   const double* y, double p, const double* const* Us,
-                                                   const double* const* Ws, double* LAM, double* tmp, double* GA,
-                                                   double* GE, const Grp1& g) {
-  using DT = DualN<NT>;
-  DT* dw = static_cast<DT*>(dwv);
-  DT* yd = dw + Ld.y;
+// Second-order terms of kTangentsPerPass stages of one step: J(y)^T W_st differentiated along U_st, then the state
+// part into LAM and the parameter part into GA, GE.  cell: the dual-number cell (shared memory, which holds nothing
+// else then, or global); tmp: m doubles of scratch.
+__device__ __forceinline__ void second_order_terms(const MechView& M, ContractDual* cell, const CellLayout& Ld,
+                                                   ContractVec* slots, const double* y, double p,
+                                                   const double* const* Us, const double* const* Ws, double* LAM,
+                                                   double* tmp, double* GA, double* GE, const Grp1& g) {
+  ContractDual* yd = cell + Ld.y;
   for (int i = g.lane; i < M.m; i += g.size) {
-    DT x(y[i]);
+    ContractDual x(y[i]);
 #pragma unroll
-    for (int st = 0; st < NT; ++st) x.d[st] = Us[st][i];
+    for (int st = 0; st < kTangentsPerPass; ++st) x.d[st] = Us[st][i];
     yd[i] = x;
   }
   g.sync();
-  const ScalT<DT> scd = eval_jac(M, dw, Ld, yd, p, g);
-  vjp_tangents<NT>(M, dw + Ld.S, dw + Ld.u, dw + Ld.v, Ws, tmp, reinterpret_cast<double*>(dw + Ld.part), g);
+  contract<ContractDual>(M, cell, Ld, yd, p, Ws, slots, tmp, GA, GE, g);
   for (int i = g.lane; i < M.m; i += g.size) LAM[i] += tmp[i];
   g.sync();
-  theta_tangents<NT>(M, dw, Ld, scd, Ws, reinterpret_cast<Dual*>(dw + Ld.z), GA, GE, g);
 }
 
 // One adjoint step at state y with step h, whose stage vectors U1..U4 and step record jr (the Jacobian
 // at y and the factor of the step) the segment recompute kept.  lambda (A.LAM) is updated in place, the
 // parameter gradients accumulate into GA, GE.
-__device__ __forceinline__ void adjoint_step(const MechView& M, double* s, double* ws, const AdjLayout& A, Dual4* dw,
+__device__ __forceinline__ void adjoint_step(const MechView& M, double* s, double* ws, const AdjLayout& A, double* ctr,
                                              const double* jr, const double* y, const double* U1, const double* U2,
                                              const double* U3, const double* U4, double p, double h, double* GA,
                                              double* GE, const Grp1& g) {
@@ -261,9 +344,8 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
     if (st >= 2) {
       // stage 4: r4 = f(Y4) + (c41 U1 + c42 U2 + c43 U3)/h, Y4 = y + a41 U1 + a43 U3;
       // stage 3: r3 = f(Y3) + (c31 U1 + c32 U2)/h,          Y3 = y + a31 U1
-      const ScalT<double> sc = eval_jac(M, s, L, st == 3 ? Y4 : Y3, p, g);
-      theta_terms(M, s + L.hRT, s + L.q, sc.T, sc.rho, sc.cp, sc.irho, W, a, GA, GE, g);
-      vjp(M, s + L.S, s + L.u, s + L.v, W, G, shared_ptr(s + L.part), g);
+      const double* w1[1] = {W};
+      contract<double>(M, s, L, st == 3 ? Y4 : Y3, p, w1, A.slots_shared ? s + L.S : ctr, G, GA, GE, g);
       if (st == 3) {
         for (int i = g.lane; i < m; i += g.size) {
           MU1[i] = fma(C41 * ih, W4[i], fma(A41, G[i], MU1[i]));
@@ -290,18 +372,19 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
   for (int i = g.lane; i < m; i += g.size) LAM[i] += G[i];
   g.sync();
   theta_terms(M, jr + A.HY, jr + A.QY, jr[A.SC], jr[A.SC + 1], jr[A.SC + 2], jr[A.SC + 3], WS, a, GA, GE, g);
-  // ---- Hessian and mixed parameter terms: derivative of J(y) along U_i, contracted with w_i, for the
-  //      four stages in one evaluation of the Jacobian with four tangents
+  // ---- Hessian and mixed parameter terms: J(y)^T w_i differentiated along U_i, kTangentsPerPass stages at a time
   const double* Us[4] = {U1, U2, U3, U4};
   const double* Ws[4] = {W1, W2, W3, W4};
+  ContractVec* slots = reinterpret_cast<ContractVec*>(ctr);
+  ContractDual* cell = A.dual_shared ? reinterpret_cast<ContractDual*>(s) : reinterpret_cast<ContractDual*>(slots + A.slots);
 #pragma unroll 1
   for (int s0 = 0; s0 < 4; s0 += kTangentsPerPass)
-    second_order_terms<kTangentsPerPass>(M, dw, L, y, p, Us + s0, Ws + s0, LAM, G, GA, GE, g);
+    second_order_terms(M, cell, A.Ld, slots, y, p, Us + s0, Ws + s0, LAM, G, GA, GE, g);
 }
 
 // Reverse pass of one cell from its tape.  ws: the warp's global workspace.  Returns false on a singular
 // factor.
-__device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, double* ws, const AdjLayout& A, Dual4* dw,
+__device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, double* ws, const AdjLayout& A, double* ctr,
                                              double p, int n_acc, const double* rec_h, const double* rec_ck, int K,
                                              int N, int cell, const Grp1& g, const IntOpts& o) {
   const int m = M.m;
@@ -320,16 +403,17 @@ __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, doubl
     for (int nn = n0; nn < n1; ++nn) {
       double* jr = ws + A.JREC + (size_t)(nn - n0) * A.jstride;
       vset(s + L.y, seg + (size_t)(nn - n0) * m, m, g);
-      const ScalT<double> sy = eval_jac(M, s, L, s + L.y, p, g);
-      vset(jr + A.SY, s + L.S, M.nnz_S, g);
-      vset(jr + A.UY, s + L.u, m, g);
-      vset(jr + A.VY, s + L.v, m, g);
-      vset(jr + A.QY, s + L.q, M.R, g);
-      vset(jr + A.HY, s + L.hRT, M.n, g);
-      if (g.lane == 0) {
-        jr[A.SC] = sy.T; jr[A.SC + 1] = sy.rho; jr[A.SC + 2] = sy.cp; jr[A.SC + 3] = sy.irho;
-      }
-      const StepOut so = ros_attempt(M, s, L, p, rec_h[(size_t)nn * N + cell], o.rtol, o.atol, g, 0, false);
+      auto record = [&](const Scal& sy) {
+        vset(jr + A.SY, s + L.S, M.nnz_S, g);
+        vset(jr + A.UY, s + L.u, m, g);
+        vset(jr + A.VY, s + L.v, m, g);
+        vset(jr + A.QY, s + L.q, M.R, g);
+        vset(jr + A.HY, s + L.hRT, M.n, g);
+        if (g.lane == 0) {
+          jr[A.SC] = sy.T; jr[A.SC + 1] = sy.rho; jr[A.SC + 2] = sy.cp; jr[A.SC + 3] = sy.irho;
+        }
+      };
+      const StepOut so = ros_attempt(M, s, L, p, rec_h[(size_t)nn * N + cell], o.rtol, o.atol, g, 0, true, record);
       if (!so.good) return false;   // also a singular factor (cannot happen for a step the forward pass accepted)
       vset(jr + A.LUG, s + L.LU, M.nnz_LU + m, g);
       double* u4 = ust + (size_t)(nn - n0) * 4 * m;
@@ -341,7 +425,7 @@ __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, doubl
     }
     for (int nn = n1 - 1; nn >= n0; --nn) {
       const double* u4 = ust + (size_t)(nn - n0) * 4 * m;
-      adjoint_step(M, s, ws, A, dw, ws + A.JREC + (size_t)(nn - n0) * A.jstride, seg + (size_t)(nn - n0) * m, u4,
+      adjoint_step(M, s, ws, A, ctr, ws + A.JREC + (size_t)(nn - n0) * A.jstride, seg + (size_t)(nn - n0) * m, u4,
                    u4 + m, u4 + 2 * m, u4 + 3 * m, p, rec_h[(size_t)nn * N + cell], GA, GE, g);
     }
   }

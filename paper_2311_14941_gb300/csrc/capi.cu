@@ -147,12 +147,28 @@ AdjLayout make_adj_layout(const HostMech& hm, int K) {
   AdjLayout A{};
   A.L = make_layout(hm);
   int o = 0;
-  const int m = hm.m;
+  const int m = hm.m, n = hm.n;
   // 256-byte aligned pieces (32 doubles): coalesced lane-strided access
   auto take = [&](int cnt) { int at = o; o += (cnt + 31) / 32 * 32; return at; };
   A.Y3 = take(m); A.Y4 = take(m); A.W1 = take(m); A.W2 = take(m); A.W3 = take(m); A.W4 = take(m);
   A.MU1 = take(m); A.MU2 = take(m); A.MU3 = take(m); A.MU4 = take(m); A.LAM = take(m); A.G = take(m);
   A.ZT = take(m); A.WS = take(m);
+  {   // the dual-number cell of the contracted Jacobian: state, weights a (U1), column sums (U2), thermo
+    CellLayout& D = A.Ld;
+    int d = 0;
+    auto dtake = [&](size_t bytes) { int at = d; d += (int)((bytes + sizeof(ContractDual) - 1) / sizeof(ContractDual)); return at; };
+    auto vec = [&](int cnt) { return dtake(cnt * sizeof(ContractDual)); };
+    D.y = vec(m);
+    D.U1 = dtake((size_t)kTangentsPerPass * n * sizeof(Dual));
+    D.U2 = dtake((size_t)n * sizeof(ContractVec));
+    D.C = vec(n); D.hRT = vec(n); D.eg = vec(n); D.emg = vec(n); D.cpR = vec(n);
+    D.total = d;
+    A.dual_bytes = d * (int)sizeof(ContractDual);
+    A.slots = hm.n_dslot + hm.prog[0].g_slot.n_partial;
+    A.slots_shared = A.slots <= A.L.part - A.L.S;
+    A.dual_shared = A.dual_bytes <= A.L.total * (int)sizeof(double);
+    A.ctr = (int)(align_up((size_t)A.slots * sizeof(ContractVec) + (A.dual_shared ? 0 : A.dual_bytes), 256) / sizeof(double));
+  }
   {   // one step record: offsets within it
     int r = 0;
     auto rtake = [&](int cnt) { int at = r; r += (cnt + 31) / 32 * 32; return at; };
@@ -606,15 +622,15 @@ chem_status chem_create(const chem_mech_desc* desc, int device, chem_handle* out
          o_rxr = put(buf, hm.rxr);
   const int n_jp = (int)hm.jpass.size() / 4;
   if (n_jp > kMaxJPass) { delete h; return fail(CHEM_EUNSUPPORTED, "too many Jacobian passes"); }
-  constexpr int kMaxG = 3 + kMaxJPass;
+  constexpr int kMaxG = 4 + kMaxJPass;
   size_t o_g[kNumGroups][kMaxG][2], o_p[kNumGroups][4][2];
   HostFma progs[kNumGroups][4];   // elimination, substitution for all and for half the lanes, transposed
   const HostGather* gs[kNumGroups][kMaxG];
   for (int w = 0; w < kNumGroups; ++w) {
     const HostProg& P = hm.prog[w];
-    gs[w][0] = &P.g_omega; gs[w][1] = &P.g_row; gs[w][2] = &P.g_col;
-    for (int i = 0; i < n_jp; ++i) gs[w][3 + i] = &P.g_jac[i];
-    for (int i = 0; i < 3 + n_jp; ++i) { o_g[w][i][0] = put(buf, gs[w][i]->ops); o_g[w][i][1] = put(buf, gs[w][i]->comb); }
+    gs[w][0] = &P.g_omega; gs[w][1] = &P.g_row; gs[w][2] = &P.g_col; gs[w][3] = &P.g_slot;
+    for (int i = 0; i < n_jp; ++i) gs[w][4 + i] = &P.g_jac[i];
+    for (int i = 0; i < 4 + n_jp; ++i) { o_g[w][i][0] = put(buf, gs[w][i]->ops); o_g[w][i][1] = put(buf, gs[w][i]->comb); }
     progs[w][0] = device_program(P.lu_ops, P.lu_kind, P.width, P.width, hm.nnz_LU, true);
     progs[w][1] = device_program(P.sv_ops, P.sv_kind, P.width, P.width, hm.nnz_LU, false);
     progs[w][2] = device_program(P.sv_ops, P.sv_kind, P.width, P.width / 2, hm.nnz_LU, false);
@@ -649,9 +665,9 @@ chem_status chem_create(const chem_mech_desc* desc, int device, chem_handle* out
     V.n_jpass = n_jp;
     for (int i = 0; i < n_jp; ++i)
       for (int j = 0; j < 4; ++j) V.jpass[i][j] = hm.jpass[(size_t)i * 4 + j];
-    Gather* vg[kMaxG] = {&V.g_omega, &V.g_row, &V.g_col};
-    for (int i = 0; i < n_jp; ++i) vg[3 + i] = &V.g_jac[i];
-    for (int i = 0; i < 3 + n_jp; ++i) {
+    Gather* vg[kMaxG] = {&V.g_omega, &V.g_row, &V.g_col, &V.g_slot};
+    for (int i = 0; i < n_jp; ++i) vg[4 + i] = &V.g_jac[i];
+    for (int i = 0; i < 4 + n_jp; ++i) {
       vg[i]->ops = (const GatherOp*)(b + o_g[w][i][0]);
       vg[i]->blocks = gs[w][i]->steps / kProgBlock;
       vg[i]->n_partial = gs[w][i]->n_partial;
@@ -981,7 +997,7 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
   bps = std::max(bps, 1);
   const int grid = std::min(h->num_sms * bps, N);
   // scratch: head, tape (h, checkpoints, counts), h_io/nsub of the forward pass, per-cell gradients,
-  // dual workspaces
+  // contraction workspaces
   const size_t nck = (size_t)(cap / K + 1);
   const size_t b_head = 256;
   const size_t b_rh = align_up((size_t)cap * N * 8, 256);
@@ -990,7 +1006,7 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
   const size_t b_hio = align_up((size_t)N * 8, 256);
   const size_t b_ns = align_up((size_t)N * 4, 256);
   const size_t b_gc = grad_cell ? 0 : align_up((size_t)2 * hm.R * N * 8, 256);
-  const size_t b_dw = align_up((size_t)grid * h->L.total * sizeof(Dual4), 256);
+  const size_t b_dw = align_up((size_t)grid * A.ctr * sizeof(double), 256);
   const size_t b_ww = align_up((size_t)grid * (size_t)A.total * 8, 256);
   const size_t need = b_head + b_rh + b_ck + b_rn + b_hio + b_ns + b_gc + b_dw + b_ww;
   if (need > h->adj_scratch_bytes) {
@@ -1012,7 +1028,7 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
   int* nsub = (int*)q; q += b_ns;
   double* gcell = grad_cell;
   if (!gcell) { gcell = (double*)q; q += b_gc; }
-  Dual4* dws = (Dual4*)q; q += b_dw;
+  double* dws = (double*)q; q += b_dw;
   double* wws = (double*)q;
   cudaStream_t strm = (cudaStream_t)stream;
   // forward pass with the tape

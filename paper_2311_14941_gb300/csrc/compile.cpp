@@ -787,6 +787,11 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
         if (kv.second != 0) gw[kv.first].push_back({pos[r], enc_nu(kv.second)});
     for (HostProg& Pg : hm.prog)
       if (!build_gather(gw, Pg.g_omega, err, Pg.width)) return CHEM_EUNSUPPORTED;
+    std::vector<std::vector<std::pair<int, int>>> gs(n);
+    for (int r = 0; r < R; ++r)
+      for (size_t c = 0; c < slots_sp[r].size(); ++c)
+        gs[slots_sp[r][c]].push_back({hm.rxi[(size_t)pos[r] * RX_I + 13] + (int)c, 0});
+    if (!build_gather(gs, hm.prog[0].g_slot, err, hm.prog[0].width)) return CHEM_EUNSUPPORTED;
     hm.jpass.clear();
     for (HostProg& Pg : hm.prog) Pg.g_jac.assign(P, HostGather());
     for (int p = 0; p < P; ++p) {

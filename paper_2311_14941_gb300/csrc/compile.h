@@ -19,7 +19,7 @@ struct HostGather {
 // The warp programs for one group width (the lanes that integrate a cell: 32, 64 or 16).
 struct HostProg {
   int width = kWarp;
-  HostGather g_omega, g_row, g_col;
+  HostGather g_omega, g_row, g_col, g_slot;
   std::vector<HostGather> g_jac;       // one gather program per Jacobian pass
   std::vector<ElimOp> lu_ops, sv_ops, svT_ops;   // [steps * width]
   std::vector<uint8_t> lu_kind, sv_kind, svT_kind;

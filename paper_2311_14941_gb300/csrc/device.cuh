@@ -329,6 +329,7 @@ struct pointee<const T*> {
 template <class P>
 using num = typename pointee<P>::type;
 
+
 // ---- running the warp programs.  A program is tens of kilobytes, more than the L1 that the cells' shared memory
 // leaves, so every step's ops come from L2, 300 to 600 cycles away.  The steps are therefore taken in blocks of
 // kProgBlock: a lane loads its ops of the next block (independent loads) before it executes the current one.  A
@@ -609,11 +610,11 @@ __device__ __forceinline__ ScalT<num<P>> eval_species(const MV& M, P s, const LT
   const Sc T = sc.T;
   Sc sig = Sc(0.0), cps = Sc(0.0), dcps = Sc(0.0), first = Sc(0.0);
   bool odd = false;
-  const P hRT = s + L.hRT;
-  const P egv = s + L.eg;
-  const P emg = s + L.emg;
-  const P cpv = s + L.cpR;
-  const P C = s + L.C;
+  const auto hRT = s + L.hRT;
+  const auto egv = s + L.eg;
+  const auto emg = s + L.emg;
+  const auto cpv = s + L.cpR;
+  const auto C = s + L.C;
   double tmid = __ldg(M.sp + 2 * M.n + min(g.lane, M.n - 1));   // the range decides which coefficients to read
 #pragma unroll 1
   for (int k = g.lane; k < M.n; k += g.size) {
@@ -679,11 +680,11 @@ __device__ __forceinline__ Sc rx_kf(const MV& M, int r, const RxIn& x, const Sca
 // from s[d_off + so] on).  The FP64 pipe takes one warp instruction per 64 cycles and is what bounds this code:
 // with it and the tables as structures of arrays, the source term of 65,536 cells of 53 species / 325 reactions
 // went from 2999 to 2667 us, the Jacobian of 8,191 cells from 1236 to 1071 us.
-template <class Sc, class P, class MV, class LT>
+template <class Sc, class P, class MV, class LT, class Sink>
 __device__ __forceinline__ void rx_simple(const MV& M, int r, const RxIn& in, P s, const LT& L, const ScalT<Sc>& sc,
-                                          bool valid, int dq_off, int d_off, bool deriv) {
+                                          bool valid, bool deriv, Sink& to) {
   const int r0 = in.i.r01 & 0xffff, r1 = in.i.r01 >> 16, p0 = in.i.r2p0 >> 16, p1 = in.i.p12 & 0xffff;
-  const P C = s + L.C, eg = s + L.eg, emg = s + L.emg;
+  const auto C = s + L.C, eg = s + L.eg, emg = s + L.emg;
   Sc lnk;
   const Sc kf = rx_kf(M, r, in, sc, lnk);
   const Sc cr0 = C[r0], cr1 = C[r1], cp0 = C[p0], cp1 = C[p1];
@@ -692,9 +693,9 @@ __device__ __forceinline__ void rx_simple(const MV& M, int r, const RxIn& in, P 
   ik *= Sc(emg[r1]);
   const Sc kr = kf * ik;
   const Sc q = sfma(kf, cr0 * cr1, -(kr * (cp0 * cp1)));
-  if (valid) s[L.q + r] = q;
+  if (valid) to.rate(r, in.i, q);
   if (deriv) {
-    const P hRT = s + L.hRT;
+    const auto hRT = s + L.hRT;
     const int so = (int)(in.i.flags >> 16);
     const Sc dlnkf = sfma(Sc(in.Ta), sc.invT, Sc(in.b)) * sc.invT;
     Sc sh = Sc(hRT[p0]) - Sc(hRT[r0]);
@@ -713,9 +714,8 @@ __device__ __forceinline__ void rx_simple(const MV& M, int r, const RxIn& in, P 
       dq = dq - Sc(0.0) * sc.ctot * sc.invT;
     }
     if (valid) {
-      s[dq_off + r] = dq;
-      const P d = s + (d_off + so);
-      d[0] = s0; d[1] = s1; d[2] = s2; d[3] = s3;
+      to.dT(r, dq);
+      to.slot(so, s0); to.slot(so + 1, s1); to.slot(so + 2, s2); to.slot(so + 3, s3);
     }
   }
 }
@@ -866,11 +866,11 @@ __device__ __forceinline__ RxCore<Sc> rx_core(const MV& M, int r, int type, cons
 
 // Store q (and with deriv: dq/dT at fixed C into s[dq_off + r], and the derivative slots dq/dC_j into
 // s[d_off + slot]) of reaction r.
-template <class Sc, class P, class MV, class LT>
-__device__ __forceinline__ void rx_store(const MV& M, int r, int type, const RxCore<Sc>& x, P s, const LT& L,
-                                         const ScalT<Sc>& sc, bool valid, int dq_off, int d_off, bool deriv) {
+template <class Sc, class MV, class Sink>
+__device__ __forceinline__ void rx_store(const MV& M, int r, int type, const RxRec& rec, const RxCore<Sc>& x,
+                                         const ScalT<Sc>& sc, bool valid, bool deriv, Sink& to) {
   if (!valid) return;
-  s[L.q + r] = x.q;
+  to.rate(r, rec, x.q);
   if (!deriv) return;
   const Sc kfM = x.kf * x.Mfac, krM = x.kr * x.Mfac;
   const Sc qf = kfM * x.cr0 * x.cr1 * x.cr2, qr = krM * x.cp0 * x.cp1 * x.cp2;
@@ -878,22 +878,22 @@ __device__ __forceinline__ void rx_store(const MV& M, int r, int type, const RxC
   if (type == 1) dqdM = x.qn;
   if (type == 2) dqdM = x.dlnk_dlnM * x.q * x.iM;
   // [M] depends on T through the total concentration p/(Ru T)
-  s[dq_off + r] = sfma(x.dlnkf_dT, qf, -((x.dlnkf_dT - x.dlnKc_dT) * qr)) - dqdM * sc.ctot * sc.invT;
+  to.dT(r, sfma(x.dlnkf_dT, qf, -((x.dlnkf_dT - x.dlnKc_dT) * qr)) - dqdM * sc.ctot * sc.invT);
   // partial products: d(prod)/d(occurrence i) = product of the other occurrences
   const Sc dr0 = x.cr1 * x.cr2, dr1 = x.cr0 * x.cr2, dr2 = x.cr0 * x.cr1;
   const Sc dp0 = x.cp1 * x.cp2, dp1 = x.cp0 * x.cp2, dp2 = x.cp0 * x.cp1;
   const bool fin = finite_bits(val(kfM)) && finite_bits(val(krM));
   constexpr int kBatch = batch_of<Sc>();
   for (int i0 = 0; i0 < x.scn; i0 += kBatch) {
-    SlotRec rec[kBatch];
+    SlotRec slots[kBatch];
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j) rec[j] = ld_rec(M.dslot + x.so + min(i0 + j, x.scn - 1));
+    for (int j = 0; j < kBatch; ++j) slots[j] = ld_rec(M.dslot + x.so + min(i0 + j, x.scn - 1));
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
-      const int i = i0 + j, mask = rec[j].mask;
+      const int i = i0 + j, mask = slots[j].mask;
       if (i >= x.scn) break;
       // elementary reactions list no colliders: their (efficiency - 1) is 0 and so is the [M] term
-      Sc v = type == 0 ? Sc(0.0) : rec[j].am1 * dqdM;
+      Sc v = type == 0 ? Sc(0.0) : slots[j].am1 * dqdM;
       if (mask != 0 || !fin) {   // a participant (a species that only collides has no factor: the [M] term is all)
         // the slot's factor on a side is the sum over the species' occurrences there, nearly always one: it is
         // selected, and a second or third one added
@@ -910,19 +910,30 @@ __device__ __forceinline__ void rx_store(const MV& M, int r, int type, const RxC
         v = sfma(kfM, fr, v);
         v = sfma(-krM, fq, v);
       }
-      s[d_off + x.so + i] = v;
+      to.slot(x.so + i, v);
     }
   }
 }
 
-// Rates of progress of reactions [rb, re), in rounds of one reaction per lane.  A round whose reactions are all
-// simple takes the short form (every lane of a round's warp takes part: lanes past the end repeat the last reaction
-// and store nothing).  The other types stand first (Troe, third-body) and share their rounds: what a Troe or
-// third-body reaction needs beyond an elementary one is a branch that the round takes once.
-template <class Sc, class P, class Gp, class MV, class LT>
+// Where eval_reactions leaves its results: q, and with derivatives dq/dT and the slots, in the cell's memory.
+template <class P>
+struct ToCell {
+  P s;
+  int q_off, dq_off, d_off;
+  __device__ __forceinline__ void rate(int r, const RxRec&, const num<P>& q) const { s[q_off + r] = q; }
+  __device__ __forceinline__ void dT(int r, const num<P>& v) const { s[dq_off + r] = v; }
+  __device__ __forceinline__ void slot(int i, const num<P>& v) const { s[d_off + i] = v; }
+};
+
+// Rates of progress of reactions [rb, re), in rounds of one reaction per lane; to.rate(), and with deriv to.dT() and
+// to.slot(), take each reaction's results.  A round whose reactions are all simple takes the short form (every lane
+// of a round's warp takes part: lanes past the end repeat the last reaction and leave nothing).  The other types
+// stand first (Troe, third-body) and share their rounds: what a Troe or third-body reaction needs beyond an
+// elementary one is a branch that the round takes once.
+template <class Sc, class P, class Gp, class MV, class LT, class Sink>
 __device__ __forceinline__ void eval_reactions(const MV& M, P s, const LT& L, const ScalT<Sc>& sc,
-                                               const Gp& g, int rb, int re, int dq_off, int d_off, bool deriv) {
-  const P C = s + L.C, eg = s + L.eg, emg = s + L.emg, hRT = s + L.hRT;
+                                               const Gp& g, int rb, int re, bool deriv, Sink& to) {
+  const auto C = s + L.C, eg = s + L.eg, emg = s + L.emg, hRT = s + L.hRT;
   if (rb < re) {
     RxIn next = ld_rx(M, min(rb + g.lane, re - 1));
 #pragma unroll 1
@@ -932,11 +943,10 @@ __device__ __forceinline__ void eval_reactions(const MV& M, P s, const LT& L, co
       const RxIn in = next;
       if (base + g.size < re) next = ld_rx(M, min(base + g.size + g.lane, re - 1));
       if (wall(g, (in.i.flags & RXF_SIMPLE) != 0)) {
-        rx_simple<Sc>(M, r, in, s, L, sc, valid, dq_off, d_off, deriv);
+        rx_simple<Sc>(M, r, in, s, L, sc, valid, deriv, to);
       } else {
         const int type = r < M.n_troe ? 2 : r < M.n_troe + M.n_tb ? 1 : 0;
-        rx_store<Sc>(M, r, type, rx_core<Sc, P>(M, r, type, in, C, eg, emg, hRT, sc, deriv), s, L, sc, valid, dq_off,
-                     d_off, deriv);
+        rx_store<Sc>(M, r, type, in.i, rx_core<Sc>(M, r, type, in, C, eg, emg, hRT, sc, deriv), sc, valid, deriv, to);
       }
     }
   }
@@ -948,12 +958,12 @@ __device__ __forceinline__ void eval_reactions(const MV& M, P s, const LT& L, co
 // Y block of S (Dtil) and w_T in the T-column slots of S.  For those the reactions run in passes (see
 // MechView::jpass): each pass leaves dq/dT and the derivative slots of its reactions in the region D, and its
 // gather adds them into S.  deriv is a run-time flag so that a kernel that needs both holds the code once.
-template <class P, class Q, class Gp, class MV, class LT>
-__device__ __forceinline__ ScalT<num<P>> eval_rates(const MV& M, P s, const LT& L, Q y, double p, P w, const Gp& g,
+template <class P, class Q, class W, class Gp, class MV, class LT>
+__device__ __forceinline__ ScalT<num<P>> eval_rates(const MV& M, P s, const LT& L, Q y, double p, W w, const Gp& g,
                                                     bool deriv) {
   using Sc = num<P>;
   const ScalT<Sc> sc = eval_species(M, s, L, y, p, g, deriv);
-  const P S = s + L.S;
+  const auto S = s + L.S;
   const auto sp = prog_ptr(s);
   if (deriv)
     for (int e = g.lane; e < M.nY + M.n; e += g.size) S[e] = Sc(0.0);
@@ -962,7 +972,8 @@ __device__ __forceinline__ ScalT<num<P>> eval_rates(const MV& M, P s, const LT& 
   for (int ps = 0; ps < passes; ++ps) {
     const int rb = deriv ? M.jpass[ps][JP_RB] : 0, re = deriv ? M.jpass[ps][JP_RE] : M.R;
     const int cnt = M.jpass[ps][JP_CNT];
-    eval_reactions<Sc>(M, s, L, sc, g, rb, re, L.D - rb, L.D + cnt - M.jpass[ps][JP_SB], deriv);
+    const ToCell<P> to{s, L.q, L.D - rb, L.D + cnt - M.jpass[ps][JP_SB]};
+    eval_reactions<Sc>(M, s, L, sc, g, rb, re, deriv, to);
     if (deriv && ps == 0) gather_nu<false>(M.g_jac[0], sp + L.S, sp + L.part, sp + L.D, g);
     if (deriv && ps > 0) gather_nu<true>(M.g_jac[ps], sp + L.S, sp + L.part, sp + L.D, g);
   }
@@ -997,12 +1008,12 @@ __device__ __forceinline__ ScalT<num<P>> eval_f(const MV& M, P s, const LT& L, Q
 // w_T in S (the T column takes w_T's place).  Scratch: U1 (g), U2 (t).
 template <class Sc, class P, class Gp, class MV, class LT>
 __device__ __forceinline__ void finish_jac(const MV& M, P s, const LT& L, const ScalT<Sc>& sc, const Gp& g) {
-  const P w = s + L.x, gk = s + L.U1, tk = s + L.U2, S = s + L.S, wT = s + (L.S + M.nY);
-  const P C = s + L.C, hRT = s + L.hRT;
+  const auto w = s + L.x, gk = s + L.U1, tk = s + L.U2, S = s + L.S, wT = s + (L.S + M.nY);
+  const auto C = s + L.C, hRT = s + L.hRT;
   const auto sp = prog_ptr(s);
   gather_xy(M.g_row, sp + L.U1, sp + L.part, sp + L.S, sp + L.C, g);
   gather_xy(M.g_col, sp + L.U2, sp + L.part, sp + L.S, sp + L.hRT, g);
-  const P f = s + L.f0, u = s + L.u, v = s + L.v;
+  const auto f = s + L.f0, u = s + L.u, v = s + L.v;
   const Sc T = sc.T;
   // f, u and the T column; partial sums for the T row scalars
   Sc Qs = Sc(0.0), A1 = Sc(0.0), A2 = Sc(0.0);
@@ -1104,15 +1115,19 @@ struct StepOut {
 };
 
 // One attempt of size h from y with method 0 RODAS3, 1 ROS2 or 2 RODAS4; need_jac: f0, S, u, v are evaluated at y
-// first (otherwise they hold that already).  ynew into ytmp, err into the return value.  U1..U4, x, z, LU are
+// first (otherwise they hold that already), then after_jac sees the evaluation's scalars.  ynew into ytmp, err into the return value.  U1..U4, x, z, LU are
 // scratch: RODAS4's U5 lives in the Jacobian's w_k vector (x), its stage 6 gathers the coefficient sum into U1 and
 // takes U2's place, both dead by then.
 // All stages of all methods, the Jacobian included, go through one loop with one copy of the rates and of the
 // solve.  Written out, the kernel held four copies of the rates and nine of the solve and waited on instruction
 // fetch.
-template <class Gp, class MV, class LT>
+struct NoHook {
+  __device__ __forceinline__ void operator()(const Scal&) const {}
+};
+template <class Gp, class MV, class LT, class Hook = NoHook>
 __device__ __forceinline__ StepOut ros_attempt(const MV& M, double* sd, const LT& L, double p, double h,
-                                               double rtol, double atol, const Gp& g, int method, bool need_jac) {
+                                               double rtol, double atol, const Gp& g, int method, bool need_jac,
+                                               Hook after_jac = Hook()) {
   StepOut so{false, 0.0};
   const int m = M.m;
   const SPtr s = shared_ptr(sd);
@@ -1151,8 +1166,12 @@ __device__ __forceinline__ StepOut ros_attempt(const MV& M, double* sd, const LT
     if (rates) {
       double* to = sd + (k == 0 ? L.x - 1 : k < 4 ? L.U1 + k * (L.U2 - L.U1) : k == 4 ? L.x : L.U2);
       const Scal sc = eval_rates(M, sd, L, sd + (k == 0 ? L.y : L.ytmp), p, to + 1, g, k == 0);
-      if (k == 0) finish_jac(M, sd, L, sc, g);
-      else finish_f(M, sd, L, sc, to, g);
+      if (k == 0) {
+        finish_jac(M, sd, L, sc, g);
+        after_jac(sc);
+      } else {
+        finish_f(M, sd, L, sc, to, g);
+      }
     }
     if (k == 0) {
       fine = lu_build_factor(M, s, L, ih * (method == 1 ? 1.0 / RG2 : method == 2 ? 1.0 / RG4 : 1.0 / RG), g);

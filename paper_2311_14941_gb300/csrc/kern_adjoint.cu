@@ -8,18 +8,18 @@
 namespace chemgb {
 
 // ---- discrete adjoint: resident warps pull cells (longest tapes first).  Shared memory: the forward cell
-// layout; each warp's workspace (AdjLayout offsets) and dual-number workspace are in global memory.
+// layout; each warp's workspace (AdjLayout offsets) and contraction workspace are in global memory.
 __global__ void __launch_bounds__(32, 8)
 k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const double* __restrict__ rec_h,
           const double* __restrict__ rec_ck, const int* __restrict__ rec_n, int K, const double* __restrict__ gT,
           const double* __restrict__ gY, double* __restrict__ grad_cell, double* __restrict__ gT0,
           double* __restrict__ gY0, int* __restrict__ status, int* __restrict__ head, const int* __restrict__ perm,
-          Dual4* dual_ws, double* warp_ws, IntOpts o) {
+          double* ctr_ws, double* warp_ws, IntOpts o) {
   extern __shared__ double smem[];
   const int lane = threadIdx.x % kWarp;
   const int gw = blockIdx.x;   // one warp per block
   double* s = smem;
-  Dual4* dw = dual_ws + (size_t)gw * A.L.total;
+  double* ctr = ctr_ws + (size_t)gw * A.ctr;
   double* ws = warp_ws + (size_t)gw * A.total;
   const int m = M.m;
   double* LAM = ws + A.LAM;
@@ -36,7 +36,7 @@ k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const do
     for (int r = lane; r < M.R; r += kWarp) { GA[r] = 0.0; GE[r] = 0.0; }
     __syncwarp();
     bool ok = na >= 0;
-    if (ok) ok = adjoint_cell(M, s, ws, A, dw, p[c], na, rec_h, rec_ck, K, N, c, Grp1{lane}, o);
+    if (ok) ok = adjoint_cell(M, s, ws, A, ctr, p[c], na, rec_h, rec_ck, K, N, c, Grp1{lane}, o);
     if (!ok) {
       for (int i = lane; i < m; i += kWarp) LAM[i] = 0.0;
       for (int r = lane; r < M.R; r += kWarp) { GA[r] = 0.0; GE[r] = 0.0; }

@@ -154,6 +154,7 @@ struct MechView {
                              // Y block), b = top 16 bits of double(nu)
   Gather g_row;              // species k <- sum_j Dtil_kj C_j (a = entry, b = species j)
   Gather g_col;              // species i <- sum_k h_k Dtil_ki (a = entry, b = species k)
+  Gather g_slot;             // species j <- derivative slots of column j (one warp per cell only: the adjoint)
   const int* lu_src;         // [nnz_LU] S index feeding the slot (-1: fill)
   const int* lu_diag;        // [m] LU slot of the diagonal of state index s (natural order)
   FmaProgram lu;             // elimination

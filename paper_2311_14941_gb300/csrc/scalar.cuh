@@ -89,7 +89,7 @@ struct DualN {
     for (int i = 0; i < K; ++i) d[i] = 0.0;
   }
 };
-using Dual4 = DualN<4>;
+
 
 template <int K>
 __device__ __forceinline__ DualN<K> operator+(const DualN<K>& a, const DualN<K>& b) {
