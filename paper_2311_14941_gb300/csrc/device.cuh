@@ -487,8 +487,9 @@ __device__ __forceinline__ void gather_blocks(const GT& G, P out, PP part, Ld ld
       const bool end = o.dst != DST_NONE, partial = (o.dst & PARTIAL_BIT) != 0;
       if (ADD) {
         if (o.flags & GF_END) {
-          if (end && !partial) out[o.dst] += acc;
-          if (end && partial) part[o.dst & 0x7FFF] = acc;
+          const Sc old = out[partial ? 0 : (int)o.dst];
+          store_if(out, o.dst, old + acc, !partial);
+          store_if(part, o.dst & 0x7FFF, acc, end && partial);
           if (end) acc = Sc(0.0);
         }
       } else {
@@ -1011,6 +1012,9 @@ __device__ __forceinline__ void finish_jac(const MV& M, P s, const LT& L, const 
   const auto w = s + L.x, gk = s + L.U1, tk = s + L.U2, S = s + L.S, wT = s + (L.S + M.nY);
   const auto C = s + L.C, hRT = s + L.hRT;
   const auto sp = prog_ptr(s);
+  // the tables of the loops below are asked for ahead of the sums before them
+  const int k0 = min(g.lane, M.n - 1);
+  double nW = __ldg(M.sp + M.n + k0), niW = __ldg(M.sp + k0);
   gather_xy(M.g_row, sp + L.U1, sp + L.part, sp + L.S, sp + L.C, g);
   gather_xy(M.g_col, sp + L.U2, sp + L.part, sp + L.S, sp + L.hRT, g);
   const auto f = s + L.f0, u = s + L.u, v = s + L.v;
@@ -1018,19 +1022,26 @@ __device__ __forceinline__ void finish_jac(const MV& M, P s, const LT& L, const 
   // f, u and the T column; partial sums for the T row scalars
   Sc Qs = Sc(0.0), A1 = Sc(0.0), A2 = Sc(0.0);
   for (int k = g.lane; k < M.n; k += g.size) {
-    const double Wk = __ldg(M.sp + M.n + k);
+    const double Wk = nW, iWk = niW;
+    const int kn = min(k + g.size, M.n - 1);
+    nW = __ldg(M.sp + M.n + kn);
+    niW = __ldg(M.sp + kn);
     const Sc om = w[k], g = gk[k];
     const Sc dwT = sfma(-g, sc.invT, Sc(wT[k]));   // read before the T column overwrites w_T
     const Sc fk = Wk * om * sc.irho;
     f[1 + k] = fk;
     u[1 + k] = Wk * sc.irho * (om - g);
     S[M.nY + k] = sfma(Wk * sc.irho, dwT, fk * sc.invT);
-    v[1 + k] = sc.Wbar * __ldg(M.sp + k);
+    v[1 + k] = sc.Wbar * iWk;
     const Sc h = hRT[k];
     Qs = sfma(h, om, Qs);
     A1 = sfma(Sc(s[L.cpR + k]), om, sfma(T * h, dwT, A1));
     A2 = sfma(h, g, A2);
   }
+  constexpr int kScale = 8;   // the first batch of the species block's factors
+  double ratio[kScale];
+#pragma unroll
+  for (int i = 0; i < kScale; ++i) ratio[i] = __ldg(M.entry_wratio + min(g.lane + i * g.size, M.nY - 1));
   gsum3(g, Qs, A1, A2);
   const Sc rcp = sc.rho * sc.cp;
   const Sc fT = sdiv(-kRu * T * Qs, rcp);
@@ -1047,8 +1058,14 @@ __device__ __forceinline__ void finish_jac(const MV& M, P s, const LT& L, const 
   }
   g.sync();
   // species block: S_kj = (W_k / W_j) Dtil_kj (after the row and column sums used Dtil)
-#pragma unroll 8
-  for (int e = g.lane; e < M.nY; e += g.size) S[e] *= __ldg(M.entry_wratio + e);
+  for (int e0 = 0; e0 < M.nY; e0 += kScale * g.size) {
+#pragma unroll
+    for (int i = 0; i < kScale; ++i) {
+      const int e = e0 + g.lane + i * g.size;
+      if (e < M.nY) S[e] *= ratio[i];
+      ratio[i] = __ldg(M.entry_wratio + min(e + kScale * g.size, M.nY - 1));
+    }
+  }
   g.sync();
 }
 
