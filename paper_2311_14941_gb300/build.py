@@ -23,8 +23,9 @@ NVCC = os.environ.get("NVCC", "nvcc")
 # Registers per thread of the integration kernels: as many as they ask for (about 200; nine warps per SM, which
 # is what shared memory allows at 53 species).  Held to 168 or 128, the programs' ops that are read ahead spill: a
 # 4,096-cell jet field took 320 and 370 ms instead of 300, 6,000 small cells 371 (at 168) instead of 351.
-REG_CAP = {f: ["-maxrregcount=224"] for f in ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd_half")}
-CUDA_UNITS = ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd_half", "kern_rates",
+REG_CAP = {f: ["-maxrregcount=224"] for f in ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd_half",
+                                                    "kern_fwd_help", "kern_fwd_help_pair")}
+CUDA_UNITS = ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd_half", "kern_fwd_help", "kern_fwd_help_pair", "kern_rates",
               "kern_adjoint")
 HOST_UNITS = ("compile", "balance", "specialize")
 # device headers the run-time compiler sees, under the names integrate.cuh includes them by

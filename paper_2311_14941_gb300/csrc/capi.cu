@@ -66,6 +66,7 @@ struct chem_handle_s {
   int max_cells[kNumGroups] = {1, 1, 2};
   int default_cells[kNumGroups] = {1, 1, 2};
   int resident_cells[kNumGroups] = {0, 0, 0};
+  int helped_cells[kHelpForms] = {0, 0, 0};   // resident cells per SM of the kernels with helper warps (0: not used)
   int bps_cache[kNumGroups][kMaxBlockCells + 1] = {};   // resident blocks per SM of the persistent kernel
   int auto_wpc = 1;                // warps per cell when the caller leaves the choice to the library
   int auto_cpw = 1;                // cells per warp when the caller leaves the choice to the library
@@ -278,6 +279,26 @@ chem_status check_handle(chem_handle h, DeviceScope& ds) {
 
 int max_cells_per_block(const chem_handle h, int grp) { return h->max_cells[grp]; }
 
+constexpr int kHelpStatic = 256;   // bytes of a block's shared memory left for the helper's order
+static_assert(sizeof(HelpOrder) <= kHelpStatic, "the order of a block");
+
+// The kernel (an index of forward_kernel) for N cells of lane group grp in blocks of the library's choice: the one with
+// the most helper warps that still holds all cells at once (188 registers per thread: 8 warps per SM, so 2 cells with
+// three helpers, 4 with one).  Beyond that the helpers' registers would cost resident cells, and the FP64 pipe is
+// busy without them: held to 168 registers so that as many cells fit as without, a cell of two warps at 150 species
+// gains 1-2% (500 cells: 322 against 318 ms) where it gains 12% with room.  Only where every warp of the cell gets at
+// least two rounds of reactions (below): with the one or two rounds of 27 reactions there is nothing to share, and the
+// barriers cost 4% (304 cells of one warp each: 155 against 161 ms; two cells per warp gained 1%).
+int pick_kernel(const chem_handle h, int grp, int N) {
+  for (int i = kHelpForms - 1; i >= 0; --i)
+    if (kHelpGroups[i] == grp && N <= h->num_sms * h->helped_cells[i]) return kNumGroups + i;
+  return grp;
+}
+int kernel_threads(int kernel, int cells) {   // threads of a block
+  if (kernel < kNumGroups) return cells * kGroupWidth[kernel];
+  return kGroupWidth[kHelpGroups[kernel - kNumGroups]] + kHelpWarps[kernel - kNumGroups] * kWarp;
+}
+
 chem_status set_attrs(chem_handle h) {
   if (h->attr_set) return CHEM_OK;
   const int bytes = h->smem_optin;
@@ -285,10 +306,10 @@ chem_status set_attrs(chem_handle h) {
   if ((e = cudaFuncSetAttribute(k_rates, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(k_jacobian, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)
     return cuda_fail(e, "cudaFuncSetAttribute");
-  for (int grp = 0; grp < kNumGroups; ++grp)
+  for (int grp = 0; grp < kNumGroups + kHelpForms; ++grp)
     for (ForwardKernel kind : {KF_PLAIN, KF_PERSISTENT})
-      if ((e = cudaFuncSetAttribute(forward_kernel(kind, grp), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) !=
-          cudaSuccess)
+      if ((e = cudaFuncSetAttribute(forward_kernel(kind, grp), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    grp < kNumGroups ? bytes : bytes - kHelpStatic)) != cudaSuccess)
         return cuda_fail(e, "cudaFuncSetAttribute");
   h->L_rates = make_rates_layout(h->hm, h->L);
   auto fill = [&](const void* kernel, int cell_bytes, int most, int& cells) {   // ties: larger blocks (wider loads)
@@ -337,6 +358,16 @@ chem_status set_attrs(chem_handle h) {
     }
     h->default_cells[grp] = best_c;
     h->resident_cells[grp] = best_cells;
+  }
+  for (int i = 0; i < kHelpForms; ++i) {
+    const int warps = kernel_threads(kNumGroups + i, 1) / kWarp;
+    if (h->cell_bytes > bytes - kHelpStatic || (h->hm.R + kWarp - 1) / kWarp < 2 * warps) continue;
+    int blocks[2] = {0, 0};
+    for (ForwardKernel kind : {KF_PLAIN, KF_PERSISTENT})
+      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks[kind], forward_kernel(kind, kNumGroups + i),
+                                                             warps * kWarp, h->cell_bytes)) != cudaSuccess)
+        return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+    h->helped_cells[i] = std::min(blocks[KF_PLAIN], blocks[KF_PERSISTENT]);
   }
   // automatic choice: two warps per cell when one-warp cells leave fewer than 6 warps per SM (a cell
   // larger than ~35 KB of shared memory) and two-warp cells fit as many cells
@@ -426,7 +457,9 @@ struct IntCall {
   IntOpts io{};
   unsigned long long budget_ns = 0;
   int grp = 0;     // lane group: 0 one warp, 1 two warps, 2 half a warp per cell
+  int kernel = 0;  // lane group, or kNumGroups + i: the i-th kernel with helper warps
   int cpb = 1;     // cells per block
+  int threads = kWarp;   // threads per block
   int grid = 1;    // persistent form: resident blocks on the device
   int chunk = 1;   // persistent form: cells per queue pull
   int tab = 0;     // tabulated temperature functions
@@ -467,8 +500,15 @@ chem_status parse_integrate(chem_handle h, int N, const chem_integrate_opts* opt
   else c.grp = (o.warps_per_cell > 0 ? o.warps_per_cell : h->auto_wpc) - 1;
   c.cpb = cells_per_block(h, o.block_cells, c.grp);
   if (c.spec) c.cpb = std::min(c.cpb, h->spec_max_cells);
+  c.kernel = c.spec || o.block_cells != 0 ? c.grp : pick_kernel(h, c.grp, N);
   int bps = 1;
-  if ((st = persistent_blocks_per_sm(h, c.grp, c.cpb, bps, c.spec != 0)) != CHEM_OK) return st;
+  if (c.kernel >= kNumGroups) {
+    c.cpb = 1;
+    bps = h->helped_cells[c.kernel - kNumGroups];
+  } else if ((st = persistent_blocks_per_sm(h, c.grp, c.cpb, bps, c.spec != 0)) != CHEM_OK) {
+    return st;
+  }
+  c.threads = kernel_threads(c.kernel, c.cpb);
   c.grid = h->num_sms * bps;
   // a pull larger than an even share of the cells over the resident lane groups only leaves groups idle
   const long long groups = (long long)c.grid * c.cpb;
@@ -483,8 +523,8 @@ cudaError_t launch_plain(const chem_handle h, const IntCall& c, dim3 grid, dim3 
                          cudaStream_t strm, const MechView& V, int N, double* T, const double* p, double* Y,
                          const double* dt, double* h_io, int* nsub, int* status, const unsigned long long* stamp) {
   if (!c.spec)
-    return launch_integrate_plain(c.grp, grid, block, smem, strm, V, h->L, N, T, p, Y, dt, h_io, nsub, status,
-                                  c.o.naccept, c.io, stamp, c.budget_ns);
+    return launch_integrate_plain(c.kernel, grid, block, smem, strm, V, h->L, N, T, p, Y, dt, h_io, nsub,
+                                  status, c.o.naccept, c.io, stamp, c.budget_ns);
   if (block.x % kWarp != 0 || block.y != 1 || block.z != 1) return cudaErrorInvalidValue;
   MechView v = V;
   CellLayout L = h->L;
@@ -500,8 +540,8 @@ cudaError_t launch_persistent(const chem_handle h, const IntCall& c, dim3 grid, 
                               const double* dt, double* h_io, int* nsub, int* status, const int* perm,
                               unsigned long long* head, const unsigned long long* stamp) {
   if (!c.spec)
-    return launch_integrate_persistent(c.grp, grid, block, smem, strm, V, h->L, N, T, p, Y, dt, h_io, nsub, status,
-                                       c.o.naccept, perm, head, c.chunk, c.io, stamp, c.budget_ns);
+    return launch_integrate_persistent(c.kernel, grid, block, smem, strm, V, h->L, N, T, p, Y, dt, h_io,
+                                       nsub, status, c.o.naccept, perm, head, c.chunk, c.io, stamp, c.budget_ns);
   if (block.x % kWarp != 0 || block.y != 1 || block.z != 1) return cudaErrorInvalidValue;
   MechView v = V;
   CellLayout L = h->L;
@@ -881,7 +921,6 @@ chem_status chem_integrate(chem_handle h, int N, double* T, const double* p, dou
   cudaStream_t strm = (cudaStream_t)stream;
   cudaError_t e;
   const int grp = c.grp;
-  const int width = kGroupWidth[grp];
   if (c.tab && (st = ensure_tables(h, c.tab_tol, true)) != CHEM_OK) return st;
   const MechView V = view_for(h, grp, c.tab);
   const int cpb = c.cpb;
@@ -892,7 +931,7 @@ chem_status chem_integrate(chem_handle h, int N, double* T, const double* p, dou
       stamp = (unsigned long long*)((char*)h->scratch + kScrStamp);
       k_stamp<<<1, 32, 0, strm>>>(stamp);
     }
-    if ((e = launch_plain(h, c, (N + cpb - 1) / cpb, cpb * width, cpb * h->cell_bytes, strm, V, N, T, p, Y, dt, h_io,
+    if ((e = launch_plain(h, c, (N + cpb - 1) / cpb, c.threads, cpb * h->cell_bytes, strm, V, N, T, p, Y, dt, h_io,
                           nsub, status, stamp)) != cudaSuccess)
       return cuda_fail(e, "chem_integrate launch shape");
     return launch_check("chem_integrate launch");
@@ -907,7 +946,7 @@ chem_status chem_integrate(chem_handle h, int N, double* T, const double* p, dou
   for (int i = 0; i < 10; ++i) key.ptr[i] = ptrs[i];
   key.d[0] = io.rtol; key.d[1] = io.atol; key.d[2] = io.h_init; key.d[3] = io.h_min; key.d[4] = o.time_budget_s;
   key.i[0] = io.max_substeps; key.i[1] = io.max_nonfinite; key.i[2] = io.trace_cap; key.i[3] = io.method;
-  key.i[4] = c.tab + 2 * c.spec;
+  key.i[4] = c.tab + 2 * c.spec + 4 * c.kernel;
   key.d[5] = c.tab ? c.tab_tol : 0.0;
   if (!h->gexec || !(h->gkey == key)) {
     if (h->gexec) { cudaGraphExecDestroy(h->gexec); h->gexec = nullptr; }
@@ -928,7 +967,7 @@ chem_status chem_integrate(chem_handle h, int N, double* T, const double* p, dou
     k_stamp<<<1, 32, 0, cs>>>(stamp);
     k_sort_count<<<sblocks, 256, 0, cs>>>(N, nsub, counts);
     k_sort_scatter<<<sblocks, 256, 0, cs>>>(N, nsub, counts, cursor, perm);
-    const cudaError_t se = launch_persistent(h, c, grid, cpb * width, cpb * h->cell_bytes, cs, V, N, T, p, Y, dt,
+    const cudaError_t se = launch_persistent(h, c, grid, c.threads, cpb * h->cell_bytes, cs, V, N, T, p, Y, dt,
                                              h_io, nsub, status, perm, head, stamp);
     cudaGraph_t graph = nullptr;
     cudaError_t le = se != cudaSuccess ? se : cudaGetLastError();
@@ -1034,8 +1073,9 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
   // forward pass with the tape
   io.rec_h = rec_h; io.rec_ck = rec_ck; io.rec_n = rec_n; io.rec_cap = cap; io.rec_K = K;
   if ((e = cudaMemsetAsync(hio, 0, (size_t)N * 8, strm)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-  if ((e = launch_integrate_plain(0, N, kWarp, h->cell_bytes, strm, h->view[0], h->L, N, T, p, Y, dt, hio, nsub, status,
-                                  nullptr, io, nullptr, 0ull)) != cudaSuccess)
+  const int kernel = pick_kernel(h, 0, N);
+  if ((e = launch_integrate_plain(kernel, N, kernel_threads(kernel, 1), h->cell_bytes, strm, h->view[0], h->L, N,
+                                  T, p, Y, dt, hio, nsub, status, nullptr, io, nullptr, 0ull)) != cudaSuccess)
     return cuda_fail(e, "chem_adjoint forward launch shape");
   if ((st = launch_check("chem_adjoint forward launch")) != CHEM_OK) return st;
   // reverse pass, cells ordered by tape length (longest first) as in the sorted work queue
@@ -1115,7 +1155,7 @@ extern "C" chem_status chem_integrate_noalloc(chem_handle h, int N, double* T, c
   k_stamp<<<1, 32, 0, strm>>>(stamp);
   k_sort_count<<<sblocks, 256, 0, strm>>>(N, nsub, counts);
   k_sort_scatter<<<sblocks, 256, 0, strm>>>(N, nsub, counts, cursor, perm);
-  if ((e = launch_persistent(h, c, grid, wpb * kGroupWidth[grp], wpb * h->cell_bytes, strm, view_for(h, grp, c.tab),
+  if ((e = launch_persistent(h, c, grid, c.threads, wpb * h->cell_bytes, strm, view_for(h, grp, c.tab),
                              N, T, p, Y, dt, h_io, nsub, status, perm, head, stamp)) != cudaSuccess)
     return cuda_fail(e, "chem_integrate_noalloc launch shape");
   return launch_check("chem_integrate_noalloc launch");

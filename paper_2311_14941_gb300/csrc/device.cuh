@@ -954,6 +954,56 @@ __device__ __forceinline__ void eval_reactions(const MV& M, P s, const LT& L, co
   g.sync();
 }
 
+// One pass over the reactions (all of them in one for a right-hand side; for the Jacobian those whose slots fit).
+template <class MV, class P, class LT, class Sc, class Gp>
+__device__ __forceinline__ void eval_pass(const MV& M, P s, const LT& L, const ScalT<Sc>& sc, const Gp& g, int ps,
+                                          bool deriv) {
+  const int rb = deriv ? M.jpass[ps][JP_RB] : 0, re = deriv ? M.jpass[ps][JP_RE] : M.R;
+  const int cnt = M.jpass[ps][JP_CNT];
+  const ToCell<P> to{s, L.q, L.D - rb, L.D + cnt - M.jpass[ps][JP_SB]};
+  eval_reactions<Sc>(M, s, L, sc, g, rb, re, deriv, to);
+}
+
+// ---- helper warps.  With few cells a call takes as long as its longest cell's chain of attempts, and the chip is not
+// full.  Then a block holds one cell of one or two warps and some helper warps, which take their shares of its reaction
+// rounds and wait at the block's barrier for the rest of the time.  A reaction's results don't depend on the lane that
+// evaluates it, and sums and programs stay with the cell's own lanes, so the results are bit for bit those without the
+// helpers.  53 species / 325 reactions: the 11 rounds of a rate evaluation become 3 with three helpers, 6 with one; a
+// 10 us call takes 108 ms instead of 131 at 304 cells and 144 instead of 165 at 456 (RODAS4, 300 cells: 55 instead of
+// 71).  150 / 1000: with two helpers for a cell of two warps 255 ms instead of 284 at 100 cells, with three for a cell
+// of one warp 290 instead of 378 at 300.
+struct HelpOrder {   // what the helpers need to know besides the cell's memory
+  Scal sc;
+  int ps, deriv, more;   // more = 0: the cell's own warps have ended
+};
+__device__ __forceinline__ HelpOrder& help_order() {
+  __shared__ HelpOrder order;
+  return order;
+}
+template <class Gp, int H>
+struct GrpHelp {   // a cell's own lanes and its helpers
+  static constexpr int size = Gp::size + H * kWarp;
+  int lane;
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
+template <class Gp, int H>
+__device__ __forceinline__ bool wall(const GrpHelp<Gp, H>&, bool ok) { return __all_sync(0xffffffffu, ok); }
+template <class Gp, class MV, class LT>
+__device__ __forceinline__ void help(const MV& M, double* s, const LT& L) {
+  const HelpOrder& o = help_order();
+#pragma unroll 1
+  while (true) {
+    __syncthreads();
+    if (!o.more) return;
+    const Scal sc = o.sc;
+    eval_pass(M, s, L, sc, GrpHelp<Gp, MV::kHelpers>{(int)threadIdx.x}, o.ps, o.deriv != 0);   // ends with the block's barrier
+  }
+}
+__device__ __forceinline__ void help_end() {
+  if (threadIdx.x == 0) help_order().more = 0;
+  __syncthreads();
+}
+
 // -------------------------------------------------------------------------------------- f and J
 // The rates at y: C, h/RT, the rates of progress q and the production rates w_k into w[n].  With deriv also the
 // Y block of S (Dtil) and w_T in the T-column slots of S.  For those the reactions run in passes (see
@@ -971,10 +1021,19 @@ __device__ __forceinline__ ScalT<num<P>> eval_rates(const MV& M, P s, const LT& 
   const int passes = deriv ? M.n_jpass : 1;
 #pragma unroll 1
   for (int ps = 0; ps < passes; ++ps) {
-    const int rb = deriv ? M.jpass[ps][JP_RB] : 0, re = deriv ? M.jpass[ps][JP_RE] : M.R;
-    const int cnt = M.jpass[ps][JP_CNT];
-    const ToCell<P> to{s, L.q, L.D - rb, L.D + cnt - M.jpass[ps][JP_SB]};
-    eval_reactions<Sc>(M, s, L, sc, g, rb, re, deriv, to);
+    if constexpr (MV::kHelpers > 0) {
+      if (g.lane == 0) {
+        HelpOrder& o = help_order();
+        if (ps == 0) o.sc = sc;
+        o.ps = ps;
+        o.deriv = deriv;
+        o.more = 1;
+      }
+      __syncthreads();
+      eval_pass(M, s, L, sc, GrpHelp<Gp, MV::kHelpers>{g.lane}, ps, deriv);
+    } else {
+      eval_pass(M, s, L, sc, g, ps, deriv);
+    }
     if (deriv && ps == 0) gather_nu<false>(M.g_jac[0], sp + L.S, sp + L.part, sp + L.D, g);
     if (deriv && ps > 0) gather_nu<true>(M.g_jac[ps], sp + L.S, sp + L.part, sp + L.D, g);
   }

@@ -90,6 +90,13 @@ __device__ __forceinline__ void idle_state(double* s, const LT& L, int m, const 
   for (int i = g.lane; i < m; i += g.size) s[L.y + i] = i == 0 ? 1000.0 : 1.0 / (m - 1);
 }
 
+// Whole lane groups and whole warps; with helpers, one cell's warps and its helpers.
+template <class Gp, class MV>
+__device__ __forceinline__ bool block_shape() {
+  if (MV::kHelpers > 0) return blockDim.x == Gp::size + MV::kHelpers * kWarp;
+  return blockDim.x % Gp::size == 0 && blockDim.x % kWarp == 0;
+}
+
 // Plain form: one lane group per cell, cells in index order, one launch.
 template <class Gp, class MV = MechView, class LT = CellLayout>
 __global__ void k_integrate_plain(MV M, LT L, int N, double* __restrict__ T, const double* __restrict__ p,
@@ -97,13 +104,15 @@ __global__ void k_integrate_plain(MV M, LT L, int N, double* __restrict__ T, con
                                   int* __restrict__ nsub, int* __restrict__ status, int* __restrict__ nacc_out,
                                   IntOpts o, const unsigned long long* stamp, unsigned long long budget_ns) {
   extern __shared__ double smem[];
-  if (blockDim.x % Gp::size != 0 || blockDim.x % kWarp != 0) return;   // the launchers reject such shapes
-  const int cpb = blockDim.x / Gp::size;
+  if (!block_shape<Gp, MV>()) return;   // the launchers reject such shapes
+  const int cpb = MV::kHelpers > 0 ? 1 : blockDim.x / Gp::size;
   int w = 0;
   double* s = nullptr;
   const Gp g = cell_group<Gp>(L, smem, w, s);
   const int c0 = blockIdx.x * cpb;
   load_tile(smem, L, M.m, N, c0, cpb, T, Y);
+  if constexpr (MV::kHelpers > 0)
+    if (threadIdx.x >= Gp::size) return help<Gp>(M, smem, L);
   const int c = c0 + w;
   const IntOpts oo = with_deadline(o, stamp, budget_ns);
   CellRun r;
@@ -111,6 +120,7 @@ __global__ void k_integrate_plain(MV M, LT L, int N, double* __restrict__ T, con
   else idle_state(s, L, M.m, g);
   g.sync();
   while (any_cell(g, r.active)) cell_step(M, s, L, oo, g, r);
+  if constexpr (MV::kHelpers > 0) help_end();
   if (c < N) {
     cell_end(oo, g, r);
     store_cell(M, s, L, N, g, r, T, Y, h_io, nsub, status, nacc_out);
@@ -134,7 +144,9 @@ __global__ void k_integrate_persistent(MV M, LT L, int N, double* __restrict__ T
                                        unsigned long long* __restrict__ head, int chunk, IntOpts o,
                                        const unsigned long long* stamp, unsigned long long budget_ns) {
   extern __shared__ double smem[];
-  if (blockDim.x % Gp::size != 0 || blockDim.x % kWarp != 0) return;   // the launchers reject such shapes
+  if (!block_shape<Gp, MV>()) return;   // the launchers reject such shapes
+  if constexpr (MV::kHelpers > 0)
+    if (threadIdx.x >= Gp::size) return help<Gp>(M, smem, L);
   int w = 0;
   double* s = nullptr;
   const Gp g = cell_group<Gp>(L, smem, w, s);
@@ -172,6 +184,7 @@ __global__ void k_integrate_persistent(MV M, LT L, int N, double* __restrict__ T
       gs.sync();
     }
   }
+  if constexpr (MV::kHelpers > 0) help_end();
 }
 
 }  // namespace chemgb

@@ -19,7 +19,8 @@ __global__ void k_jacobian(MechView M, CellLayout L, int N, const double* __rest
 
 // The integration kernels are templates on the lane group (one warp, two warps or half a warp per cell);
 // their instantiations keep internal linkage inside their translation unit, so the ABI reaches them
-// through these host functions (group g: 0 one warp, 1 two warps, 2 half a warp per cell).
+// through these host functions (group g: 0 one warp, 1 two warps, 2 half a warp per cell; kNumGroups + i the
+// i-th kernel with helper warps).
 //   plain form: one lane group per cell, cells in index order;
 //   persistent form: resident lane groups pull `chunk` cells at a time from the sorted queue `perm`.
 enum ForwardKernel { KF_PLAIN = 0, KF_PERSISTENT = 1 };
@@ -36,16 +37,16 @@ cudaError_t launch_integrate_persistent(int g, dim3 grid, dim3 block, size_t sme
                                  const unsigned long long* stamp, unsigned long long budget_ns);
 
 // Per-group pieces, one translation unit each.
-template <class Gp>
+template <class Gp, class MV>
 const void* plain_kernel();
-template <class Gp>
+template <class Gp, class MV>
 const void* persistent_kernel();
-template <class Gp>
+template <class Gp, class MV>
 cudaError_t launch_plain_g(dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const MechView& M, const CellLayout& L,
                     int N, double* T, const double* p, double* Y, const double* dt, double* h_io, int* nsub,
                     int* status, int* nacc_out, const IntOpts& o, const unsigned long long* stamp,
                     unsigned long long budget_ns);
-template <class Gp>
+template <class Gp, class MV>
 cudaError_t launch_persistent_g(dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const MechView& M,
                          const CellLayout& L, int N, double* T, const double* p, double* Y, const double* dt,
                          double* h_io, int* nsub, int* status, int* nacc_out, const int* perm,

@@ -28,6 +28,11 @@ constexpr int kMaxWarpsPerCell = 2;   // a cell is integrated by one warp or by 
 //   group 0: one warp (32 lanes), group 1: two warps of a block (64 lanes), group 2: half a warp
 //   (16 lanes; two cells share a warp, for mechanisms with few species).
 constexpr int kNumGroups = 3;
+// Kernels with helper warps, numbered after the lane groups whose programs they run: kHelpWarps[i] helpers for a cell of
+// group kHelpGroups[i], those of a group with rising numbers of helpers.
+constexpr int kHelpForms = 3;
+constexpr int kHelpGroups[kHelpForms] = {0, 0, 1};
+constexpr int kHelpWarps[kHelpForms] = {1, 3, 2};
 constexpr int kGroupWidth[kNumGroups] = {32, 64, 16};
 
 // ---- species table, structure of arrays: field f of species k at sp[f * n + k], SP_STRIDE fields (lanes hold
@@ -130,6 +135,7 @@ constexpr int kMaxJPass = 8;
 enum : int { JP_RB = 0, JP_RE = 1, JP_SB = 2, JP_CNT = 3 };   // first/end reaction, first slot, reactions
 
 struct MechView {
+  static constexpr int kHelpers = 0;   // helper warps of a cell (HelpedView: kernels that have some)
   int width;                 // lanes of the programs below: the lane group's width (32, 64 or 16)
   int n, R, m;
   int n_troe, n_tb;          // reactions [0, n_troe) Troe, [n_troe, n_troe + n_tb) third-body
@@ -172,6 +178,12 @@ struct MechView {
   double tab_ulo, tab_du;    // interval j covers u = 1/T in [tab_ulo + j du, tab_ulo + (j + 1) du)
   double tab_tlo, tab_thi;   // tabulated range of T
   int tab_ni;                // intervals
+};
+
+// The same tables for the kernels whose cells have H helper warps.
+template <int H>
+struct HelpedView : MechView {
+  static constexpr int kHelpers = H;
 };
 
 // Per-cell shared-memory layout (offsets in doubles).
