@@ -46,7 +46,8 @@ struct AdjLayout {
   int UST;             // K * 4m: U1..U4 of every step of the current segment
   int SEG;             // K * m: the segment's states
   int GA, GE;          // R each: the cell's gradient accumulators (compiled reaction order)
-  int total;           // doubles per warp
+  int total;           // doubles per block
+  int GA2, GE2, second;   // with two warps: the second one's sums behind it (m doubles, GA, GE), and their size
 };
 
 // out = J^T w = S^T w + v (u . w) with S in the internal entry order
@@ -274,13 +275,13 @@ __device__ __forceinline__ void contract(const MechView& M, Sc* s, const CellLay
   g.sync();
 }
 
-// Second-order terms of kTangentsPerPass stages of one step: J(y)^T W_st differentiated along U_st, then the state
-// part into LAM and the parameter part into GA, GE.  cell: the dual-number cell (shared memory, which holds nothing
-// else then, or global); tmp: m doubles of scratch.
+// Second-order terms of kTangentsPerPass stages of one step: J(y)^T W_st differentiated along U_st, the state part into
+// out (m), the parameter part into GA, GE.  cell: the dual-number cell (shared memory, which holds nothing else then, or
+// global).
 __device__ __forceinline__ void second_order_terms(const MechView& M, ContractDual* cell, const CellLayout& Ld,
                                                    ContractVec* slots, const double* y, double p,
-                                                   const double* const* Us, const double* const* Ws, double* LAM,
-                                                   double* tmp, double* GA, double* GE, const Grp1& g) {
+                                                   const double* const* Us, const double* const* Ws, double* out,
+                                                   double* GA, double* GE, const Grp1& g) {
   ContractDual* yd = cell + Ld.y;
   for (int i = g.lane; i < M.m; i += g.size) {
     ContractDual x(y[i]);
@@ -289,15 +290,13 @@ __device__ __forceinline__ void second_order_terms(const MechView& M, ContractDu
     yd[i] = x;
   }
   g.sync();
-  contract<ContractDual>(M, cell, Ld, yd, p, Ws, slots, tmp, GA, GE, g);
-  for (int i = g.lane; i < M.m; i += g.size) LAM[i] += tmp[i];
-  g.sync();
+  contract<ContractDual>(M, cell, Ld, yd, p, Ws, slots, out, GA, GE, g);
 }
 
 // One adjoint step at state y with step h, whose stage vectors U1..U4 and step record jr (the Jacobian
-// at y and the factor of the step) the segment recompute kept.  lambda (A.LAM) is updated in place, the
-// parameter gradients accumulate into GA, GE.
-__device__ __forceinline__ void adjoint_step(const MechView& M, double* s, double* ws, const AdjLayout& A, double* ctr,
+// at y and the factor of the step) the segment recompute kept, up to the second-order terms.  lambda (A.LAM) is
+// updated in place, the parameter gradients accumulate into GA, GE; W1..W4 are left in the workspace.
+__device__ __forceinline__ void adjoint_stages(const MechView& M, double* s, double* ws, const AdjLayout& A, double* ctr,
                                              const double* jr, const double* y, const double* U1, const double* U2,
                                              const double* U3, const double* U4, double p, double h, double* GA,
                                              double* GE, const Grp1& g) {
@@ -372,35 +371,38 @@ __device__ __forceinline__ void adjoint_step(const MechView& M, double* s, doubl
   for (int i = g.lane; i < m; i += g.size) LAM[i] += G[i];
   g.sync();
   theta_terms(M, jr + A.HY, jr + A.QY, jr[A.SC], jr[A.SC + 1], jr[A.SC + 2], jr[A.SC + 3], WS, a, GA, GE, g);
-  // ---- Hessian and mixed parameter terms: J(y)^T w_i differentiated along U_i, kTangentsPerPass stages at a time
-  const double* Us[4] = {U1, U2, U3, U4};
-  const double* Ws[4] = {W1, W2, W3, W4};
-  ContractVec* slots = reinterpret_cast<ContractVec*>(ctr);
-  ContractDual* cell = A.dual_shared ? reinterpret_cast<ContractDual*>(s) : reinterpret_cast<ContractDual*>(slots + A.slots);
-#pragma unroll 1
-  for (int s0 = 0; s0 < 4; s0 += kTangentsPerPass)
-    second_order_terms(M, cell, A.Ld, slots, y, p, Us + s0, Ws + s0, LAM, G, GA, GE, g);
 }
 
-// Reverse pass of one cell from its tape.  ws: the warp's global workspace.  Returns false on a singular
-// factor.
+// Reverse pass of one cell from its tape.  ws, ctr: the block's global workspaces.  Returns false on a singular factor.
+// With two warps, warp 1 takes the second half of each step's second-order terms, which need only the step's state,
+// stage vectors and weights: its dual-number cell lies behind the first warp's shared memory, its sums behind the
+// first warp's workspace, and it waits at the block's barrier for the rest of the step.  Both warps run one copy of the
+// code.  53 species / 325 reactions, igniting cells to 2 us: 308 ms instead of 384 at 300 cells (two fifths of a step
+// are these terms), 455-472 instead of 480-490 at 600.
+template <int kWarps>
 __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, double* ws, const AdjLayout& A, double* ctr,
                                              double p, int n_acc, const double* rec_h, const double* rec_ck, int K,
-                                             int N, int cell, const Grp1& g, const IntOpts& o) {
+                                             int N, int cell, const Grp1& g, const IntOpts& o, int w) {
   const int m = M.m;
   const CellLayout& L = A.L;
   double* seg = ws + A.SEG;
   double* ust = ws + A.UST;
-  double* GA = ws + A.GA;
-  double* GE = ws + A.GE;
+  double* GA = w == 0 ? ws + A.GA : ws + A.total + A.GA2;
+  double* GE = w == 0 ? ws + A.GE : ws + A.total + A.GE2;
+  double* G = w == 0 ? ws + A.G : ws + A.total;
+  ContractVec* slots = reinterpret_cast<ContractVec*>(ctr + (size_t)w * A.ctr);
+  ContractDual* dual = A.dual_shared ? reinterpret_cast<ContractDual*>(s + (size_t)w * L.total)
+                                     : reinterpret_cast<ContractDual*>(slots + A.slots);
   const int nseg = (n_acc + K - 1) / K;
   for (int sg = nseg - 1; sg >= 0; --sg) {
     const int n0 = sg * K, n1 = min(n_acc, n0 + K);
-    for (int i = g.lane; i < m; i += g.size) seg[i] = rec_ck[((size_t)sg * m + i) * N + cell];
+    bool ok = true;
+    if (w == 0)
+      for (int i = g.lane; i < m; i += g.size) seg[i] = rec_ck[((size_t)sg * m + i) * N + cell];
     g.sync();
     // recompute the segment's states and stage vectors with the forward arithmetic, and keep each step's
     // Jacobian at y and its factor for the reverse sweep
-    for (int nn = n0; nn < n1; ++nn) {
+    for (int nn = n0; w == 0 && nn < n1; ++nn) {
       double* jr = ws + A.JREC + (size_t)(nn - n0) * A.jstride;
       vset(s + L.y, seg + (size_t)(nn - n0) * m, m, g);
       auto record = [&](const Scal& sy) {
@@ -414,7 +416,8 @@ __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, doubl
         }
       };
       const StepOut so = ros_attempt(M, s, L, p, rec_h[(size_t)nn * N + cell], o.rtol, o.atol, g, 0, true, record);
-      if (!so.good) return false;   // also a singular factor (cannot happen for a step the forward pass accepted)
+      ok = so.good;   // false also for a singular factor (cannot happen for a step the forward pass accepted)
+      if (!ok) break;
       vset(jr + A.LUG, s + L.LU, M.nnz_LU + m, g);
       double* u4 = ust + (size_t)(nn - n0) * 4 * m;
       for (int i = g.lane; i < m; i += g.size) {
@@ -423,10 +426,30 @@ __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, doubl
       }
       g.sync();
     }
+    if (kWarps > 1) ok = __syncthreads_and(ok);
+    if (!ok) return false;
     for (int nn = n1 - 1; nn >= n0; --nn) {
       const double* u4 = ust + (size_t)(nn - n0) * 4 * m;
-      adjoint_step(M, s, ws, A, ctr, ws + A.JREC + (size_t)(nn - n0) * A.jstride, seg + (size_t)(nn - n0) * m, u4,
-                   u4 + m, u4 + 2 * m, u4 + 3 * m, p, rec_h[(size_t)nn * N + cell], GA, GE, g);
+      const double* y = seg + (size_t)(nn - n0) * m;
+      double* LAM = ws + A.LAM;
+      if (w == 0)
+        adjoint_stages(M, s, ws, A, ctr, ws + A.JREC + (size_t)(nn - n0) * A.jstride, y, u4, u4 + m, u4 + 2 * m,
+                       u4 + 3 * m, p, rec_h[(size_t)nn * N + cell], GA, GE, g);
+      if (kWarps > 1) __syncthreads();
+      // Hessian and mixed parameter terms: J(y)^T w_i differentiated along U_i, kTangentsPerPass stages at a time
+      const double* Us[4] = {u4, u4 + m, u4 + 2 * m, u4 + 3 * m};
+      const double* Ws[4] = {ws + A.W1, ws + A.W2, ws + A.W3, ws + A.W4};
+#pragma unroll 1
+      for (int s0 = w * kTangentsPerPass; s0 < 4; s0 += kWarps * kTangentsPerPass) {
+        second_order_terms(M, dual, A.Ld, slots, y, p, Us + s0, Ws + s0, G, GA, GE, g);
+        if (kWarps > 1) __syncthreads();
+        if (w == 0)
+          for (int i = g.lane; i < m; i += g.size) {
+            LAM[i] += G[i];
+            if (kWarps > 1) LAM[i] += ws[A.total + i];
+          }
+        g.sync();
+      }
     }
   }
   return true;

@@ -177,6 +177,12 @@ AdjLayout make_adj_layout(const HostMech& hm, int K) {
     A.SC = rtake(8); A.LUG = rtake(hm.nnz_LU + m);
     A.jstride = r;
   }
+  {   // the second warp's sums, behind the first warp's workspace: the state part, GA, GE
+    auto round32 = [](int cnt) { return (cnt + 31) / 32 * 32; };
+    A.GA2 = round32(m);
+    A.GE2 = A.GA2 + round32(std::max(hm.R, 1));
+    A.second = A.GE2 + round32(std::max(hm.R, 1));
+  }
   A.JREC = take(K * A.jstride);
   A.UST = take(K * 4 * m);
   A.SEG = take(K * m);
@@ -1026,15 +1032,26 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
     return fail(CHEM_EUNSUPPORTED, "adjoint needs " + std::to_string(adj_bytes) + " bytes of shared memory per cell");
   cudaError_t e;
   if (!h->adj_attr_set) {
-    if ((e = cudaFuncSetAttribute(k_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin)) != cudaSuccess)
-      return cuda_fail(e, "cudaFuncSetAttribute");
+    for (int w : {1, 2})
+      if ((e = cudaFuncSetAttribute(adjoint_kernel(w), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    w == 1 ? h->smem_optin : h->smem_optin - kHelpStatic)) != cudaSuccess)
+        return cuda_fail(e, "cudaFuncSetAttribute");
     h->adj_attr_set = true;
   }
-  int bps = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_adjoint, kWarp, (size_t)adj_bytes)) != cudaSuccess)
-    return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+  // two warps per cell while all cells fit at once (255 registers: 8 warps per SM either way, so 4 cells instead of 8);
+  // beyond that the second warps would take the place of cells
+  int warps = 2, bps = 0, grid = 0;
+  size_t smem = 0;
+  for (; warps >= 1; --warps) {
+    smem = (size_t)adj_bytes + (warps > 1 && A.dual_shared ? A.dual_bytes : 0);
+    if (warps > 1 && smem > (size_t)(h->smem_optin - kHelpStatic)) continue;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, adjoint_kernel(warps), warps * kWarp, smem)) !=
+        cudaSuccess)
+      return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+    if (warps == 1 || N <= h->num_sms * bps) break;
+  }
   bps = std::max(bps, 1);
-  const int grid = std::min(h->num_sms * bps, N);
+  grid = std::min(h->num_sms * bps, N);
   // scratch: head, tape (h, checkpoints, counts), h_io/nsub of the forward pass, per-cell gradients,
   // contraction workspaces
   const size_t nck = (size_t)(cap / K + 1);
@@ -1045,8 +1062,8 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
   const size_t b_hio = align_up((size_t)N * 8, 256);
   const size_t b_ns = align_up((size_t)N * 4, 256);
   const size_t b_gc = grad_cell ? 0 : align_up((size_t)2 * hm.R * N * 8, 256);
-  const size_t b_dw = align_up((size_t)grid * A.ctr * sizeof(double), 256);
-  const size_t b_ww = align_up((size_t)grid * (size_t)A.total * 8, 256);
+  const size_t b_dw = align_up((size_t)grid * warps * A.ctr * sizeof(double), 256);
+  const size_t b_ww = align_up((size_t)grid * (size_t)(A.total + (warps - 1) * A.second) * 8, 256);
   const size_t need = b_head + b_rh + b_ck + b_rn + b_hio + b_ns + b_gc + b_dw + b_ww;
   if (need > h->adj_scratch_bytes) {
     if (h->adj_scratch) cudaFree(h->adj_scratch);
@@ -1088,8 +1105,9 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
   k_sort_count<<<sblocks, 256, 0, strm>>>(N, rec_n, (int*)(scr + kScrCounts));
   k_sort_scatter<<<sblocks, 256, 0, strm>>>(N, rec_n, (int*)(scr + kScrCounts), (int*)(scr + kScrCursor), perm);
   if ((e = cudaMemsetAsync(head, 0, 4, strm)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-  k_adjoint<<<grid, kWarp, adj_bytes, strm>>>(h->view[0], A, N, p, rec_h, rec_ck, rec_n, K, gT, gY, gcell, gT0, gY0,
-                                               status, head, perm, dws, wws, io);
+  if ((e = launch_adjoint(warps, grid, smem, strm, h->view[0], A, N, p, rec_h, rec_ck, rec_n, K, gT, gY, gcell, gT0, gY0,
+                          status, head, perm, dws, wws, io)) != cudaSuccess)
+    return cuda_fail(e, "chem_adjoint reverse launch shape");
   if ((st = launch_check("chem_adjoint reverse launch")) != CHEM_OK) return st;
   const int P = 2 * hm.R;
   if (P > 0) {

@@ -7,9 +7,10 @@
 
 namespace chemgb {
 
-// ---- discrete adjoint: resident warps pull cells (longest tapes first).  Shared memory: the forward cell
-// layout; each warp's workspace (AdjLayout offsets) and contraction workspace are in global memory.
-__global__ void __launch_bounds__(32, 8)
+// ---- discrete adjoint: resident blocks pull cells (longest tapes first).  Shared memory: the forward cell
+// layout; the workspaces (AdjLayout offsets) and contraction workspaces are in global memory.
+template <int kWarps>
+__global__ void __launch_bounds__(32 * kWarps, 8 / kWarps)
 k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const double* __restrict__ rec_h,
           const double* __restrict__ rec_ck, const int* __restrict__ rec_n, int K, const double* __restrict__ gT,
           const double* __restrict__ gY, double* __restrict__ grad_cell, double* __restrict__ gT0,
@@ -17,35 +18,47 @@ k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const do
           double* ctr_ws, double* warp_ws, IntOpts o) {
   extern __shared__ double smem[];
   const int lane = threadIdx.x % kWarp;
-  const int gw = blockIdx.x;   // one warp per block
+  const int gw = blockIdx.x, w = threadIdx.x / kWarp;   // one cell per block
   double* s = smem;
-  double* ctr = ctr_ws + (size_t)gw * A.ctr;
-  double* ws = warp_ws + (size_t)gw * A.total;
+  double* ctr = ctr_ws + (size_t)gw * kWarps * A.ctr;
+  double* ws = warp_ws + (size_t)gw * (A.total + (kWarps - 1) * A.second);
   const int m = M.m;
   double* LAM = ws + A.LAM;
-  double* GA = ws + A.GA;
-  double* GE = ws + A.GE;
+  double* GA = w == 0 ? ws + A.GA : ws + A.total + A.GA2;
+  double* GE = w == 0 ? ws + A.GE : ws + A.total + A.GE2;
   while (true) {
     int c = 0;
-    if (lane == 0) c = atomicAdd(head, 1);
+    if (threadIdx.x == 0) c = atomicAdd(head, 1);
     c = __shfl_sync(0xffffffffu, c, 0);
+    if (kWarps > 1) {
+      __shared__ int pulled;
+      __syncthreads();   // warp 0 has taken the other's sums of the cell before
+      if (threadIdx.x == 0) pulled = c;
+      __syncthreads();
+      c = pulled;
+    }
     if (c >= N) break;
     c = perm[c];   // costliest cells (longest tapes) first
     const int na = rec_n[c];
-    for (int i = lane; i < m; i += kWarp) LAM[i] = (i == 0) ? gT[c] : gY[(size_t)(i - 1) * N + c];
+    for (int i = lane; w == 0 && i < m; i += kWarp) LAM[i] = (i == 0) ? gT[c] : gY[(size_t)(i - 1) * N + c];
     for (int r = lane; r < M.R; r += kWarp) { GA[r] = 0.0; GE[r] = 0.0; }
     __syncwarp();
     bool ok = na >= 0;
-    if (ok) ok = adjoint_cell(M, s, ws, A, ctr, p[c], na, rec_h, rec_ck, K, N, c, Grp1{lane}, o);
+    if (ok) ok = adjoint_cell<kWarps>(M, s, ws, A, ctr, p[c], na, rec_h, rec_ck, K, N, c, Grp1{lane}, o, w);
     if (!ok) {
-      for (int i = lane; i < m; i += kWarp) LAM[i] = 0.0;
+      for (int i = lane; w == 0 && i < m; i += kWarp) LAM[i] = 0.0;
       for (int r = lane; r < M.R; r += kWarp) { GA[r] = 0.0; GE[r] = 0.0; }
       __syncwarp();
     }
+    if (kWarps > 1) {
+      __syncthreads();
+      if (w != 0) continue;
+    }
     for (int r = lane; r < M.R; r += kWarp) {
       const int d = __ldg(M.rx_order + r);
-      grad_cell[(size_t)d * N + c] = GA[r];
-      grad_cell[(size_t)(M.R + d) * N + c] = GE[r];
+      const bool two = kWarps > 1;
+      grad_cell[(size_t)d * N + c] = two ? GA[r] + ws[A.total + A.GA2 + r] : GA[r];
+      grad_cell[(size_t)(M.R + d) * N + c] = two ? GE[r] + ws[A.total + A.GE2 + r] : GE[r];
     }
     if (gT0 && lane == 0) gT0[c] = LAM[0];
     if (gY0)
@@ -53,6 +66,18 @@ k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const do
     if (status && lane == 0 && !ok && status[c] == CHEM_CELL_OK) status[c] = CHEM_CELL_NOTAPE;
     __syncwarp();
   }
+}
+
+const void* adjoint_kernel(int warps) { return warps == 1 ? (const void*)k_adjoint<1> : (const void*)k_adjoint<2>; }
+
+cudaError_t launch_adjoint(int warps, int grid, size_t smem, cudaStream_t stream, const MechView& M, const AdjLayout& A,
+                           int N, const double* p, const double* rec_h, const double* rec_ck, const int* rec_n, int K,
+                           const double* gT, const double* gY, double* grad_cell, double* gT0, double* gY0, int* status,
+                           int* head, const int* perm, double* ctr_ws, double* warp_ws, const IntOpts& o) {
+  const auto k = warps == 1 ? k_adjoint<1> : k_adjoint<2>;
+  k<<<grid, warps * kWarp, smem, stream>>>(M, A, N, p, rec_h, rec_ck, rec_n, K, gT, gY, grad_cell, gT0, gY0, status,
+                                           head, perm, ctr_ws, warp_ws, o);
+  return cudaSuccess;
 }
 
 // sums over cells in a fixed order (one warp per parameter): deterministic gradients

@@ -53,15 +53,14 @@ cudaError_t launch_persistent_g(dim3 grid, dim3 block, size_t smem, cudaStream_t
                          unsigned long long* head, int chunk, const IntOpts& o, const unsigned long long* stamp,
                          unsigned long long budget_ns);
 
-// Discrete adjoint: resident warps (one per block) pull cells, longest tapes first; shared memory holds the
-// forward cell layout, each warp's workspace (A.total doubles) and contraction workspace (A.ctr) are in
-// global memory.
-__global__ void k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const double* __restrict__ rec_h,
-                          const double* __restrict__ rec_ck, const int* __restrict__ rec_n, int K,
-                          const double* __restrict__ gT, const double* __restrict__ gY, double* __restrict__ grad_cell,
-                          double* __restrict__ gT0, double* __restrict__ gY0, int* __restrict__ status,
-                          int* __restrict__ head, const int* __restrict__ perm, double* ctr_ws, double* warp_ws,
-                          IntOpts o);
+// Discrete adjoint: resident blocks of one or two warps pull one cell at a time, longest tapes first; shared memory
+// holds the forward cell layout (with two warps, a second dual-number cell behind it), a block's workspace (A.total
+// doubles, A.second more for the second warp) and contraction workspaces (A.ctr per warp) are in global memory.
+const void* adjoint_kernel(int warps);
+cudaError_t launch_adjoint(int warps, int grid, size_t smem, cudaStream_t stream, const MechView& M, const AdjLayout& A,
+                           int N, const double* p, const double* rec_h, const double* rec_ck, const int* rec_n, int K,
+                           const double* gT, const double* gY, double* grad_cell, double* gT0, double* gY0, int* status,
+                           int* head, const int* perm, double* ctr_ws, double* warp_ws, const IntOpts& o);
 
 __global__ void k_grad_reduce(int N, int P, const double* __restrict__ grad_cell, double* __restrict__ out1,
                               double* __restrict__ out2, int half);
