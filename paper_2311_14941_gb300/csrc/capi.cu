@@ -376,8 +376,10 @@ chem_status set_attrs(chem_handle h) {
     h->helped_cells[i] = std::min(blocks[KF_PLAIN], blocks[KF_PERSISTENT]);
   }
   // automatic choice: two warps per cell when one-warp cells leave fewer than 6 warps per SM (a cell
-  // larger than ~35 KB of shared memory) and two-warp cells fit as many cells
-  h->auto_wpc = (h->resident_cells[0] < 6 && h->resident_cells[1] >= h->resident_cells[0]) ? 2 : 1;
+  // larger than ~38 KB of shared memory) and two-warp cells bring more lanes (registers hold at most four two-warp
+  // cells: 8 warps against the 5 of one-warp cells of 39 to 46 KB).  One against two warps per cell, queue: 90 / 600 at
+  // 600 cells 103 and 91 ms, at 1,200 136 and 102, at 6,000 133 and 108; 100 / 650 at 3,000 cells 510 and 431 ms.
+  h->auto_wpc = (h->resident_cells[0] < 6 && 2 * h->resident_cells[1] > h->resident_cells[0]) ? 2 : 1;
   // two cells per warp for mechanisms whose species loops fit half a warp, unless shared memory would
   // then hold fewer cells per SM
   h->auto_cpw = (h->hm.n <= 16 && h->resident_cells[2] >= h->resident_cells[0]) ? 2 : 1;
