@@ -233,6 +233,19 @@ const char* chem_last_error(void);
 
 chem_status chem_info(chem_handle h, chem_info_t* info);
 
+/* The launch shape that calls with N cells and these options (NULL: all defaults) take on the handle's device.
+   helper_warps: warps beside a cell's own that only evaluate reaction rates (calls with few cells and block_cells
+   0; they change no bit of the results); adjoint_*: chem_adjoint's forward and reverse pass.  Errors as
+   chem_integrate; CHEM_EINVAL for a host-only handle. */
+typedef struct {
+  int warps_per_cell, cells_per_warp;   /* of chem_integrate and chem_integrate_noalloc */
+  int helper_warps;                     /* per cell */
+  int block_cells;                      /* cells per block */
+  int adjoint_helper_warps;             /* forward pass of chem_adjoint: helper warps per cell */
+  int adjoint_warps;                    /* reverse pass: warps per cell, 1 or 2 */
+} chem_launch_t;
+chem_status chem_launch_shape(chem_handle h, int N, const chem_integrate_opts* opts, chem_launch_t* out);
+
 /* The static pattern of S in natural state order (0 = T, 1 + k = Y_k), CSR, HOST arrays:
    row_ptr [m+1], col_idx [nnz_S]. Entry e of chem_jacobian's S_vals is (row of e, col_idx[e]). */
 chem_status chem_jacobian_pattern(chem_handle h, int* row_ptr, int* col_idx);

@@ -52,6 +52,11 @@ class OptsC(C.Structure):
                 ("tabulate", C.c_int), ("tab_tol", C.c_double), ("specialized", C.c_int)]
 
 
+class LaunchC(C.Structure):
+    _fields_ = [(f, C.c_int) for f in ("warps_per_cell", "cells_per_warp", "helper_warps", "block_cells",
+                                       "adjoint_helper_warps", "adjoint_warps")]
+
+
 class MapOptsC(C.Structure):
     _fields_ = [("T_max", C.c_double), ("dT", C.c_double), ("n_species", C.c_int), ("species", C.c_int * 8),
                 ("dY", C.c_double * 8)]
@@ -79,6 +84,7 @@ def lib():
         L.chem_destroy.argtypes = [_vp]
         L.chem_last_error.restype = C.c_char_p
         L.chem_info.argtypes = [_vp, C.POINTER(InfoC)]
+        L.chem_launch_shape.argtypes = [_vp, C.c_int, C.POINTER(OptsC), C.POINTER(LaunchC)]
         L.chem_jacobian_pattern.argtypes = [_vp, _ip, _ip]
         L.chem_export_plan.argtypes = [_vp, C.c_int, _ip, _ip]
         L.chem_rates.argtypes = [_vp, C.c_int, _vp, _vp, _vp, _vp, _vp, _vp, _vp]
@@ -190,6 +196,12 @@ class Mechanism:
             v = getattr(inf, f)
             out[f] = list(v) if hasattr(v, "__len__") else v
         return out
+
+    def launch_shape(self, n_cells, **options) -> dict:
+        """chem_launch_shape: the launch shape of calls with n_cells cells; options: chem_integrate_opts fields."""
+        o, out = OptsC(**options), LaunchC()
+        _check(lib().chem_launch_shape(self._h, n_cells, C.byref(o), C.byref(out)), "chem_launch_shape")
+        return {f: getattr(out, f) for f, _ in LaunchC._fields_}
 
     def jacobian_pattern(self):
         m, nnz = self.info["n_state"], self.info["nnz_S"]

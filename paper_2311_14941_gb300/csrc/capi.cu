@@ -1004,6 +1004,38 @@ extern "C" chem_status chem_set_params(chem_handle h, const double* dlnA, const 
   return launch_check("chem_set_params launch");
 }
 
+namespace {
+// The reverse pass for N cells: two warps per cell while all cells fit at once (255 registers: 8 warps per SM either
+// way, so 4 cells instead of 8); beyond that the second warps would take the place of cells.
+struct AdjShape {
+  int warps = 0, blocks_per_sm = 0;
+  size_t smem = 0;
+};
+chem_status adjoint_shape(chem_handle h, int N, const AdjLayout& A, AdjShape& s) {
+  const int adj_bytes = A.L.total * (int)sizeof(double);
+  if (adj_bytes > h->smem_optin)
+    return fail(CHEM_EUNSUPPORTED, "adjoint needs " + std::to_string(adj_bytes) + " bytes of shared memory per cell");
+  cudaError_t e;
+  if (!h->adj_attr_set) {
+    for (int w : {1, 2})
+      if ((e = cudaFuncSetAttribute(adjoint_kernel(w), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    w == 1 ? h->smem_optin : h->smem_optin - kHelpStatic)) != cudaSuccess)
+        return cuda_fail(e, "cudaFuncSetAttribute");
+    h->adj_attr_set = true;
+  }
+  for (s.warps = 2; s.warps >= 1; --s.warps) {
+    s.smem = (size_t)adj_bytes + (s.warps > 1 && A.dual_shared ? A.dual_bytes : 0);
+    if (s.warps > 1 && s.smem > (size_t)(h->smem_optin - kHelpStatic)) continue;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s.blocks_per_sm, adjoint_kernel(s.warps), s.warps * kWarp,
+                                                           s.smem)) != cudaSuccess)
+      return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+    if (s.warps == 1 || N <= h->num_sms * s.blocks_per_sm) break;
+  }
+  s.blocks_per_sm = std::max(s.blocks_per_sm, 1);
+  return CHEM_OK;
+}
+}  // namespace
+
 extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const double* p, double* Y, const double* dt,
                                     const double* gT, const double* gY, double* grad_lnA, double* grad_Ea,
                                     double* grad_cell, double* gT0, double* gY0, int* status,
@@ -1029,31 +1061,12 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
   const HostMech& hm = h->hm;
   const int m = hm.m;
   const AdjLayout A = make_adj_layout(hm, K);
-  const int adj_bytes = A.L.total * (int)sizeof(double);
-  if (adj_bytes > h->smem_optin)
-    return fail(CHEM_EUNSUPPORTED, "adjoint needs " + std::to_string(adj_bytes) + " bytes of shared memory per cell");
   cudaError_t e;
-  if (!h->adj_attr_set) {
-    for (int w : {1, 2})
-      if ((e = cudaFuncSetAttribute(adjoint_kernel(w), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    w == 1 ? h->smem_optin : h->smem_optin - kHelpStatic)) != cudaSuccess)
-        return cuda_fail(e, "cudaFuncSetAttribute");
-    h->adj_attr_set = true;
-  }
-  // two warps per cell while all cells fit at once (255 registers: 8 warps per SM either way, so 4 cells instead of 8);
-  // beyond that the second warps would take the place of cells
-  int warps = 2, bps = 0, grid = 0;
-  size_t smem = 0;
-  for (; warps >= 1; --warps) {
-    smem = (size_t)adj_bytes + (warps > 1 && A.dual_shared ? A.dual_bytes : 0);
-    if (warps > 1 && smem > (size_t)(h->smem_optin - kHelpStatic)) continue;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, adjoint_kernel(warps), warps * kWarp, smem)) !=
-        cudaSuccess)
-      return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    if (warps == 1 || N <= h->num_sms * bps) break;
-  }
-  bps = std::max(bps, 1);
-  grid = std::min(h->num_sms * bps, N);
+  AdjShape shape;
+  if ((st = adjoint_shape(h, N, A, shape)) != CHEM_OK) return st;
+  const int warps = shape.warps;
+  const size_t smem = shape.smem;
+  const int grid = std::min(h->num_sms * shape.blocks_per_sm, N);
   // scratch: head, tape (h, checkpoints, counts), h_io/nsub of the forward pass, per-cell gradients,
   // contraction workspaces
   const size_t nck = (size_t)(cap / K + 1);
@@ -1116,6 +1129,24 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
     k_grad_reduce<<<(P * kWarp + 255) / 256, 256, 0, strm>>>(N, P, gcell, grad_lnA, grad_Ea, hm.R);
     if ((st = launch_check("chem_adjoint reduction launch")) != CHEM_OK) return st;
   }
+  return CHEM_OK;
+}
+
+extern "C" chem_status chem_launch_shape(chem_handle h, int N, const chem_integrate_opts* opts, chem_launch_t* out) {
+  DeviceScope ds;
+  chem_status st = check_handle(h, ds);
+  if (st != CHEM_OK) return st;
+  if (!out) return fail(CHEM_EINVAL, "null argument");
+  if (N < 0) return fail(CHEM_EINVAL, "N must be >= 0");
+  IntCall c;
+  if ((st = parse_integrate(h, N, opts, c)) != CHEM_OK) return st;
+  const int K = opts && opts->ckpt_every > 0 ? opts->ckpt_every : 16;
+  AdjShape a;
+  if ((st = adjoint_shape(h, N, make_adj_layout(h->hm, K), a)) != CHEM_OK) return st;
+  const int fwd = pick_kernel(h, 0, N);
+  *out = chem_launch_t{kGroupWidth[c.grp] > kWarp ? 2 : 1, c.grp == 2 ? 2 : 1,
+                       c.kernel < kNumGroups ? 0 : kHelpWarps[c.kernel - kNumGroups], c.cpb,
+                       fwd < kNumGroups ? 0 : kHelpWarps[fwd - kNumGroups], a.warps};
   return CHEM_OK;
 }
 
