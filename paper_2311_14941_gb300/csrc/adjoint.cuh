@@ -47,7 +47,9 @@ struct AdjLayout {
   int SEG;             // K * m: the segment's states
   int GA, GE;          // R each: the cell's gradient accumulators (compiled reaction order)
   int total;           // doubles per block
-  int GA2, GE2, second;   // with two warps: the second one's sums behind it (m doubles, GA, GE), and their size
+  // sums of the second half of the second-order terms, behind it (m doubles, GA, GE), and their size: apart from the
+  // first half's with one warp per cell as with two, so that a cell's gradient does not depend on how many cells a call has
+  int GA2, GE2, second;
 };
 
 // out = J^T w = S^T w + v (u . w) with S in the internal entry order
@@ -387,9 +389,7 @@ __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, doubl
   const CellLayout& L = A.L;
   double* seg = ws + A.SEG;
   double* ust = ws + A.UST;
-  double* GA = w == 0 ? ws + A.GA : ws + A.total + A.GA2;
-  double* GE = w == 0 ? ws + A.GE : ws + A.total + A.GE2;
-  double* G = w == 0 ? ws + A.G : ws + A.total;
+  double* ws2 = ws + A.total;   // the sums of the second half of the second-order terms
   ContractVec* slots = reinterpret_cast<ContractVec*>(ctr + (size_t)w * A.ctr);
   ContractDual* dual = A.dual_shared ? reinterpret_cast<ContractDual*>(s + (size_t)w * L.total)
                                      : reinterpret_cast<ContractDual*>(slots + A.slots);
@@ -434,19 +434,21 @@ __device__ __forceinline__ bool adjoint_cell(const MechView& M, double* s, doubl
       double* LAM = ws + A.LAM;
       if (w == 0)
         adjoint_stages(M, s, ws, A, ctr, ws + A.JREC + (size_t)(nn - n0) * A.jstride, y, u4, u4 + m, u4 + 2 * m,
-                       u4 + 3 * m, p, rec_h[(size_t)nn * N + cell], GA, GE, g);
+                       u4 + 3 * m, p, rec_h[(size_t)nn * N + cell], ws + A.GA, ws + A.GE, g);
       if (kWarps > 1) __syncthreads();
       // Hessian and mixed parameter terms: J(y)^T w_i differentiated along U_i, kTangentsPerPass stages at a time
       const double* Us[4] = {u4, u4 + m, u4 + 2 * m, u4 + 3 * m};
       const double* Ws[4] = {ws + A.W1, ws + A.W2, ws + A.W3, ws + A.W4};
 #pragma unroll 1
       for (int s0 = w * kTangentsPerPass; s0 < 4; s0 += kWarps * kTangentsPerPass) {
-        second_order_terms(M, dual, A.Ld, slots, y, p, Us + s0, Ws + s0, G, GA, GE, g);
+        double* G = s0 == 0 ? ws + A.G : ws2;
+        second_order_terms(M, dual, A.Ld, slots, y, p, Us + s0, Ws + s0, G, s0 == 0 ? ws + A.GA : ws2 + A.GA2,
+                           s0 == 0 ? ws + A.GE : ws2 + A.GE2, g);
         if (kWarps > 1) __syncthreads();
         if (w == 0)
           for (int i = g.lane; i < m; i += g.size) {
             LAM[i] += G[i];
-            if (kWarps > 1) LAM[i] += ws[A.total + i];
+            if (kWarps > 1) LAM[i] += ws2[i];
           }
         g.sync();
       }

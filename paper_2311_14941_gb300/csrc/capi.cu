@@ -177,7 +177,7 @@ AdjLayout make_adj_layout(const HostMech& hm, int K) {
     A.SC = rtake(8); A.LUG = rtake(hm.nnz_LU + m);
     A.jstride = r;
   }
-  {   // the second warp's sums, behind the first warp's workspace: the state part, GA, GE
+  {   // the second half's sums, behind the workspace: the state part, GA, GE
     auto round32 = [](int cnt) { return (cnt + 31) / 32 * 32; };
     A.GA2 = round32(m);
     A.GE2 = A.GA2 + round32(std::max(hm.R, 1));
@@ -1078,7 +1078,7 @@ extern "C" chem_status chem_adjoint(chem_handle h, int N, double* T, const doubl
   const size_t b_ns = align_up((size_t)N * 4, 256);
   const size_t b_gc = grad_cell ? 0 : align_up((size_t)2 * hm.R * N * 8, 256);
   const size_t b_dw = align_up((size_t)grid * warps * A.ctr * sizeof(double), 256);
-  const size_t b_ww = align_up((size_t)grid * (size_t)(A.total + (warps - 1) * A.second) * 8, 256);
+  const size_t b_ww = align_up((size_t)grid * (size_t)(A.total + A.second) * 8, 256);
   const size_t need = b_head + b_rh + b_ck + b_rn + b_hio + b_ns + b_gc + b_dw + b_ww;
   if (need > h->adj_scratch_bytes) {
     if (h->adj_scratch) cudaFree(h->adj_scratch);

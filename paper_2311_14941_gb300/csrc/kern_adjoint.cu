@@ -21,11 +21,20 @@ k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const do
   const int gw = blockIdx.x, w = threadIdx.x / kWarp;   // one cell per block
   double* s = smem;
   double* ctr = ctr_ws + (size_t)gw * kWarps * A.ctr;
-  double* ws = warp_ws + (size_t)gw * (A.total + (kWarps - 1) * A.second);
+  double* ws = warp_ws + (size_t)gw * (A.total + A.second);
   const int m = M.m;
   double* LAM = ws + A.LAM;
-  double* GA = w == 0 ? ws + A.GA : ws + A.total + A.GA2;
-  double* GE = w == 0 ? ws + A.GE : ws + A.total + A.GE2;
+  double* GA = ws + A.GA;
+  double* GE = ws + A.GE;
+  double* GA2 = ws + A.total + A.GA2;
+  double* GE2 = ws + A.total + A.GE2;
+  auto clear = [&]() {   // every warp its own sums; one warp both
+    if (w == 0)
+      for (int r = lane; r < M.R; r += kWarp) { GA[r] = 0.0; GE[r] = 0.0; }
+    if (w == kWarps - 1)
+      for (int r = lane; r < M.R; r += kWarp) { GA2[r] = 0.0; GE2[r] = 0.0; }
+    __syncwarp();
+  };
   while (true) {
     int c = 0;
     if (threadIdx.x == 0) c = atomicAdd(head, 1);
@@ -41,14 +50,12 @@ k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const do
     c = perm[c];   // costliest cells (longest tapes) first
     const int na = rec_n[c];
     for (int i = lane; w == 0 && i < m; i += kWarp) LAM[i] = (i == 0) ? gT[c] : gY[(size_t)(i - 1) * N + c];
-    for (int r = lane; r < M.R; r += kWarp) { GA[r] = 0.0; GE[r] = 0.0; }
-    __syncwarp();
+    clear();
     bool ok = na >= 0;
     if (ok) ok = adjoint_cell<kWarps>(M, s, ws, A, ctr, p[c], na, rec_h, rec_ck, K, N, c, Grp1{lane}, o, w);
     if (!ok) {
       for (int i = lane; w == 0 && i < m; i += kWarp) LAM[i] = 0.0;
-      for (int r = lane; r < M.R; r += kWarp) { GA[r] = 0.0; GE[r] = 0.0; }
-      __syncwarp();
+      clear();
     }
     if (kWarps > 1) {
       __syncthreads();
@@ -56,9 +63,8 @@ k_adjoint(MechView M, AdjLayout A, int N, const double* __restrict__ p, const do
     }
     for (int r = lane; r < M.R; r += kWarp) {
       const int d = __ldg(M.rx_order + r);
-      const bool two = kWarps > 1;
-      grad_cell[(size_t)d * N + c] = two ? GA[r] + ws[A.total + A.GA2 + r] : GA[r];
-      grad_cell[(size_t)(M.R + d) * N + c] = two ? GE[r] + ws[A.total + A.GE2 + r] : GE[r];
+      grad_cell[(size_t)d * N + c] = GA[r] + GA2[r];
+      grad_cell[(size_t)(M.R + d) * N + c] = GE[r] + GE2[r];
     }
     if (gT0 && lane == 0) gT0[c] = LAM[0];
     if (gY0)

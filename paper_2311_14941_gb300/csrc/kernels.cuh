@@ -55,7 +55,7 @@ cudaError_t launch_persistent_g(dim3 grid, dim3 block, size_t smem, cudaStream_t
 
 // Discrete adjoint: resident blocks of one or two warps pull one cell at a time, longest tapes first; shared memory
 // holds the forward cell layout (with two warps, a second dual-number cell behind it), a block's workspace (A.total
-// doubles, A.second more for the second warp) and contraction workspaces (A.ctr per warp) are in global memory.
+// doubles, then A.second for the sums of the second half of the second-order terms) and contraction workspaces (A.ctr per warp) are in global memory.
 const void* adjoint_kernel(int warps);
 cudaError_t launch_adjoint(int warps, int grid, size_t smem, cudaStream_t stream, const MechView& M, const AdjLayout& A,
                            int N, const double* p, const double* rec_h, const double* rec_ck, const int* rec_n, int K,

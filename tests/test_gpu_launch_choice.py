@@ -2,9 +2,9 @@
 cell in the reverse pass of the adjoint.  The counts at which it changes are found by asking the library
 (chem_launch_shape), so the runs compared on either side are known to take different kernels.
 
-Helper warps change no bit of a result (tolerance 0).  The reverse pass with one and with two warps adds the same terms to
-the state's adjoint in the same order: final states and initial-state gradients agree bit for bit; the parameter
-gradients to 1e-10 of the cell's largest (up to 4,096 steps of 4 contributions: 2^14 x 2^-53 = 2e-12).
+Neither choice may change a bit of a result (tolerance 0): helper warps only evaluate reactions, and the reverse pass adds
+the same terms in the same order with one warp as with two, so that a cell's gradient does not depend on how a field is
+split over calls.
 """
 import numpy as np
 import pytest
@@ -49,7 +49,7 @@ def test_helpers_up_to_where_all_cells_fit(mech, wpc, forms):
                     assert np.array_equal(x, y, equal_nan=True)
 
 
-@pytest.mark.parametrize("mech,n_cells,dt", [("small", 7, 1e-7), ("methane", 33, 3e-8), ("large", 5, 3e-9)])
+@pytest.mark.parametrize("mech,n_cells,dt", [("small", 7, 1e-7), ("methane", 33, 2e-7), ("large", 5, 2e-8)])
 def test_reverse_pass_where_two_warps_no_longer_fit(mech, n_cells, dt):
     m = MECH[mech]()
     h = chem.create(m, 0)
@@ -61,9 +61,5 @@ def test_reverse_pass_where_two_warps_no_longer_fit(mech, n_cells, dt):
     rep = np.arange(edge + 1) % n_cells
     one = _adjoint(h, F.T[rep], F.p[rep], F.Y[:, rep], F.dt[rep], gT[rep], gY[:, rep])
     two = _adjoint(h, F.T, F.p, F.Y, F.dt, gT, gY)
-    for a, b in zip(two[:5], one[:5]):
+    for a, b in zip(two, one):
         assert np.array_equal(a, b[..., :n_cells], equal_nan=True)
-    for c in range(n_cells):
-        a, b = two[5][:, c], one[5][:, c]
-        for half in (slice(0, h.R), slice(h.R, 2 * h.R)):
-            assert np.max(np.abs(a[half] - b[half])) <= 1e-10 * np.max(np.abs(b[half])), c
