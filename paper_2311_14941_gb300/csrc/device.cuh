@@ -966,7 +966,7 @@ __device__ __forceinline__ void eval_pass(const MV& M, P s, const LT& L, const S
 
 // ---- helper warps.  With few cells a call takes as long as its longest cell's chain of attempts, and the chip is not
 // full.  Then a block holds one cell of one or two warps and some helper warps, which take their shares of its reaction
-// rounds and wait at the block's barrier for the rest of the time.  A reaction's results don't depend on the lane that
+// rounds and wait at their common barrier for the rest of the time.  A reaction's results don't depend on the lane that
 // evaluates it, and sums and programs stay with the cell's own lanes, so the results are bit for bit those without the
 // helpers.  53 species / 325 reactions: the 11 rounds of a rate evaluation become 3 with three helpers, 6 with one; a
 // 10 us call takes 108 ms instead of 131 at 304 cells and 144 instead of 165 at 456 (RODAS4, 300 cells: 55 instead of
@@ -980,28 +980,37 @@ __device__ __forceinline__ HelpOrder& help_order() {
   __shared__ HelpOrder order;
   return order;
 }
+// A cell's own lanes and its helpers.  They meet at a named barrier with their number spelt out, because they come to it
+// from different places (the helpers from their loop, the cell's warps from its rate evaluations), which
+// __syncthreads() does not allow for.  (Barrier 0 is __syncthreads(), 1 a two-warp cell's own.)
 template <class Gp, int H>
-struct GrpHelp {   // a cell's own lanes and its helpers
+struct GrpHelp {
   static constexpr int size = Gp::size + H * kWarp;
+  static constexpr int bar = 2;
   int lane;
-  __device__ __forceinline__ void sync() const { __syncthreads(); }
+  __device__ __forceinline__ void sync() const {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"n"(bar), "n"(size) : "memory");
+  }
 };
 template <class Gp, int H>
 __device__ __forceinline__ bool wall(const GrpHelp<Gp, H>&, bool ok) { return __all_sync(0xffffffffu, ok); }
 template <class Gp, class MV, class LT>
 __device__ __forceinline__ void help(const MV& M, double* s, const LT& L) {
   const HelpOrder& o = help_order();
+  const GrpHelp<Gp, MV::kHelpers> g{(int)threadIdx.x};
 #pragma unroll 1
   while (true) {
-    __syncthreads();
+    g.sync();
     if (!o.more) return;
     const Scal sc = o.sc;
-    eval_pass(M, s, L, sc, GrpHelp<Gp, MV::kHelpers>{(int)threadIdx.x}, o.ps, o.deriv != 0);   // ends with the block's barrier
+    eval_pass(M, s, L, sc, g, o.ps, o.deriv != 0);   // ends with a barrier of the group
   }
 }
+template <class Gp, int H>
 __device__ __forceinline__ void help_end() {
   if (threadIdx.x == 0) help_order().more = 0;
-  __syncthreads();
+  GrpHelp<Gp, H>{(int)threadIdx.x}.sync();
 }
 
 // -------------------------------------------------------------------------------------- f and J
@@ -1029,8 +1038,9 @@ __device__ __forceinline__ ScalT<num<P>> eval_rates(const MV& M, P s, const LT& 
         o.deriv = deriv;
         o.more = 1;
       }
-      __syncthreads();
-      eval_pass(M, s, L, sc, GrpHelp<Gp, MV::kHelpers>{g.lane}, ps, deriv);
+      const GrpHelp<Gp, MV::kHelpers> all{g.lane};
+      all.sync();
+      eval_pass(M, s, L, sc, all, ps, deriv);
     } else {
       eval_pass(M, s, L, sc, g, ps, deriv);
     }

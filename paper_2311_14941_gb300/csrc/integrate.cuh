@@ -120,7 +120,7 @@ __global__ void k_integrate_plain(MV M, LT L, int N, double* __restrict__ T, con
   else idle_state(s, L, M.m, g);
   g.sync();
   while (any_cell(g, r.active)) cell_step(M, s, L, oo, g, r);
-  if constexpr (MV::kHelpers > 0) help_end();
+  if constexpr (MV::kHelpers > 0) help_end<Gp, MV::kHelpers>();
   if (c < N) {
     cell_end(oo, g, r);
     store_cell(M, s, L, N, g, r, T, Y, h_io, nsub, status, nacc_out);
@@ -184,7 +184,7 @@ __global__ void k_integrate_persistent(MV M, LT L, int N, double* __restrict__ T
       gs.sync();
     }
   }
-  if constexpr (MV::kHelpers > 0) help_end();
+  if constexpr (MV::kHelpers > 0) help_end<Gp, MV::kHelpers>();
 }
 
 }  // namespace chemgb
