@@ -272,17 +272,19 @@ constexpr double kLn10 = 2.30258509299404568402;
 
 // ---- doubles in shared memory by 32-bit address.  The compiler carries a pointer into shared memory as a 64-bit
 // number and rebuilds addresses in 64 bits; a step of a substitution takes 166 cycles with plain pointers and 130
-// with these.  The accesses are volatile: they keep their order among themselves and around barriers, which the
-// rate code, with many independent loads in flight, would pay for: it keeps plain pointers.
+// with these.  The accesses are volatile and name memory as clobbered: they keep their order among themselves, around
+// barriers and against plain accesses of the same cell, which they do not show the compiler otherwise (the clobber costs
+// neither registers nor time).  The rate code, with many independent loads in flight, would pay for that order: it keeps
+// plain pointers.  Between lanes, a barrier stands between one kind of access and the other, as between any two.
 struct SRef {
   uint32_t a;
   __device__ __forceinline__ operator double() const {
     double v;
-    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a));
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
     return v;
   }
   __device__ __forceinline__ SRef& operator=(double v) {
-    asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v));
+    asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
     return *this;
   }
   __device__ __forceinline__ SRef& operator=(const SRef& o) { return *this = (double)o; }
@@ -304,7 +306,7 @@ __device__ __forceinline__ T* prog_ptr(T* p) { return p; }
 // when lanes disagree).
 __device__ __forceinline__ void store_if(const SPtr& p, int i, double v, bool yes) {
   asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.shared.f64 [%0], %1;\n\t}" ::"r"(p.a + (uint32_t)i * 8u),
-               "d"(v), "r"((int)yes));
+               "d"(v), "r"((int)yes) : "memory");
 }
 template <class T>
 __device__ __forceinline__ void store_if(T* p, int i, const T& v, bool yes) {
