@@ -136,7 +136,11 @@ typedef struct {
                              1: persistent work-queue kernel over cells sorted by their previous
                              substep count */
   int block_cells;        /* cells in flight per block (each takes warps_per_cell warps); 0: automatic;
-                             larger requests are reduced to the largest block that launches */
+                             larger requests are reduced to the largest block that launches.  With 0, and while
+                             all cells fit at once beside them, a cell's block also holds one to three helper
+                             warps that only evaluate reaction rates (chem_launch_shape tells); they change no
+                             bit of the results.  Any other value selects the kernels without helpers, which
+                             take 4 to 30% longer in such calls with few cells */
   int chunk;              /* cells taken per queue pull in mode 1; 0: automatic (1).  Values above an even
                              share of the cells over the resident lane groups, ceil(N / groups), are
                              reduced to that share (a larger pull only leaves lane groups idle); results
@@ -152,7 +156,8 @@ typedef struct {
                              flight for mechanisms whose cells fill shared memory); 0: automatic (two when
                              one-warp cells leave fewer than 6 per SM, see chem_info).  Results of the two
                              choices agree to rounding, not bit for bit (different summation orders).
-                             chem_adjoint uses one warp per cell. */
+                             chem_adjoint integrates with one warp per cell; its reverse pass takes a second
+                             one while all cells fit at once, which changes no bit of the results. */
   int method;             /* Rosenbrock method: 0 RODAS3 (Sandu et al. 1997; order 3, embedded order 2,
                              L-stable; the default and the only one chem_adjoint differentiates),
                              1 ROS2 (Verwer et al. 1999; order 2, embedded order 1, L-stable,
@@ -162,11 +167,11 @@ typedef struct {
   int cells_per_warp;     /* chem_integrate and chem_integrate_noalloc: 2 = two cells share a warp, 16 lanes
                              each (for mechanisms with few species, whose loops and sparse programs leave
                              most of a warp idle; needs warps_per_cell 0 or 1; block_cells is rounded to
-                             an even count; in mode 1 the two halves of a warp take consecutive cells of the
-                             sorted queue); 1 = one cell per warp (or per two warps); 0: automatic (see
-                             chem_info: two for mechanisms of at most 16 species when half-warp blocks
-                             keep at least as many cells resident per SM, else one).  Results agree with
-                             one warp per cell to rounding. */
+                             an even count; the two cells take their attempts together, and in mode 1 each
+                             half pulls from the sorted queue when its own cells have ended); 1 = one cell
+                             per warp (or per two warps); 0: automatic (see chem_info: two for mechanisms of
+                             at most 16 species when half-warp blocks keep at least as many cells resident
+                             per SM, else one).  Results agree with one warp per cell to rounding. */
   int tabulate;           /* chem_integrate, chem_integrate_noalloc, chem_integrate_mapped: 1 = evaluate the
                              costly temperature functions from tables (an approximation; Sec. 2.5: SpeedCHEM
                              interpolates costly thermodynamic functions with polynomials of optimal
@@ -209,11 +214,13 @@ chem_status chem_destroy(chem_handle h);
 
 /* Mechanism-specialised integration kernels (opt-in).  The one-warp-per-cell integration kernels (plain
    and persistent form) are compiled again at run time (NVRTC, loaded with dlopen) with this mechanism's
-   sizes (species, reactions, nonzeros of S and of the factor, steps of the elimination and substitution
-   programs) and the cell's shared-memory offsets as compile-time constants, so that the compiler folds
-   the trip counts and addresses of the sparse-analytical evaluation into the code (Sec. 2.5: SpeedCHEM
-   manages the mechanism's sparse algebra internally).  The tables and
-   programs stay in device memory; only sizes and offsets become constants.  The kernels are loaded into
+   sizes (species, reactions, nonzeros of S and of the factor, Jacobian passes) and the cell's
+   shared-memory offsets as compile-time constants, so that the compiler folds the trip counts and
+   addresses of the sparse-analytical evaluation into the code (Sec. 2.5: SpeedCHEM manages the
+   mechanism's sparse algebra internally).  The tables and programs, and the programs' lengths, stay in
+   device memory; only sizes and offsets become constants.  They have no helper warps: in calls with few
+   cells the library's kernels, which have some (see block_cells), are the faster ones (53 species / 325
+   reactions: 123 against 139 ms at 300 cells, 164 against 154 at 1,200).  The kernels are loaded into
    the handle's device and used by calls with chem_integrate_opts.specialized = 1 until chem_destroy.
    Compiled code is cached on disk (directory CHEM_RTC_CACHE, else rtc_cache beside the library), keyed
    by the source, the headers, the options and the compiler's version; a second handle of the same

@@ -20,9 +20,10 @@ LIB = os.path.join(OUT, "libchemgb.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 # kernel translation units besides capi.cu: the integration kernels per lane group, and the adjoint
-# Registers per thread of the integration kernels: as many as they ask for (about 200; nine warps per SM, which
-# is what shared memory allows at 53 species).  Held to 168 or 128, the programs' ops that are read ahead spill: a
-# 4,096-cell jet field took 320 and 370 ms instead of 300, 6,000 small cells 371 (at 168) instead of 351.
+# Registers per thread of the integration kernels: as many as they ask for (185 to 201 without helpers, so eight warps
+# per SM where shared memory would hold nine cells of 53 species and more of fewer).  Held to 168 or 128, nine and more
+# warps fit, but the programs' ops that are read ahead spill: a 4,096-cell jet field took 320 and 370 ms instead of
+# 300, 6,000 small cells 371 (at 168) instead of 351.
 REG_CAP = {f: ["-maxrregcount=224"] for f in ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd_half",
                                                     "kern_fwd_help", "kern_fwd_help_pair")}
 CUDA_UNITS = ("kern_fwd_warp", "kern_fwd_warp_plain", "kern_fwd_pair", "kern_fwd_half", "kern_fwd_help", "kern_fwd_help_pair", "kern_rates",

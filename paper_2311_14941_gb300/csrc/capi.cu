@@ -93,7 +93,7 @@ struct chem_handle_s {
 namespace {
 
 // Shared-memory layout of one cell (offsets in doubles).
-CellLayout make_layout(const HostMech& hm, bool separate_lu = false) {
+CellLayout make_layout(const HostMech& hm) {
   CellLayout L{};
   int o = 0;
   const int m = hm.m, n = hm.n, R = hm.R;
@@ -104,19 +104,9 @@ CellLayout make_layout(const HostMech& hm, bool separate_lu = false) {
   L.q = take(std::max(R, 1));
   L.S = take(hm.nnz_S);
   // the Jacobian passes' dq/dT values and derivative slots are dead once S is assembled; the factor and
-  // 1/diag reuse their space (the adjoint keeps the factor apart: separate_lu)
-  const int lu_part = hm.nnz_LU + m;
-  if (separate_lu) {
-    L.D = take(std::max(hm.jreg, 1));
-    L.LU = take(hm.nnz_LU);
-    L.dinv = take(m);
-  } else {
-    const int reuse = std::max(lu_part, hm.jreg);
-    L.D = o;
-    L.LU = o;
-    L.dinv = o + hm.nnz_LU;
-    o += reuse;
-  }
+  // 1/diag reuse their space
+  L.D = L.LU = take(std::max(hm.nnz_LU + m, hm.jreg));
+  L.dinv = L.LU + hm.nnz_LU;
   int np = 1;
   for (const HostProg& P : hm.prog) {
     for (const HostGather* g : {&P.g_omega, &P.g_row, &P.g_col}) np = std::max(np, g->n_partial);
@@ -292,9 +282,9 @@ static_assert(sizeof(HelpOrder) <= kHelpStatic, "the order of a block");
 // the most helper warps that still holds all cells at once (188 registers per thread: 8 warps per SM, so 2 cells with
 // three helpers, 4 with one).  Beyond that the helpers' registers would cost resident cells, and the FP64 pipe is
 // busy without them: held to 168 registers so that as many cells fit as without, a cell of two warps at 150 species
-// gains 1-2% (500 cells: 322 against 318 ms) where it gains 12% with room.  Only where every warp of the cell gets at
+// gains 1-2% (500 cells: 318 ms with helpers, 322 without) where it gains 12% with room.  Only where every warp of the cell gets at
 // least two rounds of reactions (below): with the one or two rounds of 27 reactions there is nothing to share, and the
-// barriers cost 4% (304 cells of one warp each: 155 against 161 ms; two cells per warp gained 1%).
+// barriers cost 4% (304 cells of one warp each: 161 ms with helpers, 155 without; two cells per warp gained 1%).
 int pick_kernel(const chem_handle h, int grp, int N) {
   for (int i = kHelpForms - 1; i >= 0; --i)
     if (kHelpGroups[i] == grp && N <= h->num_sms * h->helped_cells[i]) return kNumGroups + i;

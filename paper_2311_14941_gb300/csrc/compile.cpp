@@ -747,14 +747,12 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
     for (int r = 0; r < R; ++r) {
       const Rx& x = rx[hm.rx_order[r]];
       auto sp_of = [&](const std::vector<int>& o, size_t i) { return (uint32_t)(i < o.size() ? o[i] : 0); };
-      auto rep = [](const std::vector<int>& o) { return std::set<int>(o.begin(), o.end()).size() < o.size(); };
       std::set<int> all(x.ro.begin(), x.ro.end());
       all.insert(x.po.begin(), x.po.end());
       const bool simple = x.type == 0 && x.rev && x.ro.size() == 2 && x.po.size() == 2 && all.size() == 4;
       rec[r] = RxRec{sp_of(x.ro, 0) | sp_of(x.ro, 1) << 16, sp_of(x.ro, 2) | sp_of(x.po, 0) << 16,
                      sp_of(x.po, 1) | sp_of(x.po, 2) << 16,
                      (uint32_t)((x.rev ? RXF_REV : 0) | x.ro.size() << 1 | x.po.size() << 3 | (simple ? RXF_SIMPLE : 0) |
-                                (rep(x.ro) || rep(x.po) ? RXF_REP : 0) |
                                 (uint32_t)hm.rxi[(size_t)r * RX_I + 13] << 16)};
     }
     std::vector<int> at(R), pos(R);   // at[i]: reaction placed at i; pos: its inverse

@@ -337,7 +337,7 @@ using num = typename pointee<P>::type;
 // kProgBlock: a lane loads its ops of the next block (independent loads) before it executes the current one.  A
 // step has no branch (a divergent branch costs about 60 cycles, as much as its FP64 instruction): idle lanes take
 // part and do not store.  A step of the elimination so takes 125 to 155 cycles, of which 64 are the FP64
-// instruction; reading two steps ahead in a loop over kinds it took 640.
+// instruction; read two steps ahead in a loop over kinds it took 640 in the kernel (one warp on an SM), ops included.
 __device__ __forceinline__ GatherOp as_gop(uint2 v) {
   GatherOp o;
   o.a = (uint16_t)(v.x & 0xFFFF); o.b = (uint16_t)(v.x >> 16);
@@ -375,7 +375,7 @@ __device__ __forceinline__ bool run_fma(const FmaProgram& P, SPtr A, SPtr v, int
 #pragma unroll
       for (int u = 0; u < slots; ++u) nxt[u] = __ldg(op + u * width);
     }
-    if (!RECIP) {   // whole blocks (the first slots of the first one may be idle)
+    if (!RECIP) {   // whole blocks (the first slots of the last one may be idle)
 #pragma unroll
       for (int u = 0; u < kProgBlock; ++u) step(cur[u]);
     } else {

@@ -76,9 +76,8 @@ struct alignas(16) SlotRec {
   int mask, pad;
 };
 // flags (bits 16-31: derivative-slot offset): bit 0 reversible, bits 1-2 reactant occurrences, bits 3-4 product occurrences, bit 5 simple
-// (elementary, reversible, two reactants and two products, all four different species), bit 6: a species
-// occurs more than once on one side
-enum : int { RXF_REV = 1, RXF_SIMPLE = 32, RXF_REP = 64 };
+// (elementary, reversible, two reactants and two products, all four different species)
+enum : int { RXF_REV = 1, RXF_SIMPLE = 32 };
 
 // ---- warp programs, compiled for a group of `width` lanes (one warp per cell: 32, two: 64, half: 16)
 // The device reads every program in blocks of kProgBlock steps, a block ahead.

@@ -189,7 +189,7 @@ std::string specialized_source(const HostMech& hm, const CellLayout& L) {
     << ", n_troe = " << hm.n_troe << ", n_tb = " << hm.n_tb << ", nY = " << hm.nY << ", nnz_S = " << hm.nnz_S
     << ", nnz_LU = " << hm.nnz_LU << ", n_dslot = " << hm.n_dslot << ";\n"
     << "  static constexpr int lu_steps = " << P.lu_kind.size() << ", sv_steps = " << P.sv_kind.size()
-    << ", svT_steps = " << P.svT_kind.size() << ", n_jpass = " << hm.jpass.size() / 4 << ";\n"
+    << ", n_jpass = " << hm.jpass.size() / 4 << ";\n"
     << "};\n"
     << "struct SpecLayout : CellLayout {\n"
     << "  static constexpr int y = " << L.y << ", ytmp = " << L.ytmp << ", f0 = " << L.f0 << ", U1 = " << L.U1
