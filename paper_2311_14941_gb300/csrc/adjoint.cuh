@@ -187,7 +187,10 @@ struct ToContraction {
   int n;
   E iRT[W::n], e[W::n], G_T[W::n], g[W::n];
   Sc sh, scp;             // sum_r q_r times the reaction's change of h/RT and of cp/R
+  bool idle = false;      // the reaction changes nothing: its rate, infinite or NaN perhaps, must not count
   __device__ __forceinline__ void rate(int r, const RxRec& rec, const Sc& q) {
+    idle = (rec.flags & RXF_IDLE) != 0;
+    if (idle) return;
     double dA = 0.0, dE = 0.0;
 #pragma unroll
     for (int st = 0; st < W::n; ++st) {
@@ -203,6 +206,7 @@ struct ToContraction {
     scp = sfma(q, net_of<Sc>(rec, cpR), scp);
   }
   __device__ __forceinline__ void dT(int, const Sc& v) {
+    if (idle) return;
 #pragma unroll
     for (int st = 0; st < W::n; ++st) G_T[st] += e[st] * W::pick(v, st);
   }

@@ -749,10 +749,12 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
       auto sp_of = [&](const std::vector<int>& o, size_t i) { return (uint32_t)(i < o.size() ? o[i] : 0); };
       std::set<int> all(x.ro.begin(), x.ro.end());
       all.insert(x.po.begin(), x.po.end());
+      const bool idle = std::multiset<int>(x.ro.begin(), x.ro.end()) == std::multiset<int>(x.po.begin(), x.po.end());
       const bool simple = x.type == 0 && x.rev && x.ro.size() == 2 && x.po.size() == 2 && all.size() == 4;
       rec[r] = RxRec{sp_of(x.ro, 0) | sp_of(x.ro, 1) << 16, sp_of(x.ro, 2) | sp_of(x.po, 0) << 16,
                      sp_of(x.po, 1) | sp_of(x.po, 2) << 16,
                      (uint32_t)((x.rev ? RXF_REV : 0) | x.ro.size() << 1 | x.po.size() << 3 | (simple ? RXF_SIMPLE : 0) |
+                                (idle ? RXF_IDLE : 0) |
                                 (uint32_t)hm.rxi[(size_t)r * RX_I + 13] << 16)};
     }
     std::vector<int> at(R), pos(R);   // at[i]: reaction placed at i; pos: its inverse
@@ -786,8 +788,8 @@ chem_status compile_mechanism(const chem_mech_desc& d, HostMech& hm, std::string
     for (HostProg& Pg : hm.prog)
       if (!build_gather(gw, Pg.g_omega, err, Pg.width)) return CHEM_EUNSUPPORTED;
     std::vector<std::vector<std::pair<int, int>>> gs(n);
-    for (int r = 0; r < R; ++r)
-      for (size_t c = 0; c < slots_sp[r].size(); ++c)
+    for (int r = 0; r < R; ++r)   // (an idle reaction's slots may hold anything)
+      for (size_t c = 0; c < slots_sp[r].size() && !(rec[r].flags & RXF_IDLE); ++c)
         gs[slots_sp[r][c]].push_back({hm.rxi[(size_t)pos[r] * RX_I + 13] + (int)c, 0});
     if (!build_gather(gs, hm.prog[0].g_slot, err, hm.prog[0].width)) return CHEM_EUNSUPPORTED;
     hm.jpass.clear();

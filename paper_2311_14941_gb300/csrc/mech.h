@@ -76,8 +76,9 @@ struct alignas(16) SlotRec {
   int mask, pad;
 };
 // flags (bits 16-31: derivative-slot offset): bit 0 reversible, bits 1-2 reactant occurrences, bits 3-4 product occurrences, bit 5 simple
-// (elementary, reversible, two reactants and two products, all four different species)
-enum : int { RXF_REV = 1, RXF_SIMPLE = 32 };
+// (elementary, reversible, two reactants and two products, all four different species), bit 6 idle (the same species on
+// both sides: no net change)
+enum : int { RXF_REV = 1, RXF_SIMPLE = 32, RXF_IDLE = 64 };
 
 // ---- warp programs, compiled for a group of `width` lanes (one warp per cell: 32, two: 64, half: 16)
 // The device reads every program in blocks of kProgBlock steps, a block ahead.
